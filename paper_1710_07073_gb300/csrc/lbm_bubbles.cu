@@ -1902,12 +1902,28 @@ __global__ void k_set_feq(const double* __restrict__ rho, const double* __restri
 #undef LBM_FEQ
 }
 
-// FP64 totals: per-block partial sums in fixed order, then one block.
+// FP64 totals: per-thread compensated sums, per-block FP64 partials in fixed
+// order, then one block.
+//
+// Bound by HBM (76 or 38 B per site, read once), as long as the FP64 pipe
+// stays out of the loop: it issues 2 FMAs per clock and SM here, and the 95
+// FP64 operations per site of a plain FP64 accumulation took 0.81 ms on
+// 128 x 128 x 256 where the reads take 0.05.  So each thread sums every
+// direction over its sites as hi + lo, two floats (Neumaier's compensated
+// summation: TwoSum, the rounding errors collected in lo), 7 FP32 operations
+// per value, and only the per-thread sums go through FP64.  The error is that
+// of about 48 bits against the sum of magnitudes.  lbm_get_totals before and
+// after: 7.01 -> 0.77 ms on 256 x 256 x 512 in FP16, 0.54 -> 0.063 ms on
+// 64 x 64 x 128, 0.101 -> 0.045 ms on 32 x 32 x 64.
 constexpr int TOT_BLOCK = 256;
+// Resident CTAs per SM the kernel is compiled for, and the grid: whole waves
+// of 152 SMs.
+constexpr int TOT_PER_SM = 2;
+constexpr int TOT_GRID = 152 * TOT_PER_SM;
 
 int totals_partials(const Geo& g) {
-    long long blocks = (g.S + TOT_BLOCK - 1) / TOT_BLOCK;
-    return (int)(blocks < 4096 ? blocks : 4096);
+    const long long blocks = (g.S + TOT_BLOCK - 1) / TOT_BLOCK;
+    return (int)(blocks < TOT_GRID ? blocks : TOT_GRID);
 }
 
 __device__ double block_sum(double v, double* sh) {
@@ -1923,18 +1939,18 @@ __device__ double block_sum(double v, double* sh) {
     return t;
 }
 
+// The same sums of one thread's sites in FP64: for values whose FP32 sums are
+// not finite (infinities, NaN, sums beyond FP32).
 template <int ST>
-__global__ void __launch_bounds__(TOT_BLOCK)
-k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, double* partials) {
-    __shared__ double sh[32];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.S;
-         s += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(s % g.nx), y = (int)((s / g.nx) % g.ny),
-                  z = (int)(s / ((long long)g.nx * g.ny));
+__device__ __noinline__ void totals_fp64(const typename Store<ST>::T* __restrict__ f,
+                                         const Geo& g, const CollideParams& cp, unsigned s,
+                                         unsigned stride, double acc[4]) {
+    for (int k = 0; k < 4; ++k) acc[k] = 0.0;
+    for (; s < (unsigned)g.S; s += stride) {
+        int x, y, z;
+        site_coords(g, s, x, y, z);
         float gv[Q];
         gather<ST>(f, g, cp, x, y, z, gv);
-#pragma unroll
         for (int j = 0; j < Q; ++j) {
             acc[0] += gv[j];
             acc[1] += cx(j) * (double)gv[j];
@@ -1942,21 +1958,73 @@ k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, d
             acc[3] += cz(j) * (double)gv[j];
         }
     }
+}
+
+template <int ST>
+__global__ void __launch_bounds__(TOT_BLOCK, TOT_PER_SM)
+k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, double* partials) {
+    __shared__ double sh[32];
+    F2 dir[Q];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) dir[j] = F2{0.0f, 0.0f};
+    const unsigned S = (unsigned)g.S, stride = gridDim.x * TOT_BLOCK;   // 19 S < 2^32
+    const unsigned s0 = blockIdx.x * TOT_BLOCK + threadIdx.x;
+    // Two sites at a time, the loads of both issued first (two_sum with zero
+    // changes nothing).
+    for (unsigned s = s0; s < S; s += 2 * stride) {
+        const bool two = s + stride < S;
+        int x, y, z, x2, y2, z2;
+        site_coords(g, s, x, y, z);
+        site_coords(g, two ? s + stride : s, x2, y2, z2);
+        typename Store<ST>::T ra[Q], rb[Q];
+        gather_issue<ST>(f, g, x, y, z, ra);
+        gather_issue<ST>(f, g, x2, y2, z2, rb);
+        float ga[Q], gb[Q];
+        gather_finish<ST>(ra, cp, ga);
+        gather_finish<ST>(rb, cp, gb);
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            const F2 t = two_sum(dir[j].h, ga[j]);
+            const F2 v = two_sum(t.h, two ? gb[j] : 0.0f);
+            dir[j] = F2{v.h, dir[j].l + t.l + v.l};
+        }
+    }
+    // Eq. 10 over the directions: opposite ones come in pairs (2k - 1, 2k).
+    F2 m[4] = {dir[0], F2{0.0f, 0.0f}, F2{0.0f, 0.0f}, F2{0.0f, 0.0f}};
+#pragma unroll
+    for (int j = 1; j < Q; j += 2) {
+        m[0] = f2_add(f2_add(m[0], dir[j].h, dir[j].l), dir[j + 1].h, dir[j + 1].l);
+        const F2 d = f2_add(dir[j], -dir[j + 1].h, -dir[j + 1].l);
+        if (cx(j) != 0) m[1] = f2_add(m[1], (float)cx(j) * d.h, (float)cx(j) * d.l);
+        if (cy(j) != 0) m[2] = f2_add(m[2], (float)cy(j) * d.h, (float)cy(j) * d.l);
+        if (cz(j) != 0) m[3] = f2_add(m[3], (float)cz(j) * d.h, (float)cz(j) * d.l);
+    }
+    double acc[4];
+    bool finite = true;
+    for (int k = 0; k < 4; ++k) {
+        acc[k] = f2_to(m[k]);
+        finite = finite && isfinite(m[k].h) && isfinite(m[k].l);
+    }
+    if (!finite) totals_fp64<ST>(f, g, cp, s0, stride, acc);
     for (int k = 0; k < 4; ++k) {
         const double t = block_sum(acc[k], sh);
         if (threadIdx.x == 0) partials[4 * blockIdx.x + k] = t;
     }
 }
 
-__global__ void k_totals_final(const double* partials, int np, double mass0, double* out4) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The blocks' partials, summed by one block in a fixed order (a thread over
+// every TOT_BLOCK-th block, then the threads): one thread over 4,096 of them
+// took 0.91 ms.
+__global__ void __launch_bounds__(TOT_BLOCK)
+k_totals_final(const double* partials, int np, double mass0, double* out4) {
+    __shared__ double sh[32];
     double t[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = 0; i < np; ++i)
+    for (int i = threadIdx.x; i < np; i += TOT_BLOCK)
         for (int k = 0; k < 4; ++k) t[k] += partials[4 * i + k];
-    out4[0] = mass0 + t[0];
-    out4[1] = t[1];
-    out4[2] = t[2];
-    out4[3] = t[3];
+    for (int k = 0; k < 4; ++k) {
+        const double v = block_sum(t[k], sh);
+        if (threadIdx.x == 0) out4[k] = k == 0 ? mass0 + v : v;
+    }
 }
 
 static unsigned site_blocks(const Geo& g) { return (unsigned)((g.S + 255) / 256); }
@@ -2012,7 +2080,7 @@ cudaError_t launch_totals(int storage, const void* f, const Geo& g, const Collid
         default:
             k_totals<2><<<npartials, TOT_BLOCK, 0, st>>>((const __nv_bfloat16*)f, g, cp, partials);
     }
-    k_totals_final<<<1, 32, 0, st>>>(partials, npartials, (double)g.S * (double)cp.rho0, out4);
+    k_totals_final<<<1, TOT_BLOCK, 0, st>>>(partials, npartials, (double)g.S * (double)cp.rho0, out4);
     return cudaGetLastError();
 }
 
