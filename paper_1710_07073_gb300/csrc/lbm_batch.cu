@@ -45,7 +45,7 @@ struct lbm_batch {
     BatchColumn* cols_d = nullptr;
     double* col_nu_d = nullptr;
     int* flag_d = nullptr;
-    int* flag_h = nullptr;
+    HostPage* page = nullptr;       // pinned: what the kernels report to the host
     int* work_counter = nullptr;
     bool unstable = false;
 
@@ -223,7 +223,7 @@ int ensure_device(lbm_batch* b) {
         return bfail(b, LBM_ERR_ALLOC, "batch device state (%zu bytes per population buffer)",
                      bytes);
     }
-    if (!b->flag_h) LBM_BCUDA(cudaMallocHost((void**)&b->flag_h, sizeof(int)), "cudaMallocHost");
+    if (!b->page) LBM_BCUDA(cudaMallocHost((void**)&b->page, sizeof(HostPage)), "cudaMallocHost");
     cudaStream_t s = b->stream;
     LBM_BCUDA(cudaMemsetAsync(b->f[0], 0, bytes, s), "memset f");
     LBM_BCUDA(cudaMemsetAsync(b->flag_d, 0, sizeof(int), s), "flag");
@@ -316,18 +316,15 @@ int build_graph(lbm_batch* b) {
 }
 
 int check_flag(lbm_batch* b) {
-    LBM_BCUDA(cudaMemcpyAsync(b->flag_h, b->flag_d, sizeof(int), cudaMemcpyDeviceToHost, b->stream),
-              "flag");
+    LBM_BCUDA(launch_status(b->flag_d, b->small.overflow, b->page, b->stream), "flag");
     LBM_BCUDA(cudaStreamSynchronize(b->stream), "step");
-    if (*b->flag_h) {
+    if (b->page->flag) {
         b->unstable = true;
         return bfail(b, LBM_ERR_UNSTABLE,
                      "non-finite value or |u| >= 0.3 in a column, or a bubble faster than %d "
                      "cells per step", GUARD_CELLS);
     }
-    int ov = 0;
-    LBM_BCUDA(cudaMemcpy(&ov, b->small.overflow, sizeof(int), cudaMemcpyDeviceToHost), "overflow");
-    if (ov) return bfail(b, LBM_ERR_STATE, "tile list capacity exceeded");
+    if (b->page->overflow) return bfail(b, LBM_ERR_STATE, "tile list capacity exceeded");
     return LBM_OK;
 }
 
@@ -426,7 +423,7 @@ void lbm_batch_destroy(lbm_batch* b) {
         cudaEventDestroy(e.second);
     }
     while (!b->allocs.empty()) bfree(b, b->allocs.back().first);
-    if (b->flag_h) cudaFreeHost(b->flag_h);
+    if (b->page) cudaFreeHost(b->page);
     if (b->own_stream) cudaStreamDestroy(b->stream);
     delete b;
 }
@@ -756,18 +753,22 @@ int lbm_batch_get_fields(lbm_batch* b, int col, double* rho, double* u3) {
     if (!rho && !u3) return LBM_OK;
     const BatchColumn& c = b->cols[col];
     const size_t S = (size_t)c.g.S;
-    double* rd = rho ? (double*)balloc(b, sizeof(double) * S) : nullptr;
-    double* ud = u3 ? (double*)balloc(b, sizeof(double) * 3 * S) : nullptr;
-    if ((rho && !rd) || (u3 && !ud)) {
+    // Pinned outputs are written by the kernel, pageable ones staged.
+    double* const rho_map = mapped_output(rho, S);
+    double* const u_map = mapped_output(u3, 3 * S);
+    double* rd = rho && !rho_map ? (double*)balloc(b, sizeof(double) * S) : nullptr;
+    double* ud = u3 && !u_map ? (double*)balloc(b, sizeof(double) * 3 * S) : nullptr;
+    if ((rho && !rho_map && !rd) || (u3 && !u_map && !ud)) {
         bfree(b, rd);
         bfree(b, ud);
         return bfail(b, LBM_ERR_ALLOC, "field staging");
     }
     const char* base = (const char*)b->f[b->cur] + (size_t)c.pop_offset * elem_bytes(b->storage);
-    cudaError_t e = launch_fields(b->storage, base, c.g, c.cp, rd, ud, b->stream);
-    if (e == cudaSuccess && rho)
+    cudaError_t e = launch_fields(b->storage, base, c.g, c.cp, rho_map ? rho_map : rd,
+                                  u_map ? u_map : ud, b->stream);
+    if (e == cudaSuccess && rd)
         e = cudaMemcpyAsync(rho, rd, sizeof(double) * S, cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess && u3)
+    if (e == cudaSuccess && ud)
         e = cudaMemcpyAsync(u3, ud, sizeof(double) * 3 * S, cudaMemcpyDeviceToHost, b->stream);
     cudaError_t e2 = cudaStreamSynchronize(b->stream);
     bfree(b, rd);
@@ -785,11 +786,8 @@ int lbm_batch_get_bubbles(lbm_batch* b, int cap, int* n, double* pos3, double* v
     const int k = nb < cap ? nb : cap;
     if (k == 0) return LBM_OK;
     cudaStream_t s = b->stream;
-    LBM_BCUDA(download_bubble_state(b->bub, k, pos3, vel3, ul3, psi3, s), "bubbles");
-    if (active)
-        LBM_BCUDA(cudaMemcpyAsync(active, b->bub.active, sizeof(int) * (size_t)k,
-                                  cudaMemcpyDeviceToHost, s), "active");
-    LBM_BCUDA(cudaStreamSynchronize(s), "get bubbles");
+    LBM_BCUDA(download_bubble_state(b->bub, k, pos3, vel3, ul3, psi3, active, b->page, s),
+              "bubbles");
     return LBM_OK;
 }
 

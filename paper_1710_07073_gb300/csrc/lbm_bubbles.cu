@@ -18,6 +18,7 @@
 #include <climits>
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "lbm_device.cuh"
@@ -1920,6 +1921,7 @@ constexpr int TOT_BLOCK = 256;
 // of 152 SMs.
 constexpr int TOT_PER_SM = 2;
 constexpr int TOT_GRID = 152 * TOT_PER_SM;
+static_assert(TOT_GRID <= TOTALS_PARTIALS_MAX, "a context's buffer of partials");
 
 int totals_partials(const Geo& g) {
     const long long blocks = (g.S + TOT_BLOCK - 1) / TOT_BLOCK;
@@ -1960,6 +1962,15 @@ __device__ __noinline__ void totals_fp64(const typename Store<ST>::T* __restrict
     }
 }
 
+// TwoSum of a value that may itself be a product (a widened 16-bit value):
+// __fadd_rn keeps the compiler from contracting that product into the sum,
+// which would leave its rounding error out.
+__device__ __forceinline__ F2 two_sum_rn(float a, float b) {
+    const float s = __fadd_rn(a, b);
+    const float bb = __fadd_rn(s, -a);
+    return F2{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
+}
+
 template <int ST>
 __global__ void __launch_bounds__(TOT_BLOCK, TOT_PER_SM)
 k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, double* partials) {
@@ -1984,8 +1995,8 @@ k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, d
         gather_finish<ST>(rb, cp, gb);
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
-            const F2 t = two_sum(dir[j].h, ga[j]);
-            const F2 v = two_sum(t.h, two ? gb[j] : 0.0f);
+            const F2 t = two_sum_rn(dir[j].h, ga[j]);
+            const F2 v = two_sum_rn(t.h, two ? gb[j] : 0.0f);
             dir[j] = F2{v.h, dir[j].l + t.l + v.l};
         }
     }
@@ -2113,8 +2124,9 @@ cudaError_t upload_bubble_state(const BubbleDev& B, int n, const double* pos3, c
 }
 
 // FP64 copies of the first k bubbles' state: out = [x | u | u_l | psi], each
-// 3k values.
-__global__ void k_export_bubbles(BubbleDev B, int k, double* __restrict__ out) {
+// 3k values; with `act`, their active flags.
+__global__ void k_export_bubbles(BubbleDev B, int k, double* __restrict__ out,
+                                 int* __restrict__ act) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t m = 3 * (size_t)k;
     if (i >= (int)m) return;
@@ -2122,21 +2134,68 @@ __global__ void k_export_bubbles(BubbleDev B, int k, double* __restrict__ out) {
     out[m + i] = B.u[i];
     out[2 * m + i] = B.ul[i];
     out[3 * m + i] = B.psi[i];
+    if (act && i < k) act[i] = B.active[i];
 }
 
+// Up to PAGE_BUBBLES bubbles the export writes the pinned page (one launch and
+// one wait, where five copies took 70 us); more are staged on the device and
+// copied to the caller's arrays.
 cudaError_t download_bubble_state(const BubbleDev& B, int k, double* pos3, double* vel3,
-                                  double* ul3, double* psi3, cudaStream_t st) {
-    double* const stage = B.out64;
+                                  double* ul3, double* psi3, int* active, HostPage* page,
+                                  cudaStream_t st) {
+    const bool small = page != nullptr && k <= PAGE_BUBBLES;
+    double* const stage = small ? page->bub : B.out64;
     const size_t m = 3 * (size_t)k, bytes = sizeof(double) * m;
-    k_export_bubbles<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(B, k, stage);
+    k_export_bubbles<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(B, k, stage,
+                                                                 small ? page->active : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     double* dst[4] = {pos3, vel3, ul3, psi3};
+    if (small) {
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        for (int q = 0; q < 4; ++q)
+            if (dst[q]) std::memcpy(dst[q], stage + q * m, bytes);
+        if (active) std::memcpy(active, page->active, sizeof(int) * (size_t)k);
+        return cudaSuccess;
+    }
     for (int q = 0; q < 4; ++q)
         if (dst[q] && (e = cudaMemcpyAsync(dst[q], stage + q * m, bytes, cudaMemcpyDeviceToHost,
                                            st)) != cudaSuccess)
             return e;
+    if (active && (e = cudaMemcpyAsync(active, B.active, sizeof(int) * (size_t)k,
+                                       cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+        return e;
     return cudaStreamSynchronize(st);
+}
+
+__global__ void k_status(const int* flag, const int* overflow, HostPage* page) {
+    if (threadIdx.x != 0) return;
+    page->flag = *flag;
+    page->overflow = overflow ? *overflow : 0;
+}
+
+cudaError_t launch_status(const int* flag, const int* overflow, HostPage* page, cudaStream_t st) {
+    k_status<<<1, 32, 0, st>>>(flag, overflow, page);
+    return cudaGetLastError();
+}
+
+double* mapped_output(double* host, size_t n) {
+    if (!host || n == 0) return nullptr;
+    cudaPointerAttributes a, b;
+    unsigned flags = 0;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
+        cudaPointerGetAttributes(&b, host + (n - 1)) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
+        (double*)b.devicePointer - (double*)a.devicePointer != (ptrdiff_t)(n - 1))
+        return nullptr;
+    if (cudaHostGetFlags(&flags, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return (flags & cudaHostRegisterReadOnly) ? nullptr : (double*)a.devicePointer;
 }
 
 }  // namespace lbm

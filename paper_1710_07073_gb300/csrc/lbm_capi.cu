@@ -123,11 +123,12 @@ int ensure_device(lbm_ctx* c) {
     c->bins.off = (int*)dalloc(c, sizeof(int) * ((size_t)c->bins.T + 1));
     c->bins.block_sums = (int*)dalloc(c, sizeof(int) * (size_t)c->bins.nblocks);
     c->bins.overflow = (int*)dalloc(c, sizeof(int));
+    c->tot_d = (double*)dalloc(c, sizeof(double) * 4 * TOTALS_PARTIALS_MAX);
     if (!c->f[0] || !c->f[1] || !c->flag_d || !c->bins.cnt || !c->bins.off ||
-        !c->bins.block_sums || !c->bins.overflow) {
+        !c->bins.block_sums || !c->bins.overflow || !c->tot_d) {
         void** owned[] = {&c->f[0], &c->f[1], (void**)&c->flag_d, (void**)&c->bins.cnt,
                           (void**)&c->bins.off, (void**)&c->bins.block_sums,
-                          (void**)&c->bins.overflow};
+                          (void**)&c->bins.overflow, (void**)&c->tot_d};
         for (void** q : owned) {
             dfree(c, *q);
             *q = nullptr;
@@ -135,7 +136,7 @@ int ensure_device(lbm_ctx* c) {
         return fail(c, LBM_ERR_ALLOC, "device state of the column (%zu bytes per population "
                     "buffer)", bytes);
     }
-    if (!c->flag_h) LBM_CUDA(cudaMallocHost((void**)&c->flag_h, sizeof(int)), "cudaMallocHost");
+    if (!c->page) LBM_CUDA(cudaMallocHost((void**)&c->page, sizeof(HostPage)), "cudaMallocHost");
     // Rest state f = f^eq(rho_l, 0) has zero shifted value in every format.
     LBM_CUDA(cudaMemsetAsync(c->f[0], 0, bytes, c->stream), "memset f");
     LBM_CUDA(cudaMemsetAsync(c->flag_d, 0, sizeof(int), c->stream), "memset flag");
@@ -451,10 +452,12 @@ int enqueue_one_step(lbm_ctx* c) {
 
 // Wait for the enqueued steps and report the instability flag / overflow.
 int finish_steps(lbm_ctx* c) {
-    LBM_CUDA(cudaMemcpyAsync(c->flag_h, c->flag_d, sizeof(int), cudaMemcpyDeviceToHost,
-                             c->stream), "read flag");
+    const int* overflow =
+        c->bins_valid ? (c->use_small ? c->small.overflow : c->bins.overflow) : nullptr;
+    LBM_CUDA(launch_status(c->flag_d, overflow, c->page, c->stream), "read flag");
     LBM_CUDA(cudaStreamSynchronize(c->stream), "step");
-    if (*c->flag_h & 8) {
+    const int flag = c->page->flag;
+    if (flag & 8) {
         // A grid barrier of the many-bubble update gave up waiting: its
         // arrival counter may be left part-way, so it starts again at zero.
         c->unstable = true;
@@ -464,18 +467,13 @@ int finish_steps(lbm_ctx* c) {
         return fail(c, LBM_ERR_TIMEOUT,
                     "a device-wide wait of the bubble update ran out (more than 1 s)");
     }
-    if (*c->flag_h) {
+    if (flag) {
         c->unstable = true;
         return fail(c, LBM_ERR_UNSTABLE,
                     "non-finite value or |u| >= 0.3 in the liquid, or a bubble faster than %d "
                     "cells per step", GUARD_CELLS);
     }
-    if (c->bins_valid) {
-        int ov = 0;
-        LBM_CUDA(cudaMemcpy(&ov, c->use_small ? c->small.overflow : c->bins.overflow, sizeof(int),
-                            cudaMemcpyDeviceToHost), "overflow");
-        if (ov) return fail(c, LBM_ERR_STATE, "tile list capacity exceeded");
-    }
+    if (c->page->overflow) return fail(c, LBM_ERR_STATE, "tile list capacity exceeded");
     return LBM_OK;
 }
 
@@ -575,7 +573,7 @@ void lbm_destroy(lbm_ctx* c) {
         cudaEventDestroy(e.second);
     }
     while (!c->allocs.empty()) dfree(c, c->allocs.back().first);
-    if (c->flag_h) cudaFreeHost(c->flag_h);
+    if (c->page) cudaFreeHost(c->page);
     delete c;
 }
 
@@ -894,19 +892,23 @@ int lbm_get_fields(lbm_ctx* c, double* rho, double* u3) {
     if (rc) return rc;
     if (!rho && !u3) return LBM_OK;
     const Geo g = geo_of(c);
-    double* rd = rho ? (double*)dalloc(c, sizeof(double) * (size_t)g.S) : nullptr;
-    double* ud = u3 ? (double*)dalloc(c, sizeof(double) * 3 * (size_t)g.S) : nullptr;
-    if ((rho && !rd) || (u3 && !ud)) {
+    const size_t S = (size_t)g.S;
+    // Pinned outputs are written by the kernel, pageable ones staged.
+    double* const rho_map = mapped_output(rho, S);
+    double* const u_map = mapped_output(u3, 3 * S);
+    double* rd = rho && !rho_map ? (double*)dalloc(c, sizeof(double) * S) : nullptr;
+    double* ud = u3 && !u_map ? (double*)dalloc(c, sizeof(double) * 3 * S) : nullptr;
+    if ((rho && !rho_map && !rd) || (u3 && !u_map && !ud)) {
         dfree(c, rd);
         dfree(c, ud);
         return fail(c, LBM_ERR_ALLOC, "field staging");
     }
-    cudaError_t e = launch_fields(c->storage, c->f[c->cur], g, collide_params(c), rd, ud, c->stream);
-    if (e == cudaSuccess && rho)
-        e = cudaMemcpyAsync(rho, rd, sizeof(double) * (size_t)g.S, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess && u3)
-        e = cudaMemcpyAsync(u3, ud, sizeof(double) * 3 * (size_t)g.S, cudaMemcpyDeviceToHost,
-                            c->stream);
+    cudaError_t e = launch_fields(c->storage, c->f[c->cur], g, collide_params(c),
+                                  rho_map ? rho_map : rd, u_map ? u_map : ud, c->stream);
+    if (e == cudaSuccess && rd)
+        e = cudaMemcpyAsync(rho, rd, sizeof(double) * S, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess && ud)
+        e = cudaMemcpyAsync(u3, ud, sizeof(double) * 3 * S, cudaMemcpyDeviceToHost, c->stream);
     cudaError_t e2 = cudaStreamSynchronize(c->stream);
     dfree(c, rd);
     dfree(c, ud);
@@ -923,11 +925,8 @@ int lbm_get_bubbles(lbm_ctx* c, int cap, int* n, double* pos3, double* vel3, dou
     const int k = nb < cap ? nb : cap;
     if (k == 0) return LBM_OK;
     cudaStream_t s = c->stream;
-    LBM_CUDA(download_bubble_state(c->bub, k, pos3, vel3, ul3, psi3, s), "get bubbles");
-    if (active)
-        LBM_CUDA(cudaMemcpyAsync(active, c->bub.active, sizeof(int) * (size_t)k,
-                                 cudaMemcpyDeviceToHost, s), "active");
-    LBM_CUDA(cudaStreamSynchronize(s), "get bubbles");
+    LBM_CUDA(download_bubble_state(c->bub, k, pos3, vel3, ul3, psi3, active, c->page, s),
+             "get bubbles");
     return LBM_OK;
 }
 
@@ -936,18 +935,10 @@ int lbm_get_totals(lbm_ctx* c, double* out4) {
     int rc = ensure_device(c);
     if (rc) return rc;
     const Geo g = geo_of(c);
-    const int np = totals_partials(g);
-    double* part = (double*)dalloc(c, sizeof(double) * 4 * (size_t)np + sizeof(double) * 4);
-    if (!part) return fail(c, LBM_ERR_ALLOC, "totals scratch");
-    double* out_d = part + 4 * (size_t)np;
-    cudaError_t e = launch_totals(c->storage, c->f[c->cur], g, collide_params(c), part, np, out_d,
-                                  c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out4, out_d, sizeof(double) * 4, cudaMemcpyDeviceToHost, c->stream);
-    cudaError_t e2 = cudaStreamSynchronize(c->stream);
-    dfree(c, part);
-    if (e != cudaSuccess) return cuda_fail(c, e, "totals");
-    if (e2 != cudaSuccess) return cuda_fail(c, e2, "totals (sync)");
+    LBM_CUDA(launch_totals(c->storage, c->f[c->cur], g, collide_params(c), c->tot_d,
+                           totals_partials(g), c->page->totals, c->stream), "totals");
+    LBM_CUDA(cudaStreamSynchronize(c->stream), "totals (sync)");
+    std::memcpy(out4, c->page->totals, sizeof(c->page->totals));
     return LBM_OK;
 }
 

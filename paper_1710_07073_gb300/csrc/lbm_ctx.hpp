@@ -33,7 +33,8 @@ struct lbm_ctx {
     void* f[2] = {nullptr, nullptr};
     int cur = 0;
     int* flag_d = nullptr;
-    int* flag_h = nullptr;       // pinned
+    lbm::HostPage* page = nullptr;   // pinned: what the kernels report to the host
+    double* tot_d = nullptr;     // the totals' block partials
     bool unstable = false;
 
     // bubbles

@@ -318,8 +318,10 @@ cudaError_t upload_bubble_state(const BubbleDev& B, int n, const double* pos3, c
                                 cudaStream_t st);
 // Host: the first k bubbles' state as FP64 arrays (null pointers are
 // skipped), converted on the device into B.out64.  Synchronises the stream.
+struct HostPage;
 cudaError_t download_bubble_state(const BubbleDev& B, int k, double* pos3, double* vel3,
-                                  double* ul3, double* psi3, cudaStream_t st);
+                                  double* ul3, double* psi3, int* active, HostPage* page,
+                                  cudaStream_t st);
 // Many bubbles, three launches per step, in stream order:
 //   1. per tile the current binning lists (persistent over the list of
 //      covered tiles): the Eq. 10 velocity of its nodes, and for each listed
@@ -379,6 +381,26 @@ cudaError_t launch_bubble_constants_batch(const BubbleDev& b, const BubbleConst&
 // per CTA (1, 2 or 4; the same threads per SM for each).
 int batch_min_blocks(int storage, int planes);
 int totals_partials(const Geo& g);
+constexpr int TOTALS_PARTIALS_MAX = 304;   // totals_partials' largest value
 int scan_blocks(int T);
+
+// ---- read-outs ---------------------------------------------------------------
+// Small results of the device go through one page of pinned host memory that
+// the kernels write themselves (pinned memory is mapped): a copy per array to
+// the caller's pageable memory took 5 to 10 us each.
+constexpr int PAGE_BUBBLES = 1024;   // bubbles whose state fits the page
+struct HostPage {
+    int flag, overflow;
+    double totals[4];
+    double bub[12 * PAGE_BUBBLES];
+    int active[PAGE_BUBBLES];
+};
+// page->flag = *flag, page->overflow = *overflow (0 if NULL), in stream order.
+cudaError_t launch_status(const int* flag, const int* overflow, HostPage* page, cudaStream_t st);
+// The device address of host[0, n) if all of it is pinned, mapped and
+// writable: a kernel writes such an output in place, over the link at the
+// copy engine's rate (193 GB/s measured for both) without staging.  NULL
+// otherwise.
+double* mapped_output(double* host, size_t n);
 
 }  // namespace lbm

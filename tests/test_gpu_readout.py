@@ -48,13 +48,53 @@ def test_totals_against_exact_sums(dims, walls, storage, scale):
 def test_totals_beyond_fp32_and_nan():
     col = _column((20, 12, 8), 0x3F, lbm.LBM_STORE_F32, 1.0)
     f = lbm.lbm_get_populations(col.ctx)
-    f[:1920] = 3e38            # rest populations: their FP32 sum overflows
+    f[:3840] = 3e38            # two directions: a site's FP32 sum overflows
     lbm.lbm_set_populations(col.ctx, f)
-    assert abs(lbm.lbm_get_totals(col.ctx)[0] / (1920 * 3e38) - 1.0) < 1e-6
+    assert abs(lbm.lbm_get_totals(col.ctx)[0] / (3840 * 3e38) - 1.0) < 1e-6
     f[100] = np.inf
     lbm.lbm_set_populations(col.ctx, f)
     assert lbm.lbm_get_totals(col.ctx)[0] == np.inf
     f[100] = np.nan
     lbm.lbm_set_populations(col.ctx, f)
     assert np.isnan(lbm.lbm_get_totals(col.ctx)).all()
+    col.close()
+
+
+@pytest.mark.parametrize("dims,storage,scale", [((1, 1, 1), 0, 1.0), ((13, 5, 7), 1, 256.0),
+                                                ((64, 33, 20), 0, 1.0)])
+def test_fields_written_in_place_equal_staged_ones(dims, storage, scale):
+    import torch
+    col = _column(dims, 0x3F, storage, scale)
+    S = int(np.prod(dims))
+    rho, u = lbm.lbm_get_fields(col.ctx)                    # pageable: staged and copied
+    pin = torch.full((4 * S + 2,), -7.0, dtype=torch.float64, pin_memory=True).numpy()
+    # At an offset inside a pinned block, and one array of each kind.
+    lbm.lbm_get_fields(col.ctx, out_rho=pin[1:S + 1], out_u=pin[S + 1:4 * S + 1])
+    assert np.array_equal(pin[1:S + 1], rho) and np.array_equal(pin[S + 1:4 * S + 1], u)
+    assert pin[0] == -7.0 and pin[-1] == -7.0
+    pin[:] = -7.0
+    r2, _ = lbm.lbm_get_fields(col.ctx, out_u=pin[1:3 * S + 1])
+    assert np.array_equal(r2, rho) and np.array_equal(pin[1:3 * S + 1], u)
+    b = lbm.Batch([(12, 8, 6)], [1.5])
+    br, bu = lbm.lbm_batch_get_fields(b.h, 0, 576)
+    pin = torch.empty(4 * 576, dtype=torch.float64, pin_memory=True).numpy()
+    lbm.lbm_batch_get_fields(b.h, 0, 576, out_rho=pin[:576], out_u=pin[576:])
+    assert np.array_equal(pin[:576], br) and np.array_equal(pin[576:], bu)
+    b.close()
+    col.close()
+
+
+@pytest.mark.parametrize("n", [1, 1024, 1025])
+def test_bubble_state_by_page_and_by_copies(n):
+    rng = np.random.default_rng(n)
+    col = lbm.Column((64, 64, 64), 1.6)
+    pos = 4.0 + 56.0 * rng.random((n, 3))
+    vel = rng.standard_normal((n, 3)).astype(np.float32).astype(np.float64)
+    lbm.lbm_set_bubbles(col.ctx, pos, vel, np.full(n, 2.0))
+    got = lbm.lbm_get_bubbles(col.ctx)
+    assert np.abs(got["pos"] - pos).max() <= 64.0 * 2.0 ** -47      # two floats
+    assert np.array_equal(got["vel"], vel) and got["active"].all() and len(got["active"]) == n
+    assert not got["ul"].any() and not got["psi"].any()
+    few = lbm.lbm_get_bubbles(col.ctx, cap=(n + 1) // 2)
+    assert np.array_equal(few["pos"], got["pos"][:(n + 1) // 2])
     col.close()
