@@ -462,6 +462,8 @@ long long lbm_launch_count(const lbm_ctx* ctx);
  * of long tile lists), "k_collide_stream_free<S>" (even nx, no tile lists:
  * no bubbles or no two-way coupling; the many-bubble step also launches it
  * for the blocks no bubble force reaches) or "k_collide_stream<S>" (odd nx).
+ * "k_collide_stream_pair<S,4,T>" and "k_collide_stream_free<S,4>" are the
+ * four-node sweep of 16-bit storage on rows of a multiple of 4 nodes.
  * A static string; "" for NULL. */
 const char* lbm_sweep_kernel(const lbm_ctx* ctx);
 

@@ -862,21 +862,21 @@ __device__ __forceinline__ int floor_div(int a, int b) {
 // l: layer l is guarded), ascending, then the guarded ones, ascending.  Each
 // thread places a contiguous run of blocks; a block-wide scan of the cleared
 // counts gives every run's first slot.
-__device__ void write_zperm(int nbz, const unsigned* lay, int* __restrict__ zperm) {
+__device__ void write_zperm(int nbz, int planes, const unsigned* lay, int* __restrict__ zperm) {
     __shared__ int ws[33];
     const int tid = threadIdx.x, nt = blockDim.x;
     const int per = (nbz + nt - 1) / nt;
     const int b0 = min(tid * per, nbz), b1 = min(b0 + per, nbz);
     int cleared = 0;
     for (int bz = b0; bz < b1; ++bz) {
-        const int l = (bz * SWEEP_PZ) / TZ;
+        const int l = (bz * planes) / TZ;
         cleared += !((lay[l >> 5] >> (l & 31)) & 1u);
     }
     int total;
     const int before = block_exclusive_scan(cleared, ws, total);
     int sc = before, sg = total + (b0 - before);   // guarded blocks before b0: b0 - before
     for (int bz = b0; bz < b1; ++bz) {
-        const int l = (bz * SWEEP_PZ) / TZ;
+        const int l = (bz * planes) / TZ;
         if ((lay[l >> 5] >> (l & 31)) & 1u) zperm[sg++] = bz;
         else zperm[sc++] = bz;
     }
@@ -951,7 +951,7 @@ __device__ void write_safe_layers(const Geo& g, const BubbleDev& B, const SmallB
             atomicMax(&s_zr[1], l);
         }
     }
-    if (sb.zperm != nullptr) write_zperm(sb.nbz, s_lay, sb.zperm);
+    if (sb.zperm != nullptr) write_zperm(sb.nbz, sb.planes, s_lay, sb.zperm);
     __syncthreads();
     if (sb.zrange != nullptr && tid == 0) {
         sb.zrange[0] = s_zr[0];

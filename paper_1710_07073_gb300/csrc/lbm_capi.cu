@@ -141,6 +141,7 @@ int ensure_device(lbm_ctx* c) {
     LBM_CUDA(cudaMemsetAsync(c->f[0], 0, bytes, c->stream), "memset f");
     LBM_CUDA(cudaMemsetAsync(c->flag_d, 0, sizeof(int), c->stream), "memset flag");
     c->cur = 0;
+    c->planes = sweep_planes(c->storage, c->nx, c->f[0], c->f[1]);
     LBM_CUDA(cudaMemsetAsync(c->bins.overflow, 0, sizeof(int), c->stream), "memset overflow");
     c->bins.items = nullptr;
     c->bins.cap = 0;
@@ -196,11 +197,13 @@ void guard_invalidate(lbm_ctx* c) {
 
 namespace {
 
+int sweep_blocks(const lbm_ctx* c, const Geo& g) { return (g.nz + c->planes - 1) / c->planes; }
+
 // Two tag sets of ntz (zero: no layer cleared) and two sweep orders of nbz z
 // blocks (identity), by step parity.
 int alloc_guard(lbm_ctx* c, unsigned** safe, int** zperm, int* nbz, int** zrange) {
     const Geo g = geo_of(c);
-    *nbz = sweep_z_blocks(g.nz);
+    *nbz = sweep_blocks(c, g);
     *safe = (unsigned*)dalloc(c, 2 * sizeof(unsigned) * (size_t)g.ntz);
     *zperm = (int*)dalloc(c, 2 * sizeof(int) * (size_t)*nbz);
     *zrange = (int*)dalloc(c, 2 * sizeof(int));
@@ -286,15 +289,15 @@ bool guarded_blocks(lbm_ctx* c, const Geo& g, int* b0, int* b1, int* rc) {
     }
     static_assert(GUARD_CELLS <= TZ, "a bubble crosses at most one tile layer per step");
     const int zlo = c->zr_host[2 * slot], zhi = c->zr_host[2 * slot + 1];
-    const int nbz = sweep_z_blocks(g.nz);
+    const int nbz = sweep_blocks(c, g);
     if (zhi < zlo) {
         *b0 = *b1 = 0;
         return true;
     }
     const int widen = (int)(n - m) + 1;
     const int l0 = std::max(0, zlo - widen), l1 = std::min(g.ntz - 1, zhi + widen);
-    *b0 = std::min(nbz, l0 * TZ / SWEEP_PZ);
-    *b1 = std::min(nbz, (l1 + 1) * TZ / SWEEP_PZ);
+    *b0 = std::min(nbz, l0 * TZ / c->planes);
+    *b1 = std::min(nbz, (l1 + 1) * TZ / c->planes);
     return true;
 }
 
@@ -348,7 +351,7 @@ int enqueue_one_step(lbm_ctx* c) {
     }
     cudaStream_t st = c->stream;   // the update and the guarded sweep
     if (split) {
-        const int nbz = sweep_z_blocks(g.nz);
+        const int nbz = sweep_blocks(c, g);
         LBM_CUDA(cudaEventRecord(c->ev_fork, c->stream), "fork");
         LBM_CUDA(cudaStreamWaitEvent(c->side_hi, c->ev_fork, 0), "fork");
         LBM_CUDA(cudaStreamWaitEvent(c->side_lo, c->ev_fork, 0), "fork");
@@ -804,6 +807,7 @@ int lbm_set_bubbles(lbm_ctx* c, int n, const double* pos3, const double* vel3,
         // Overlap guard: tags and sweep orders, one set per step parity.
         if (c->bins.T > 0 && geo_of(c).ntz <= GUARD_LAYERS_MAX) {
             int rc = alloc_guard(c, &sb.safe, &sb.zperm, &sb.nbz, &sb.zrange);
+            sb.planes = c->planes;
             if (rc == LBM_ERR_CUDA) {
                 free_bubbles(c);
                 return rc;
@@ -1035,8 +1039,16 @@ const char* lbm_sweep_kernel(const lbm_ctx* c) {
                                           "k_collide_stream<2>"};
     static const char* const free_[3] = {"k_collide_stream_free<0>", "k_collide_stream_free<1>",
                                          "k_collide_stream_free<2>"};
+    static const char* const pair4[3][2] = {
+        {"", ""},
+        {"k_collide_stream_pair<1,4,0>", "k_collide_stream_pair<1,4,1>"},
+        {"k_collide_stream_pair<2,4,0>", "k_collide_stream_pair<2,4,1>"}};
+    static const char* const free4[3] = {"", "k_collide_stream_free<1,4>",
+                                         "k_collide_stream_free<2,4>"};
     const int st = c->storage < 0 || c->storage > 2 ? 0 : c->storage;
     if (c->nx & 1) return single[st];
+    if (sweep_planes(st, c->nx, c->f[0], c->f[1]) != SWEEP_PZ)   // four nodes per thread
+        return c->bub.nb > 0 && c->p.two_way ? pair4[st][c->use_small ? 0 : 1] : free4[st];
     if (!(c->bub.nb > 0 && c->p.two_way)) return free_[st];   // no tile lists
     return pair[st][c->use_small ? 0 : 1];
 }

@@ -554,9 +554,382 @@ __device__ __forceinline__ void sweep_block(const typename Store<ST>::T* __restr
     else collide_pair<ST, false>(sink, rv, Fx, Fy, Fz, cp, flag, active);
 }
 
-// TAB: the force gather of long tile lists (per-axis weight tables).
+// ---------------------------------------------------------------------------
+// Four nodes per thread: 16-bit storage on rows whose length is a multiple of
+// 4.  A CTA is 8 x 4 x 4 threads = one 32 x 4 x 4 binning tile.
+//
+// The 16-bit sweep moves half the bytes of FP32 per node, so with two nodes per
+// thread it was bound by its load latency and instructions (82 % of the copy
+// peak, 256 x 256 x 512).  Four nodes halve the row loads, the x-crossing loads
+// and the address arithmetic per node and double the bytes a thread has in
+// flight.  The raw values wait in shared memory (QuadSlot): kept in registers
+// the kernel spilled at 80 registers and lost (0.476 ms).  At 6 CTAs per SM
+// (80 registers, no spills without force; 4: 0.410, 5: 0.396, 7: 0.427,
+// 8: 0.476 ms) the 256 x 256 x 512 FP16 step takes 0.391 ms against 0.444 ms
+// with two nodes (96 % of the copy peak), the 384 x 384 x 768 swarm's FP16 step
+// 1.953 against 2.116 ms, its whole listed sweep 1.660 against 1.777 ms.
+// ---------------------------------------------------------------------------
+constexpr int QX = TX / 4;      // threads along x
+constexpr int QUAD_PZ = TZ;     // z-planes per CTA
+constexpr int QUAD_THREADS = QX * TY * QUAD_PZ;
+#ifndef LBM_QUAD_MINB
+#define LBM_QUAD_MINB 6
+#endif
+// CTA shape and residency of the sweep kernels, by nodes per thread.
+template <int ST, int NODES> struct SweepShape {
+    static constexpr int kThreads = PX * TY * PZ;
+    static constexpr int kMinBlocks = PairOccupancy<ST>::kMinBlocks;
+};
+template <int ST> struct SweepShape<ST, 4> {
+    static constexpr int kThreads = QUAD_THREADS;
+    static constexpr int kMinBlocks = LBM_QUAD_MINB;
+};
+
+// The raw values of a thread's quads wait in shared memory between the moments
+// and the relaxation (a slot per thread, so no synchronisation): held in
+// registers, packed and widened, they spill at any occupancy that hides the
+// load latency.
+struct QuadSlot {
+    unsigned at;   // shared-space address of direction 0
+    static constexpr unsigned STRIDE = QUAD_THREADS * 8;
+    template <int J>
+    __device__ __forceinline__ void put(unsigned a, unsigned b) const {
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at + J * STRIDE), "r"(a), "r"(b));
+    }
+    template <int J>
+    __device__ __forceinline__ void put_a(unsigned a) const {
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(at + J * STRIDE), "r"(a));
+    }
+    // Half H (0: first pair, 1: second) of direction J.
+    template <int J, int H>
+    __device__ __forceinline__ unsigned get_half() const {
+        unsigned v;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at + J * STRIDE + 4 * H));
+        return v;
+    }
+    template <int H>
+    __device__ __forceinline__ void get_all(unsigned v[Q]) const {
+#define LBM_GH(J) v[J] = get_half<J, H>()
+        LBM_GH(0); LBM_GH(1); LBM_GH(2); LBM_GH(3); LBM_GH(4); LBM_GH(5); LBM_GH(6);
+        LBM_GH(7); LBM_GH(8); LBM_GH(9); LBM_GH(10); LBM_GH(11); LBM_GH(12); LBM_GH(13);
+        LBM_GH(14); LBM_GH(15); LBM_GH(16); LBM_GH(17); LBM_GH(18);
+#undef LBM_GH
+    }
+    template <int J>
+    __device__ __forceinline__ Quad get() const {
+        Quad q;
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
+                     : "=r"(q.a), "=r"(q.b)
+                     : "r"(at + J * STRIDE));
+        return q;
+    }
+};
+
+// What the relaxation of one pair needs (collide_pair's values).
+struct PairState {
+    float2 ux, uy, uz, uF;
+    RelaxK k;
+    float2 rest;   // C0 e0
+};
+
+template <int ST, bool FORCED>
+__device__ __forceinline__ PairState pair_state(const unsigned rr[Q], float2 Fx, float2 Fy,
+                                                float2 Fz, const CollideParams& cp, int* flag,
+                                                bool live) {
+    static_assert(Store<ST>::kScaled, "16-bit storage: one coefficient class");
+    PairState p;
+    float2 drho, jx, jy, jz;
+    pair_moments<ST>(rr, cp, drho, jx, jy, jz);
+    const float2 rho = add2(f2(cp.rho0), drho);
+    const float2 inv_rho = make_float2(1.0f / rho.x, 1.0f / rho.y);
+    if (FORCED) {
+        p.ux = mul2(fma2(f2(0.5f), Fx, jx), inv_rho);
+        p.uy = mul2(fma2(f2(0.5f), Fy, jy), inv_rho);
+        p.uz = mul2(fma2(f2(0.5f), Fz, jz), inv_rho);
+    } else {
+        p.ux = mul2(jx, inv_rho);
+        p.uy = mul2(jy, inv_rho);
+        p.uz = mul2(jz, inv_rho);
+    }
+    const float2 usq = fma2(p.ux, p.ux, fma2(p.uy, p.uy, mul2(p.uz, p.uz)));
+    if (live && !(usq.x < 0.09f && usq.y < 0.09f)) atomicOr(flag, 1);
+    p.uF = FORCED ? fma2(p.ux, Fx, fma2(p.uy, Fy, mul2(p.uz, Fz))) : f2(0.0f);
+    const float2 base = fma2(mul2(f2(-1.5f), rho), usq, drho);
+    float2 e0 = mul2(f2(cp.omega), base);
+    if (FORCED) e0 = fma2(f2(-3.0f * cp.pref), p.uF, e0);
+    p.rest = mul2(f2(cp.scale), e0);
+    p.k = relax_k(cp.scale * cp.omega, base, rho);
+    return p;
+}
+
+// One pair's post-collision values of J and its opposite (relax_pair2).
+template <int ST>
+struct PackedPair {
+    unsigned v[2];
+    template <int J>
+    __device__ __forceinline__ void put(float2 x) { v[(J + 1) & 1] = Raw2<ST>::pack(x); }
+};
+
+template <int ST, int J, bool FORCED>
+__device__ __forceinline__ void relax_quad(typename Store<ST>::T* __restrict__ fout, unsigned S,
+                                           unsigned site0, const QuadSlot& slot,
+                                           const PairState& pa, const PairState& pb,
+                                           const float2 F[6], const CollideParams& cp,
+                                           bool active) {
+    unsigned ra[Q], rb[Q];   // only [J] and [J + 1] are used
+    const Quad q0 = slot.get<J>(), q1 = slot.get<J + 1>();
+    ra[J] = q0.a;
+    ra[J + 1] = q1.a;
+    rb[J] = q0.b;
+    rb[J + 1] = q1.b;
+    PackedPair<ST> a, b;
+    relax_pair2<ST, J, FORCED>(a, ra, pa.k, pa.ux, pa.uy, pa.uz, F[0], F[1], F[2], pa.uF, cp);
+    relax_pair2<ST, J, FORCED>(b, rb, pb.k, pb.ux, pb.uy, pb.uz, F[3], F[4], F[5], pb.uF, cp);
+    if (active) {
+        __stcs(reinterpret_cast<uint2*>(fout + ((unsigned)J * S + site0)), make_uint2(a.v[0], b.v[0]));
+        __stcs(reinterpret_cast<uint2*>(fout + ((unsigned)(J + 1) * S + site0)),
+               make_uint2(a.v[1], b.v[1]));
+    }
+}
+
+// Forced relaxation of one pair of a quad: the first pair's results go back
+// into the slot, the second's are stored together with them.
+template <int ST, int J, bool SECOND>
+__device__ __forceinline__ void relax_half(typename Store<ST>::T* __restrict__ fout, unsigned S,
+                                           unsigned site0, const QuadSlot& slot,
+                                           const PairState& p, const float2* F,
+                                           const CollideParams& cp, bool active) {
+    unsigned r[Q];   // only [J] and [J + 1] are used
+    const Quad q0 = slot.get<J>(), q1 = slot.get<J + 1>();
+    r[J] = SECOND ? q0.b : q0.a;
+    r[J + 1] = SECOND ? q1.b : q1.a;
+    PackedPair<ST> v;
+    relax_pair2<ST, J, true>(v, r, p.k, p.ux, p.uy, p.uz, F[0], F[1], F[2], p.uF, cp);
+    if (!SECOND) {
+        slot.put_a<J>(v.v[0]);
+        slot.put_a<J + 1>(v.v[1]);
+    } else if (active) {
+        __stcs(reinterpret_cast<uint2*>(fout + ((unsigned)J * S + site0)), make_uint2(q0.a, v.v[0]));
+        __stcs(reinterpret_cast<uint2*>(fout + ((unsigned)(J + 1) * S + site0)),
+               make_uint2(q1.a, v.v[1]));
+    }
+}
+
+// Collision of a quad whose raw values are in A, B and in the slot.  Without
+// force the two pairs' states fit the registers side by side; with it the raw
+// values are read back (none are held through the force gather) and one pair
+// is finished before the other begins.
+template <int ST, bool FORCED>
+__device__ __forceinline__ void collide_quad(typename Store<ST>::T* __restrict__ fout, unsigned S,
+                                             unsigned site0, const unsigned A[Q],
+                                             const unsigned B[Q], const QuadSlot& slot,
+                                             const float2 F[6], const CollideParams& cp,
+                                             int* flag, bool active) {
+    const float2 om1 = f2(1.0f - cp.omega);
+    if (!FORCED) {
+        const PairState pa = pair_state<ST, false>(A, F[0], F[1], F[2], cp, flag, active);
+        const PairState pb = pair_state<ST, false>(B, F[3], F[4], F[5], cp, flag, active);
+        const Quad q = slot.get<0>();
+        if (active)
+            __stcs(reinterpret_cast<uint2*>(fout + site0),
+                   make_uint2(Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(q.a), pa.rest)),
+                              Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(q.b), pb.rest))));
+#define LBM_RQ(J) relax_quad<ST, J, false>(fout, S, site0, slot, pa, pb, F, cp, active)
+        LBM_RQ(1); LBM_RQ(3); LBM_RQ(5); LBM_RQ(7); LBM_RQ(9);
+        LBM_RQ(11); LBM_RQ(13); LBM_RQ(15); LBM_RQ(17);
+#undef LBM_RQ
+        return;
+    }
+#define LBM_RH(J, N) relax_half<ST, J, N>(fout, S, site0, slot, p, F + 3 * N, cp, active)
+    {
+        unsigned v[Q];
+        slot.get_all<0>(v);
+        const PairState p = pair_state<ST, true>(v, F[0], F[1], F[2], cp, flag, active);
+        slot.put_a<0>(Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(slot.get<0>().a), p.rest)));
+        LBM_RH(1, 0); LBM_RH(3, 0); LBM_RH(5, 0); LBM_RH(7, 0); LBM_RH(9, 0);
+        LBM_RH(11, 0); LBM_RH(13, 0); LBM_RH(15, 0); LBM_RH(17, 0);
+    }
+    {
+        unsigned v[Q];
+        slot.get_all<1>(v);
+        const PairState p = pair_state<ST, true>(v, F[3], F[4], F[5], cp, flag, active);
+        const Quad q = slot.get<0>();
+        if (active)
+            __stcs(reinterpret_cast<uint2*>(fout + site0),
+                   make_uint2(q.a, Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(q.b), p.rest))));
+        LBM_RH(1, 1); LBM_RH(3, 1); LBM_RH(5, 1); LBM_RH(7, 1); LBM_RH(9, 1);
+        LBM_RH(11, 1); LBM_RH(13, 1); LBM_RH(15, 1); LBM_RH(17, 1);
+    }
+#undef LBM_RH
+}
+
+// The slot of this thread in s_raw[Q][QUAD_THREADS], filled with its raw values.
+__device__ __forceinline__ QuadSlot fill_slot(uint2* s_raw, const unsigned A[Q],
+                                              const unsigned B[Q]) {
+    const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
+    const QuadSlot slot{(unsigned)__cvta_generic_to_shared(s_raw + tid)};
+#define LBM_SP(J) slot.put<J>(A[J], B[J])
+    LBM_SP(0); LBM_SP(1); LBM_SP(2); LBM_SP(3); LBM_SP(4); LBM_SP(5); LBM_SP(6);
+    LBM_SP(7); LBM_SP(8); LBM_SP(9); LBM_SP(10); LBM_SP(11); LBM_SP(12); LBM_SP(13);
+    LBM_SP(14); LBM_SP(15); LBM_SP(16); LBM_SP(17); LBM_SP(18);
+#undef LBM_SP
+    return slot;
+}
+
+// Eq. 21 at the quad (x0 .. x0 + 3), (y, z) of a tile with long lists: as
+// gather_force_tab (same products and order), over the whole tile.  A warp is
+// one z-plane, so it visits only the listed bubbles whose z weight there is
+// not zero.  Every thread of the CTA calls it.
+template <int ST>
+__device__ __forceinline__ void gather_force_quad(const Geo& g, const int* __restrict__ items,
+                                                  const BubbleRec* __restrict__ recs, int nb,
+                                                  int beg, int end, int bx, int by, int bz,
+                                                  bool point, BubbleRec* srec, float2 F[6]) {
+    constexpr int FB = FORCE_CHUNK, NAX = TX + TY + TZ;
+    static_assert(FB == 32 && QX * TY == 32, "a lane per staged bubble, a warp per plane");
+    __shared__ __align__(16) float s_w[FB][NAX];   // x: [0, TX), y: [TX, TX + TY), z: the rest
+    const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
+    const int xb0 = bx * TX, yb0 = by * TY, zb0 = bz * TZ;
+    for (int c0 = beg; c0 < end; c0 += FB) {
+        const int cnt = min(FB, end - c0);
+        __syncthreads();
+        if (tid < cnt) {
+            const int id = __ldcg(items + c0 + tid);
+            if (id >= 0 && id < nb) srec[tid] = load_rec(recs + id);
+            else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        }
+        __syncthreads();
+        auto tabulate = [&](auto mode) {
+            constexpr int PM = decltype(mode)::value;
+            for (int e = tid; e < cnt * NAX; e += QUAD_THREADS) {
+                const int k = e / NAX, q = e - k * NAX;
+                const BubbleRec& r = srec[k];
+                if (q < TX)
+                    s_w[k][q] = axis_weight<PM>(r, xb0 + q, r.ax, r.fx, g.nx, !(g.walls & 0x01));
+                else if (q < TX + TY)
+                    s_w[k][q] = axis_weight<PM>(r, yb0 + q - TX, r.ay, r.fy, g.ny, !(g.walls & 0x04));
+                else
+                    s_w[k][q] =
+                        axis_weight<PM>(r, zb0 + q - TX - TY, r.az, r.fz, g.nz, !(g.walls & 0x10));
+            }
+        };
+        if (point) tabulate(MapMode<MAP_POINT>{});
+        else tabulate(MapMode<MAP_CELL>{});
+        __syncthreads();
+        const int lane = tid & 31, yi = TX + threadIdx.y, zi = TX + TY + threadIdx.z;
+        unsigned todo = __ballot_sync(0xffffffffu, lane < cnt && s_w[lane < cnt ? lane : 0][zi] != 0.0f);
+        while (todo) {
+            const int k = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float wyz = s_w[k][yi] * s_w[k][zi];
+            if (wyz == 0.0f) continue;
+            const float4 wx = *reinterpret_cast<const float4*>(&s_w[k][4 * threadIdx.x]);
+            const BubbleRec& r = srec[k];
+            const float2 wa = make_float2(wx.x * wyz, wx.y * wyz);
+            const float2 wb = make_float2(wx.z * wyz, wx.w * wyz);
+            F[0] = fma2(wa, f2(r.px), F[0]);
+            F[1] = fma2(wa, f2(r.py), F[1]);
+            F[2] = fma2(wa, f2(r.pz), F[2]);
+            F[3] = fma2(wb, f2(r.px), F[3]);
+            F[4] = fma2(wb, f2(r.py), F[4]);
+            F[5] = fma2(wb, f2(r.pz), F[5]);
+        }
+    }
+}
+
+// One CTA's tile of the sweep (sweep_block with four nodes per thread).
 template <int ST, bool TAB>
-__global__ void __launch_bounds__(PX * TY * PZ, PairOccupancy<ST>::kMinBlocks)
+__device__ __forceinline__ void quad_block(const typename Store<ST>::T* __restrict__ fin,
+                                           typename Store<ST>::T* __restrict__ fout,
+                                           const Geo& g, const CollideParams& cp,
+                                           const int* __restrict__ tile_start,
+                                           const int* __restrict__ tile_count,
+                                           const int* __restrict__ items, int cap,
+                                           const BubbleRec* __restrict__ recs, int nb,
+                                           int* __restrict__ flag, int bx, int by, int bz,
+                                           BubbleRec* srec, const unsigned* safe,
+                                           unsigned epoch, bool lead) {
+    __shared__ uint2 s_raw[Q * QUAD_THREADS];
+    const int x0 = bx * TX + 4 * threadIdx.x;
+    const int y = by * TY + threadIdx.y;
+    const int z = bz * QUAD_PZ + threadIdx.z;
+    const bool active = (x0 < g.nx) && (y < g.ny) && (z < g.nz);
+    // Inactive threads gather at a valid node and store nothing.
+    const int xa = active ? x0 : 0;
+    const int ya = min(y, g.ny - 1), za = min(z, g.nz - 1);
+    const int t = (bz * g.nty + by) * g.ntx + bx;
+    // The order of the tile count, the population loads and the wait for an
+    // overlapped update is sweep_block's.
+    int n_t = 0;
+    bool skip = false;
+    if (tile_count != nullptr) {
+        if (safe == nullptr) n_t = __ldcg(tile_count + t);
+        else skip = !lead && __ldcg(safe + bz) == epoch;
+    }
+    unsigned A[Q], B[Q];
+    gather_quad<ST>(fin, g, xa, ya, za, A, B);
+    if (tile_count != nullptr && safe != nullptr && !skip) {
+        pdl_wait();
+        n_t = __ldcg(tile_count + t);
+    }
+    const QuadSlot slot = fill_slot(s_raw, A, B);
+    const unsigned S = (unsigned)g.S;
+    const unsigned site0 = (unsigned)site_index(g, xa, ya, za);
+    float2 F[6] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
+    if (n_t > 0) {   // uniform over the CTA (one tile)
+        const int beg = __ldcg(tile_start + t);
+        const int end = min(beg + n_t, cap);
+        if (TAB) {
+            gather_force_quad<ST>(g, items, recs, nb, beg, end, bx, by, bz, cp.point != 0, srec, F);
+        } else {
+            const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
+            for (int c0 = beg; c0 < end; c0 += FORCE_CHUNK) {
+                const int cnt = min(FORCE_CHUNK, end - c0);
+                __syncthreads();
+                if (tid < cnt) {
+                    const int id = __ldcg(items + c0 + tid);
+                    if (id >= 0 && id < nb) srec[tid] = load_rec(recs + id);
+                    else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                }
+                __syncthreads();
+                if (active)
+                    for (int k = 0; k < cnt; ++k) {
+                        add_bubble_force_pair(srec[k], g, x0, y, z, F[0], F[1], F[2]);
+                        add_bubble_force_pair(srec[k], g, x0 + 2, y, z, F[3], F[4], F[5]);
+                    }
+            }
+        }
+        collide_quad<ST, true>(fout, S, site0, A, B, slot, F, cp, flag, active);
+    } else {
+        collide_quad<ST, false>(fout, S, site0, A, B, slot, F, cp, flag, active);
+    }
+}
+
+// The same of a block no bubble force reaches.
+template <int ST>
+__device__ __forceinline__ void quad_block_free(const typename Store<ST>::T* __restrict__ fin,
+                                                typename Store<ST>::T* __restrict__ fout,
+                                                const Geo& g, const CollideParams& cp,
+                                                int* __restrict__ flag, int bx, int by, int bz) {
+    __shared__ uint2 s_raw[Q * QUAD_THREADS];
+    const int x0 = bx * TX + 4 * threadIdx.x;
+    const int y = by * TY + threadIdx.y;
+    const int z = bz * QUAD_PZ + threadIdx.z;
+    const bool active = (x0 < g.nx) && (y < g.ny) && (z < g.nz);
+    const int xa = active ? x0 : 0;
+    const int ya = min(y, g.ny - 1), za = min(z, g.nz - 1);
+    unsigned A[Q], B[Q];
+    gather_quad<ST>(fin, g, xa, ya, za, A, B);
+    const float2 F[6] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
+    const QuadSlot slot = fill_slot(s_raw, A, B);
+    collide_quad<ST, false>(fout, (unsigned)g.S, (unsigned)site_index(g, xa, ya, za), A, B, slot,
+                            F, cp, flag, active);
+}
+
+// TAB: the force gather of long tile lists (per-axis weight tables).  NODES:
+// nodes per thread along x (four: quad_block below).
+template <int ST, int NODES, bool TAB>
+__global__ void __launch_bounds__(SweepShape<ST, NODES>::kThreads, SweepShape<ST, NODES>::kMinBlocks)
 k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
                       typename Store<ST>::T* __restrict__ fout, Geo g, CollideParams cp,
                       const int* tile_start, const int* tile_count, const int* items, int cap,
@@ -572,8 +945,12 @@ k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
     if (bz >= zs.hole) bz += zs.skip;
     if (zperm != nullptr) bz = __ldcg(zperm + blockIdx.z);
     const bool lead = (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
-    sweep_block<ST, TAB>(fin, fout, g, cp, tile_start, tile_count, items, cap, recs, nb, flag,
-                         blockIdx.x, blockIdx.y, bz, srec, safe, epoch, lead);
+    if constexpr (NODES == 4)
+        quad_block<ST, TAB>(fin, fout, g, cp, tile_start, tile_count, items, cap, recs, nb, flag,
+                            blockIdx.x, blockIdx.y, bz, srec, safe, epoch, lead);
+    else
+        sweep_block<ST, TAB>(fin, fout, g, cp, tile_start, tile_count, items, cap, recs, nb, flag,
+                             blockIdx.x, blockIdx.y, bz, srec, safe, epoch, lead);
 }
 
 // Sweeps without tile lists (no two-way coupling, or the blocks no bubble
@@ -581,13 +958,17 @@ k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
 // (collide_pair<ST, false>, as k_collide_stream_pair runs it for a block with
 // an empty list), in a kernel without the force-gather code: the 16-bit
 // sweep runs about 3 % faster in it than in k_collide_stream_pair.
-template <int ST>
-__global__ void __launch_bounds__(PX * TY * PZ, PairOccupancy<ST>::kMinBlocks)
+template <int ST, int NODES>
+__global__ void __launch_bounds__(SweepShape<ST, NODES>::kThreads, SweepShape<ST, NODES>::kMinBlocks)
 k_collide_stream_free(const typename Store<ST>::T* __restrict__ fin,
                       typename Store<ST>::T* __restrict__ fout, Geo g, CollideParams cp,
                       int* __restrict__ flag, ZSpan zs) {
     int bz = zs.first + (int)blockIdx.z;
     if (bz >= zs.hole) bz += zs.skip;
+    if constexpr (NODES == 4) {
+        quad_block_free<ST>(fin, fout, g, cp, flag, blockIdx.x, blockIdx.y, bz);
+        return;
+    }
     const int x0 = blockIdx.x * TX + 2 * threadIdx.x;
     const int y = blockIdx.y * TY + threadIdx.y;
     const int z = bz * PZ + threadIdx.z;
@@ -680,7 +1061,13 @@ cudaError_t launch_collide_batch(int storage, const void* fin, void* fout,
     return cudaGetLastError();
 }
 
-int sweep_z_blocks(int nz) { return (nz + PZ - 1) / PZ; }
+int sweep_planes(int storage, int nx, const void* fa, const void* fb) {
+    // Four nodes per thread wherever rows of 16-bit values can be read 8
+    // bytes at a time.
+    const bool quad = storage != 0 && (nx & 3) == 0 && ((uintptr_t)fa & 7) == 0 &&
+                      ((uintptr_t)fb & 7) == 0;
+    return quad ? QUAD_PZ : PZ;
+}
 int batch_min_blocks(int storage, int planes) {
     const int k = storage == 0 ? PairOccupancy<0>::kMinBlocks : PairOccupancy<1>::kMinBlocks;
     return k * PZ / planes;
@@ -697,7 +1084,9 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
     const int cap = tl ? tl->cap : 0;
     if (overlap && (safe == nullptr || tl == nullptr)) return cudaErrorInvalidValue;
     if (!overlap) safe = nullptr;
-    const int nbz = (g.nz + PZ - 1) / PZ;
+    const bool quad = sweep_planes(storage, g.nx, fin, fout) == QUAD_PZ;
+    const int planes = quad ? QUAD_PZ : PZ;
+    const int nbz = (g.nz + planes - 1) / planes;
     ZSpan zs{0, nbz, INT_MAX, 0};
     if (span) {
         if ((g.nx & 1) || zperm || span->count < 0 || span->first < 0 || span->skip < 0 ||
@@ -711,7 +1100,7 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
         // lists longer than the few-bubble path's (many bubbles per tile)
         // take the tabulated force gather.
         cudaLaunchConfig_t cfg = {};
-        cfg.blockDim = dim3(PX, TY, PZ);
+        cfg.blockDim = quad ? dim3(QX, TY, QUAD_PZ) : dim3(PX, TY, PZ);
         cfg.gridDim = dim3((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (unsigned)zs.count);
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
@@ -721,24 +1110,47 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
         cfg.numAttrs = overlap ? 1 : 0;
         if (tl == nullptr && zperm == nullptr && !overlap) {
             // No bubble force reaches these blocks.
+            if (quad && storage == 1)
+                return cudaLaunchKernelEx(&cfg, k_collide_stream_free<1, 4>, (const __half*)fin,
+                                          (__half*)fout, g, cp, flag, zs);
+            if (quad)
+                return cudaLaunchKernelEx(&cfg, k_collide_stream_free<2, 4>,
+                                          (const __nv_bfloat16*)fin, (__nv_bfloat16*)fout, g, cp,
+                                          flag, zs);
             switch (storage) {
                 case 0:
-                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<0>, (const float*)fin,
+                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<0, 2>, (const float*)fin,
                                               (float*)fout, g, cp, flag, zs);
                 case 1:
-                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<1>, (const __half*)fin,
+                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<1, 2>, (const __half*)fin,
                                               (__half*)fout, g, cp, flag, zs);
                 default:
-                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<2>,
+                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<2, 2>,
                                               (const __nv_bfloat16*)fin, (__nv_bfloat16*)fout, g,
                                               cp, flag, zs);
             }
         }
         const bool tab = tl != nullptr && tl->cap > SMALL_MAX_PAIRS;
+        if (quad) {
+            switch (storage * 2 + (tab ? 1 : 0)) {
+#define LBM_LAUNCH_QUAD(SI, TB, T)                                                                \
+    case SI * 2 + TB:                                                                             \
+        return cudaLaunchKernelEx(&cfg, k_collide_stream_pair<SI, 4, TB>, (const T*)fin, (T*)fout,   \
+                                  g, cp, start, count, items, cap, recs, nb, flag, safe, epoch,  \
+                                  zperm, zs);
+                LBM_LAUNCH_QUAD(1, 0, __half)
+                LBM_LAUNCH_QUAD(1, 1, __half)
+                LBM_LAUNCH_QUAD(2, 0, __nv_bfloat16)
+                LBM_LAUNCH_QUAD(2, 1, __nv_bfloat16)
+#undef LBM_LAUNCH_QUAD
+                default:
+                    return cudaErrorInvalidValue;
+            }
+        }
         switch (storage * 2 + (tab ? 1 : 0)) {
 #define LBM_LAUNCH_PAIR(SI, TB, T)                                                                \
     case SI * 2 + TB:                                                                             \
-        return cudaLaunchKernelEx(&cfg, k_collide_stream_pair<SI, TB>, (const T*)fin, (T*)fout,   \
+        return cudaLaunchKernelEx(&cfg, k_collide_stream_pair<SI, 2, TB>, (const T*)fin, (T*)fout,   \
                                   g, cp, start, count, items, cap, recs, nb, flag, safe, epoch,  \
                                   zperm, zs);
             LBM_LAUNCH_PAIR(0, 0, float)

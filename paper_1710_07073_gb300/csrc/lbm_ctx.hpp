@@ -32,6 +32,7 @@ struct lbm_ctx {
     int device = 0;
     void* f[2] = {nullptr, nullptr};
     int cur = 0;
+    int planes = lbm::SWEEP_PZ;  // z-planes of a sweep block (sweep_planes)
     int* flag_d = nullptr;
     lbm::HostPage* page = nullptr;   // pinned: what the kernels report to the host
     double* tot_d = nullptr;     // the totals' block partials

@@ -339,12 +339,22 @@ template <int ST> struct Raw2 {
     static __device__ __forceinline__ T hi_from(T P, T1 a) { return __byte_perm(P, a, 0x5432); }
     static __device__ __forceinline__ T join(T1 a, T1 b) { return __byte_perm(a, b, 0x5410); }
     static __device__ __forceinline__ float2 widen(T v);
+    static __device__ __forceinline__ T pack(float2 v);
 };
 template <> __device__ __forceinline__ float2 Raw2<1>::widen(unsigned v) {
     return __half22float2(*reinterpret_cast<const __half2*>(&v));
 }
 template <> __device__ __forceinline__ float2 Raw2<2>::widen(unsigned v) {
     return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
+// As Vec2<ST>::store rounds.
+template <> __device__ __forceinline__ unsigned Raw2<1>::pack(float2 v) {
+    const __half2 h = __floats2half2_rn(v.x, v.y);
+    return *reinterpret_cast<const unsigned*>(&h);
+}
+template <> __device__ __forceinline__ unsigned Raw2<2>::pack(float2 v) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+    return *reinterpret_cast<const unsigned*>(&h);
 }
 template <> struct Raw2<0> {
     using T = float2;
@@ -462,6 +472,109 @@ __device__ __forceinline__ void gather_pair(const typename Store<ST>::T* __restr
         LBM_PA(10); LBM_PA(11); LBM_PA(12); LBM_PA(13); LBM_PA(14);
         LBM_PA(15); LBM_PA(16); LBM_PA(17); LBM_PA(18);
 #undef LBM_PA
+    }
+}
+
+// ---- four nodes per thread (16-bit storage, nx a multiple of 4) ---------------
+// A thread owns the nodes x0 .. x0 + 3 (x0 a multiple of 4) as two packed
+// pairs, so a row is one aligned 8-byte access for four nodes and a population
+// crossing x costs one 2-byte load per four nodes.  A[J], B[J]: the raw values
+// of direction J arriving at (x0, x0 + 1) and (x0 + 2, x0 + 3).
+struct Quad {
+    unsigned a, b;
+};
+
+__device__ __forceinline__ Quad quad_load(const void* p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    return Quad{v.x, v.y};
+}
+
+// The quad of a source row P shifted by c_x: the node at the end of the shift
+// takes e, the value crossing from the neighbouring quad.
+template <int C>
+__device__ __forceinline__ Quad quad_shift(Quad P, unsigned e) {
+    if (C == 1) return Quad{__byte_perm(e, P.a, 0x5410), __byte_perm(P.a, P.b, 0x5432)};
+    return Quad{__byte_perm(P.a, P.b, 0x5432), __byte_perm(P.b, e, 0x5432)};
+}
+
+// Direction J at a row whose source row starts at `row` (plane and row offset
+// plus x0); own: the nodes' own site in direction opp(J)'s plane.
+template <int ST, int J>
+__device__ __forceinline__ Quad pull_quad(const typename Store<ST>::T* __restrict__ f,
+                                          unsigned row, unsigned own, unsigned nx, int x0,
+                                          bool wallx) {
+    const Quad P = quad_load(f + row);
+    if (cx(J) == 0) return P;
+    unsigned e;
+    if (cx(J) == 1) {
+        e = row - 1u;
+        if (x0 == 0) e = wallx ? own : row + nx - 1u;
+    } else {
+        e = row + 4u;
+        if ((unsigned)x0 + 4u >= nx) e = wallx ? own + 3u : row - (unsigned)x0;
+    }
+    return quad_shift<cx(J)>(P, Raw2<ST>::load1(f + e));
+}
+
+// Any row: the source row follows from y and z alone (wrap, bounce-back or the
+// free-slip mirror, as pull_source); a row that bounces off a y or z wall
+// takes the opposite plane of its own nodes, unshifted.
+template <int ST, int J>
+__device__ __forceinline__ Quad pull_quad_any(const typename Store<ST>::T* __restrict__ f,
+                                              const Geo& g, int x0, int y, int z) {
+    int sy = y - cy(J), sz = z - cz(J);
+    bool bounce = false, specular = false;
+    if (cy(J) != 0) {
+        const bool out = (unsigned)sy >= (unsigned)g.ny;
+        bounce = out && (g.walls & 0x04);
+        sy = out ? (sy < 0 ? sy + g.ny : sy - g.ny) : sy;
+    }
+    if (cz(J) != 0) {
+        const bool out = (unsigned)sz >= (unsigned)g.nz;
+        specular = cz(J) < 0 && out && (g.walls & WALL_TOP_FREE);
+        bounce = bounce || (out && !specular && (g.walls & 0x10));
+        sz = out ? (specular ? z : (sz < 0 ? sz + g.nz : sz - g.nz)) : sz;
+    }
+    const unsigned S = (unsigned)g.S;
+    const unsigned own = (unsigned)opp(J) * S + (unsigned)site_index(g, x0, y, z);
+    if (bounce) return quad_load(f + own);
+    const unsigned plane = specular ? (unsigned)mirz(J) : (unsigned)J;
+    return pull_quad<ST, J>(f, plane * S + (unsigned)site_index(g, x0, sy, sz), own,
+                            (unsigned)g.nx, x0, (g.walls & 0x01) != 0);
+}
+
+template <int ST>
+__device__ __forceinline__ void gather_quad(const typename Store<ST>::T* __restrict__ f,
+                                            const Geo& g, int x0, int y, int z, unsigned A[Q],
+                                            unsigned B[Q]) {
+    if (y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 1) {
+        const unsigned S = (unsigned)g.S;
+        const unsigned nx = (unsigned)g.nx, nxy = (unsigned)g.nx * (unsigned)g.ny;
+        const unsigned site0 = (unsigned)z * nxy + (unsigned)y * nx + (unsigned)x0;
+        const bool wallx = (g.walls & 0x01) != 0;
+#define LBM_PQ(J)                                                                               \
+    {                                                                                           \
+        const Quad q = pull_quad<ST, J>(                                                        \
+            f, (unsigned)J * S + site0 - ((unsigned)cy(J) * nx + (unsigned)cz(J) * nxy),        \
+            (unsigned)opp(J) * S + site0, nx, x0, wallx);                                       \
+        A[J] = q.a;                                                                             \
+        B[J] = q.b;                                                                             \
+    }
+        LBM_PQ(0) LBM_PQ(1) LBM_PQ(2) LBM_PQ(3) LBM_PQ(4) LBM_PQ(5) LBM_PQ(6) LBM_PQ(7)
+        LBM_PQ(8) LBM_PQ(9) LBM_PQ(10) LBM_PQ(11) LBM_PQ(12) LBM_PQ(13) LBM_PQ(14) LBM_PQ(15)
+        LBM_PQ(16) LBM_PQ(17) LBM_PQ(18)
+#undef LBM_PQ
+    } else {
+#define LBM_PQ(J)                                                                               \
+    {                                                                                           \
+        const Quad q = pull_quad_any<ST, J>(f, g, x0, y, z);                                    \
+        A[J] = q.a;                                                                             \
+        B[J] = q.b;                                                                             \
+    }
+        LBM_PQ(0) LBM_PQ(1) LBM_PQ(2) LBM_PQ(3) LBM_PQ(4) LBM_PQ(5) LBM_PQ(6) LBM_PQ(7)
+        LBM_PQ(8) LBM_PQ(9) LBM_PQ(10) LBM_PQ(11) LBM_PQ(12) LBM_PQ(13) LBM_PQ(14) LBM_PQ(15)
+        LBM_PQ(16) LBM_PQ(17) LBM_PQ(18)
+#undef LBM_PQ
     }
 }
 

@@ -234,6 +234,7 @@ struct SmallBins {
     // Null: not kept.
     int* zperm;        // [nbz] (the set this launch writes)
     int nbz;
+    int planes;        // z-planes of a sweep block (sweep_planes)
     // The first and last z tile layer the update marks as guarded (last <
     // first: none), for the host's split of later sweeps.  Null: not kept.
     int* zrange;       // [2]
@@ -350,8 +351,9 @@ cudaError_t launch_bubble_records(const Geo& g, const BubbleDev& b, cudaStream_t
 // device, and of the interpolation launch (persistent over the covered tiles).
 int swarm_grid(int storage);
 int interp_grid(int storage);
-// Sweep z blocks (planes per CTA of the pair sweep) for nz planes.
-int sweep_z_blocks(int nz);
+// Planes per z block of the sweep that launch_collide_stream takes for these
+// buffers (even nx): a CTA's planes, within one tile layer.
+int sweep_planes(int storage, int nx, const void* fa, const void* fb);
 // Kernels launched by one launch_binning call (count, 3-pass scan, fill, sort).
 // Bubbles b with select[b] != 0 are binned; select defaults to b.spread.
 constexpr int BINNING_LAUNCHES = 6;
