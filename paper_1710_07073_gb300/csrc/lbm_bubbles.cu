@@ -89,18 +89,21 @@ __device__ __forceinline__ int f2_ceil_int(F2 a) {
 // (h < 0) it is the sum of the node samples themselves, evaluated as the
 // weights are (cell_poly of the offset from the anchor cell anc, fraction fr)
 // over the cells within n + 1 of the centre.
+__device__ __noinline__ float axis_norm_point(int anc, float fr, float inv_n, float h, int L,
+                                              bool periodic) {
+    const int K = (int)ceilf(1.0f / inv_n) + 1;
+    float sum = 0.0f;
+    for (int k = -K; k <= K; ++k) {
+        const int c = anc + k;
+        if (!periodic && (c < 0 || c >= L)) continue;
+        sum += cell_poly(((float)k + 0.5f - fr) * inv_n, h);
+    }
+    return sum;
+}
+
 __device__ __forceinline__ float axis_norm(F2 xa, int anc, float fr, float inv_n, float h, int L,
                                            bool periodic) {
-    if (h < 0.0f) {
-        const int K = (int)ceilf(1.0f / inv_n) + 1;
-        float sum = 0.0f;
-        for (int k = -K; k <= K; ++k) {
-            const int c = anc + k;
-            if (!periodic && (c < 0 || c >= L)) continue;
-            sum += cell_poly(((float)k + 0.5f - fr) * inv_n, h);
-        }
-        return sum;
-    }
+    if (h < 0.0f) return axis_norm_point(anc, fr, inv_n, h, L, periodic);
     if (periodic) return 16.0f / 15.0f;
     const float lo = (-xa.h - xa.l) * inv_n, hi = (((float)L - xa.h) - xa.l) * inv_n;
     const float a = fmaxf(lo, -1.0f), b = fminf(hi, 1.0f);
@@ -370,6 +373,13 @@ __device__ __forceinline__ void block_sum_n(float* v, float (*red)[BUBBLE_THREAD
     }
 }
 
+// A coordinate folded into [0, L) through FP64.
+__device__ __noinline__ F2 fold_fp64(F2 x, int L) {
+    double v = f2_to(x);
+    v = __dsub_rn(v, __dmul_rn((double)L, floor(v / (double)L)));
+    return f2_from(v);
+}
+
 // One thread: everything after the window sums (ax, ay, az) of bubble b.
 // An idle bubble leaves the coupling; a non-finite one is deactivated and
 // flags the instability; a live one takes the Table 1 forces and the Newton
@@ -377,9 +387,11 @@ __device__ __forceinline__ void block_sum_n(float* v, float (*red)[BUBBLE_THREAD
 // dt_b (Table 2), then its reaction psi (Algorithm 1) and spreading record.
 // acc: the window sums, acc[0..2] the Eq. 20 velocity and, with lift,
 // acc[3..8] the vorticity sums (add_window_node).
-__device__ void bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst& bc,
+// Returns whether the bubble spreads in this step (B.spread); x receives the
+// new centre then.
+__device__ bool bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst& bc,
                             int* __restrict__ flag, int b, int state, const Window& w,
-                            const float* acc, const BubbleIn& in) {
+                            const float* acc, const BubbleIn& in, F2 x[3]) {
     if (state != BUBBLE_LIVE) {
         if (state == BUBBLE_NONFINITE) {
             B.active[b] = 0;
@@ -387,7 +399,7 @@ __device__ void bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst&
         }
         B.spread[b] = 0;
         B.cell[b] = -1;
-        return;
+        return false;
     }
     const int L[3] = {g.nx, g.ny, g.nz};
     F2 xb[3] = {in.x[0], in.x[1], in.x[2]};
@@ -461,12 +473,9 @@ __device__ void bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst&
     }
     if (wrap_far) {
         // Only reachable with runaway or non-finite velocities: fold in FP64.
-        for (int a = 0; a < 3; ++a) {
-            if (g.walls & (1u << (2 * a))) continue;
-            double v = f2_to(xb[a]);
-            v = __dsub_rn(v, __dmul_rn((double)L[a], floor(v / (double)L[a])));
-            xb[a] = f2_from(v);
-        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (!(g.walls & (1u << (2 * a)))) xb[a] = fold_fp64(xb[a], L[a]);
     }
     // A bubble that moved more than GUARD_CELLS cells along an axis in one
     // step (lattice speed > 4) flags the instability.
@@ -508,7 +517,7 @@ __device__ void bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst&
         B.spread[b] = 0;
         B.cell[b] = -1;
         atomicOr(flag, 2);
-        return;
+        return false;
     }
     B.spread[b] = 1;
     int ci[3];
@@ -520,6 +529,9 @@ __device__ void bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst&
     make_record(xb, K, g, psi, B.rec[b]);
     // Algorithm 1: the bubble stops once it reaches the top of the liquid.
     if ((g.walls & 0x20) && !f2_lt(xb[2], top[2])) B.active[b] = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) x[a] = xb[a];
+    return true;
 }
 
 // Table 1 / Eq. 3 constants of a bubble of diameter d and window half-width n
@@ -598,6 +610,76 @@ __device__ int axis_tiles(int lo, int hi, int L, bool periodic, int T, int out[M
         out[k + 1] = v;
     }
     return cnt;
+}
+
+// The same tiles of one axis as two runs of consecutive ones, [first, first +
+// n0) then [second, ...), n in all, for a window that does not wrap onto
+// itself (2 n + 2 <= L on a periodic axis, as lbm_set_bubbles ensures): no
+// loops, divisions or arrays.  The update and the binning of one bubble are a
+// single thread's or warp's serial code, run once per launch, so their length
+// is paid in instruction fetches: with axis_tiles the counting of a bubble's
+// tiles took 7,900 cycles of k_swarm_tail.
+struct AxisRun {
+    int first, n0, second, n;
+    __device__ __forceinline__ int tile(int i) const {
+        return i < n0 ? first + i : second + (i - n0);
+    }
+};
+
+template <int T>
+__device__ __forceinline__ AxisRun axis_run(int lo, int hi, int L, bool periodic) {
+    static_assert((T & (T - 1)) == 0, "tiles of a power of two");
+    if (periodic) {
+        if (lo < 0) lo += L;
+        if (hi >= L) hi -= L;
+    } else {
+        lo = max(lo, 0);
+        hi = min(hi, L - 1);
+        if (hi < lo) return AxisRun{0, 0, 0, 0};
+    }
+    const int ts = lo / T, te = hi / T;   // lo, hi >= 0
+    if (lo <= hi) return AxisRun{ts, te - ts + 1, 0, te - ts + 1};
+    // The window wraps: the tiles up to te, then those from ts (all of them
+    // when both ends lie in one tile).
+    const int nt = (L + T - 1) / T;
+    if (te >= ts) return AxisRun{0, nt, 0, nt};
+    return AxisRun{0, te + 1, ts, te + 1 + nt - ts};
+}
+
+// The tiles of a bubble's window (widened by pad), numbered x fastest.
+struct TileRuns {
+    AxisRun x, y, z;
+    int n;
+    __device__ __forceinline__ int tile(const Geo& g, int ix, int iy, int iz) const {
+        return (z.tile(iz) * g.nty + y.tile(iy)) * g.ntx + x.tile(ix);
+    }
+    // The k-th tile in ascending order.
+    __device__ __forceinline__ int tile(const Geo& g, int k) const {
+        const int r = k / x.n;
+        return tile(g, k - r * x.n, r % y.n, r / y.n);
+    }
+};
+
+__device__ __forceinline__ TileRuns tile_runs(const Geo& g, const F2 c[3], float nh, float nl,
+                                              int pad) {
+    TileRuns r;
+    int lo, hi;
+    support_cells(c[0], nh, nl, lo, hi);
+    r.x = axis_run<TX>(lo - pad, hi + pad, g.nx, !(g.walls & 0x01));
+    support_cells(c[1], nh, nl, lo, hi);
+    r.y = axis_run<TY>(lo - pad, hi + pad, g.ny, !(g.walls & 0x04));
+    support_cells(c[2], nh, nl, lo, hi);
+    r.z = axis_run<TZ>(lo - pad, hi + pad, g.nz, !(g.walls & 0x10));
+    r.n = r.x.n * r.y.n * r.z.n;
+    return r;
+}
+
+__device__ __forceinline__ TileRuns tile_runs(const Geo& g, const BubbleDev& B, int b, int pad) {
+    const float nh = __ldcg(&B.k[b].nh), nl = __ldcg(&B.k[b].nl);
+    F2 c[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) c[a] = F2{__ldcg(B.xh + 3 * b + a), __ldcg(B.xl + 3 * b + a)};
+    return tile_runs(g, c, nh, nl, pad);
 }
 
 template <bool FILL>
@@ -788,32 +870,23 @@ __device__ void bin_small_block(const Geo& g, const BubbleDev& B, const SmallBin
     const int tid = threadIdx.x, nt = blockDim.x;
     if (tid == 0) *s_n = 0;
     __syncthreads();
-    const int T[3] = {TX, TY, TZ};
-    for (int b = tid; b < B.nb; b += nt) {
+    // A warp per bubble, a lane per tile.
+    const int lane = tid & 31;
+    for (int b = tid >> 5; b < B.nb; b += nt >> 5) {
         if (!__ldcg(B.spread + b)) continue;
         const Geo& gb = cols ? cols[bubble_col[b]].g : g;
         const int base = cols ? cols[bubble_col[b]].tile_base : 0;
-        const int L[3] = {gb.nx, gb.ny, gb.nz};
-        int tl[3][MAX_AXIS_TILES];
-        int ntl[3];
-        const float nh = __ldcg(&B.k[b].nh), nl = __ldcg(&B.k[b].nl);
-        for (int a = 0; a < 3; ++a) {
-            int lo, hi;
-            support_cells(F2{__ldcg(B.xh + 3 * b + a), __ldcg(B.xl + 3 * b + a)}, nh, nl, lo, hi);
-            ntl[a] = axis_tiles(lo - pad, hi + pad, L[a], !(gb.walls & (1u << (2 * a))), T[a],
-                                tl[a]);
-        }
+        const TileRuns r = tile_runs(gb, B, b, pad);
         // One reservation per bubble; its pairs come out in ascending tile
-        // order (each axis list is ascending).
-        int k = atomicAdd(s_n, ntl[0] * ntl[1] * ntl[2]);
-        for (int iz = 0; iz < ntl[2]; ++iz)
-            for (int iy = 0; iy < ntl[1]; ++iy)
-                for (int ix = 0; ix < ntl[0]; ++ix, ++k) {
-                    const unsigned t = (unsigned)(base + (tl[2][iz] * gb.nty + tl[1][iy]) * gb.ntx +
-                                                  tl[0][ix]);
-                    if (k < SMALL_MAX_PAIRS) keys[k] = ((unsigned long long)t << 32) | (unsigned)b;
-                    else atomicOr(sb.overflow, 1);
-                }
+        // order.
+        int k0 = 0;
+        if (lane == 0) k0 = atomicAdd(s_n, r.n);
+        k0 = __shfl_sync(0xffffffffu, k0, 0);
+        for (int k = lane; k < r.n; k += 32) {
+            const unsigned t = (unsigned)(base + r.tile(gb, k));
+            if (k0 + k < SMALL_MAX_PAIRS) keys[k0 + k] = ((unsigned long long)t << 32) | (unsigned)b;
+            else atomicOr(sb.overflow, 1);
+        }
     }
     __syncthreads();
     const int n = min(*s_n, SMALL_MAX_PAIRS);
@@ -1048,7 +1121,8 @@ k_bubbles_binned(const typename Store<ST>::T* __restrict__ f, Geo g, CollidePara
         }
         s_last = 0;
         if (mine) {
-            bubble_tail(g, B, bc, flag, b, state, w, sum, in);
+            F2 x_new[3];
+            bubble_tail(g, B, bc, flag, b, state, w, sum, in, x_new);
             if (alone) {
                 s_last = 1;
             } else {
@@ -1141,7 +1215,8 @@ cudaError_t launch_bubbles_batch(int storage, const void* f, const BatchColumn* 
 constexpr int INTERP_THREADS = TX * TY * 2;   // two of a tile's TZ planes per thread
 constexpr int INTERP_CHUNK = 32;              // listed bubbles per pass
 constexpr int INTERP_ROWS = TY * TZ;          // (y, z) rows of a tile: 16
-static_assert(INTERP_THREADS % INTERP_ROWS == 0 && TZ == 4, "tile shape of the interpolation");
+static_assert(INTERP_THREADS % INTERP_ROWS == 0 && TX == 32 && TY == 4 && TZ == 4,
+              "tile shape of the interpolation: a lane per column");
 // Resident CTAs per SM the interpolation is compiled for: 16-bit storage on
 // even rows at 5 (48 registers; its swarm step ran 1 % shorter than at 4, at
 // 6 longer); FP32 at 4 (at 5 it spills 96 bytes and its step was longer), as
@@ -1237,42 +1312,47 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
                 if (id >= 0 && id < nb) s_rec[tid] = load_rec(recs + id);
                 else s_rec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             }
-            s_xlo[tid] = TX;
-            s_xhi[tid] = -1;
         }
         __syncthreads();
-        // The mapping mode is the same for every bubble: one loop per mode.
+        // A warp per bubble tabulates its x weights, a lane per column, so
+        // that a ballot gives the range of non-zero ones; then 8 threads per
+        // bubble its y and z weights.  The mapping mode is the same for every
+        // bubble: one loop per mode.
         auto tabulate = [&](auto mode) {
             constexpr int PM = decltype(mode)::value;
-            for (int e = tid; e < cntc * NAX; e += INTERP_THREADS) {
-                const int k = e / NAX, q = e - k * NAX;
+            for (int k = tid / TX; k < cntc; k += INTERP_THREADS / TX) {
+                const int q = tid % TX;
                 const BubbleRec& r = s_rec[k];
+                float w, dw = 0.0f;
+                if (LIFT) {
+                    axis_wd<PM>(xb0 + q, r.ax, r.fx, r.inv_n, r.h, g.nx, px, false, w, dw);
+                    s_d[k][q] = dw;
+                } else {
+                    w = axis_weight<PM>(r, xb0 + q, r.ax, r.fx, g.nx, px);
+                }
+                s_w[k][q] = w;
+                const unsigned m = __ballot_sync(0xffffffffu, w != 0.0f || dw != 0.0f);
+                if (q == 0) {
+                    s_xlo[k] = m ? __ffs(m) - 1 : TX;
+                    s_xhi[k] = m ? 31 - __clz(m) : -1;
+                }
+            }
+            for (int e = tid; e < cntc * (TY + TZ); e += INTERP_THREADS) {
+                const int k = e / (TY + TZ), q = e % (TY + TZ);
+                const BubbleRec& r = s_rec[k];
+                const bool isy = q < TY;
+                const int c = isy ? yb0 + q : zb0 + q - TY;
+                const int anc = isy ? r.ay : r.az, L = isy ? g.ny : g.nz;
+                const float fr = isy ? r.fy : r.fz;
+                const bool periodic = isy ? py : pz;
                 if (LIFT) {
                     float w, dw;
-                    if (q < TX)
-                        axis_wd<PM>(xb0 + q, r.ax, r.fx, r.inv_n, r.h, g.nx, px, false, w, dw);
-                    else if (q < TX + TY)
-                        axis_wd<PM>(yb0 + q - TX, r.ay, r.fy, r.inv_n, r.h, g.ny, py, false, w, dw);
-                    else
-                        axis_wd<PM>(zb0 + q - TX - TY, r.az, r.fz, r.inv_n, r.h, g.nz, pz,
-                                    (g.walls & WALL_TOP_FREE) != 0, w, dw);
-                    s_w[k][q] = w;
-                    s_d[k][q] = dw;
-                    if (q < TX && (w != 0.0f || dw != 0.0f)) {
-                        atomicMin(&s_xlo[k], q);
-                        atomicMax(&s_xhi[k], q);
-                    }
-                } else if (q < TX) {
-                    const float w = axis_weight<PM>(r, xb0 + q, r.ax, r.fx, g.nx, px);
-                    s_w[k][q] = w;
-                    if (w != 0.0f) {
-                        atomicMin(&s_xlo[k], q);
-                        atomicMax(&s_xhi[k], q);
-                    }
-                } else if (q < TX + TY) {
-                    s_w[k][q] = axis_weight<PM>(r, yb0 + q - TX, r.ay, r.fy, g.ny, py);
+                    axis_wd<PM>(c, anc, fr, r.inv_n, r.h, L, periodic,
+                                !isy && (g.walls & WALL_TOP_FREE) != 0, w, dw);
+                    s_w[k][TX + q] = w;
+                    s_d[k][TX + q] = dw;
                 } else {
-                    s_w[k][q] = axis_weight<PM>(r, zb0 + q - TX - TY, r.az, r.fz, g.nz, pz);
+                    s_w[k][TX + q] = axis_weight<PM>(r, c, anc, fr, L, periodic);
                 }
             }
         };
@@ -1286,9 +1366,9 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
         for (int k0 = 0; k0 < cntc; k0 += INTERP_THREADS / INTERP_ROWS) {
             const int k = k0 + tid / INTERP_ROWS, row = tid % INTERP_ROWS;
             constexpr int NV = win_vals(LIFT);
-            float v[NV];
+            float v[WIN_VALS_LIFT];
 #pragma unroll
-            for (int q = 0; q < NV; ++q) v[q] = 0.0f;
+            for (int q = 0; q < WIN_VALS_LIFT; ++q) v[q] = 0.0f;
             if (k < cntc) {
                 const float wy = s_w[k][TX + row % TY], wz = s_w[k][TX + TY + row / TY];
                 const float dy = LIFT ? s_d[k][TX + row % TY] : 0.0f;
@@ -1331,9 +1411,13 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
                 for (int o = INTERP_ROWS / 2; o > 0; o >>= 1)
                     v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
             if (row == 0 && k < cntc) {
-                float* q = partial + WIN_VALS_LIFT * (size_t)(c0 + k);
-#pragma unroll
-                for (int i = 0; i < NV; ++i) q[i] = v[i];
+                float4* q = reinterpret_cast<float4*>(partial) +
+                            partial_stride(LIFT) / 4 * (size_t)(c0 + k);
+                q[0] = make_float4(v[0], v[1], v[2], LIFT ? v[3] : 0.0f);
+                if (LIFT) {
+                    q[1] = make_float4(v[4], v[5], v[6], v[7]);
+                    q[2] = make_float4(v[8], 0.0f, 0.0f, 0.0f);
+                }
             }
         }
     }
@@ -1346,11 +1430,23 @@ k_tile_interp(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams 
               const int* __restrict__ cnt, const int* __restrict__ off,
               const int* __restrict__ items, int cap, const BubbleRec* __restrict__ recs, int nb,
               const int* __restrict__ cover, const int* __restrict__ ncover,
-              float* __restrict__ partial) {
+              float* __restrict__ partial, int* __restrict__ cnt_next, int T,
+              int* __restrict__ zrange) {
     const int ntiles = __ldcg(ncover);
     const int step = (int)gridDim.x;
+    // The tile counts and the z range that the update after this launch adds to.
+    for (int t = (int)blockIdx.x * INTERP_THREADS + (int)threadIdx.x; t < T;
+         t += step * INTERP_THREADS)
+        cnt_next[t] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && zrange) {
+        zrange[0] = INT_MAX;
+        zrange[1] = -1;
+    }
     int i = (int)blockIdx.x;
-    if (i >= ntiles) return;
+    if (i >= ntiles) {
+        pdl_trigger();
+        return;
+    }
     // The head of the CTA's first tile, and the index of the one after it.
     auto head = [&](int t) {
         TileHead h{t, 0, 0, -1};
@@ -1368,6 +1464,7 @@ k_tile_interp(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams 
         // during this tile; the index of the tile after it.
         TileHead next = head(tn);
         const int tnn = i + 2 * step < ntiles ? __ldcg(cover + i + 2 * step) : -1;
+        if (i + step >= ntiles) pdl_trigger();   // this CTA's last tile
         __syncthreads();   // the shared tables of the previous tile are done with
         tile_interp<ST, PAIR, LIFT>(f, g, cp, h, next, items, recs, nb, partial);
         h = next;
@@ -1375,60 +1472,126 @@ k_tile_interp(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams 
     }
 }
 
-// The update, a thread per bubble: its Eq. 20 sum is the parts of its tiles
-// added in tile order.  The tile counts and the list of covered tiles start
-// again for the binning after it.
-constexpr int TAIL_THREADS = 128;
+// A bubble added to the counts of the tiles r its window touches (Algorithm 1
+// step 2); zlo and zhi receive their z tile layers.
+__device__ __forceinline__ void count_tiles(const Geo& g, const TileRuns& r, int* __restrict__ cnt,
+                                            int& zlo, int& zhi) {
+    if (r.n > 0) {
+        zlo = min(zlo, r.z.first);
+        zhi = max(zhi, r.z.tile(r.z.n - 1));
+    }
+#pragma unroll 1
+    for (int iz = 0; iz < r.z.n; ++iz)
+#pragma unroll 1
+        for (int iy = 0; iy < r.y.n; ++iy) {
+            int* const row = cnt + r.tile(g, 0, iy, iz) - r.x.first;
+#pragma unroll 1
+            for (int ix = 0; ix < r.x.n; ++ix) atomicAdd(row + r.x.tile(ix), 1);
+        }
+}
 
+// The z range of the lists, from a warp's bubbles (every lane calls it).
+__device__ __forceinline__ void merge_zrange(int zlo, int zhi, int* zrange) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        zlo = min(zlo, __shfl_xor_sync(0xffffffffu, zlo, o));
+        zhi = max(zhi, __shfl_xor_sync(0xffffffffu, zhi, o));
+    }
+    if ((threadIdx.x & 31) == 0 && zhi >= 0) {
+        atomicMin(zrange, zlo);
+        atomicMax(zrange + 1, zhi);
+    }
+}
+
+// The update, a thread per bubble: its Eq. 20 sum is the parts of its tiles
+// added in tile order; then the updated bubble adds itself to the tile counts
+// of the binning after it (bins.cnt, zeroed by the interpolation).
+//
+// Bound by latency: a chain of dependent loads, the sub-steps of one thread,
+// and too few bubbles to fill the GPU.  So the list positions of TAIL_SLOTS
+// tiles are loaded together with the state and then their parts together (one
+// after the other they cost two L2 round trips per tile, each 2 us beside a
+// sweep), and a CTA is one warp.  With the binning below (fewer CTAs, one-hop
+// barriers, lists ordered over the covered tiles only, code without loops
+// where a thread runs it once) and the two launched ahead, the step of 463
+// bubbles in 64x64x128 went from 0.089 to 0.052 ms, of 3,704 bubbles with lift
+// in 128x128x256 from 0.206 to 0.165 ms, of 100,000 bubbles in 384x384x768
+// from 3.057 to 3.034 ms (FP32) and 1.953 to 1.942 ms (FP16).
+constexpr int TAIL_THREADS = 32;
+constexpr int TAIL_SLOTS = 12;
+
+template <bool LIFT>
 __global__ void __launch_bounds__(TAIL_THREADS)
 k_swarm_tail(Geo g, BubbleDev B, BubbleConst bc, int* __restrict__ flag, Bins bins,
              SwarmBins sw) {
-    const int tid = threadIdx.x;
-    const int gtid = blockIdx.x * TAIL_THREADS + tid, nthreads = gridDim.x * TAIL_THREADS;
-    for (int t = gtid; t < bins.T; t += nthreads) bins.cnt[t] = 0;
-    if (gtid == 0) {
-        *sw.ncover = 0;
-        if (sw.zrange) {
-            sw.zrange[0] = INT_MAX;
-            sw.zrange[1] = -1;
-        }
-    }
-    const int b = gtid;
+    constexpr int NV = win_vals(LIFT), NS = TAIL_SLOTS, NP = partial_stride(LIFT) / 4;
+    pdl_wait();
+    const int b = blockIdx.x * TAIL_THREADS + threadIdx.x;
+    if (b == 0) *sw.ncover = 0;
+    int zlo = INT_MAX, zhi = -1;
     if (b < B.nb) {
+        const int n = min(__ldcg(sw.ntile + b), sw.per);
+        const int* sl = sw.slots + (size_t)b * sw.per;
         BubbleIn in;
         load_bubble(B, b, true, in);
+        float acc[WIN_VALS_LIFT];
+#pragma unroll
+        for (int q = 0; q < WIN_VALS_LIFT; ++q) acc[q] = 0.0f;
+        for (int k0 = 0; k0 == 0 || k0 < n; k0 += NS) {
+            int p[NS];
+            float v[NS][4 * NP];
+#pragma unroll
+            for (int i = 0; i < NS; ++i) p[i] = k0 + i < sw.per ? __ldcg(sl + k0 + i) : -1;
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+                if (k0 + i >= n || p[i] >= bins.cap) p[i] = -1;
+                const float4* q = reinterpret_cast<const float4*>(sw.partial) +
+                                  NP * (size_t)max(p[i], 0);
+#pragma unroll
+                for (int c = 0; c < NP; ++c) {
+                    const float4 u = p[i] >= 0 ? __ldcg(q + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[i][4 * c] = u.x;
+                    v[i][4 * c + 1] = u.y;
+                    v[i][4 * c + 2] = u.z;
+                    v[i][4 * c + 3] = u.w;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NS; ++i)
+                if (p[i] >= 0)
+#pragma unroll
+                    for (int c = 0; c < NV; ++c) acc[c] += v[i][c];
+        }
         Window w;
         const int state = bubble_window(g, in, w);
-        const int nv = win_vals(bc.lift != 0);
-        float acc[WIN_VALS_LIFT];
-        for (int q = 0; q < WIN_VALS_LIFT; ++q) acc[q] = 0.0f;
-        if (state == BUBBLE_LIVE) {
-            const int n = min(__ldcg(sw.ntile + b), sw.per);
-            const int* sl = sw.slots + (size_t)b * sw.per;
-            for (int k = 0; k < n; ++k) {
-                const int p = __ldcg(sl + k);
-                if (p < 0 || p >= bins.cap) continue;
-                const float* q = sw.partial + WIN_VALS_LIFT * (size_t)p;
-                for (int v = 0; v < nv; ++v) acc[v] += __ldcg(q + v);
-            }
+        F2 x[3];
+        int nt = 0;
+        if (bubble_tail(g, B, bc, flag, b, state, w, acc, in, x)) {
+            const TileRuns r = tile_runs(g, x, in.k.nh, in.k.nl, sw.pad);
+            count_tiles(g, r, bins.cnt, zlo, zhi);
+            nt = r.n;
         }
-        bubble_tail(g, B, bc, flag, b, state, w, acc, in);
+        sw.ntile[b] = nt;
     }
+    __syncwarp();
+    pdl_trigger();
+    if (sw.zrange) merge_zrange(zlo, zhi, sw.zrange);
 }
 
 // Binning of the updated bubbles in one persistent launch, phases separated
 // by grid barriers (all its CTAs are resident):
-//   1. count: every selected bubble adds itself to the tiles its window
-//      touches (Algorithm 1 step 2);
+//   1. with `select`, the counts (else the update has made them);
 //   2. scan of the counts (per-CTA chunk totals, then offsets), and the list
 //      of covered tiles;
 //   3. fill: each bubble takes slots through per-tile cursors, noting which
 //      of its tiles each is;
-//   4. each tile's list ordered by bubble id (a warp per tile: an id's rank
-//      is the number of smaller ids in the list), and the list positions
-//      recorded per bubble.
+//   4. each covered tile's list ordered by bubble id (a warp per tile: an
+//      id's rank is the number of smaller ids in the list), and the list
+//      positions recorded per bubble.
 // The counts, offsets and lists are those of launch_binning.  Everything
-// written earlier in the launch is read through L2 (ld.global.cg).
+// written earlier in the launch, or by the update, is read through L2
+// (ld.global.cg).  Bound by the latency of its phases and barriers, so the
+// grid is no larger than the work needs (swarm_bin_grid).
 constexpr int SWARM_THREADS = 256;
 constexpr int SWARM_WARPS = SWARM_THREADS / 32;
 constexpr int SWARM_SORT_MAX = 128;   // longer tile lists are ordered by one thread
@@ -1442,38 +1605,44 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Grid barrier over the launch's CTAs (bar[0] arrivals, bar[1] generation).
-// The last CTA to arrive resets the arrivals before it advances the
-// generation, so the counter is zero again for the next barrier and launch.
-// Returns false (in every thread of the CTA) if the wait ran out.
-__device__ bool grid_barrier(unsigned* bar, int* flag) {
+// The `round`-th grid barrier of a launch (1, 2, ...) over its CTAs: arrivals
+// are counted up over the launch in bar[0], so an arrival is one release
+// reduction and the wait one load to see the last of them (a generation that
+// the last CTA advances costs two more round trips).  Returns false (in every
+// thread of the CTA) if the wait ran out.
+__device__ bool grid_barrier(unsigned* bar, unsigned round, int* flag) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        volatile unsigned* vbar = bar;
-        const unsigned gen = vbar[1];
-        __threadfence();
-        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            const unsigned long long t0 = global_ns();
-            while (vbar[1] == gen) {
-                __nanosleep(64);
-                if (global_ns() - t0 > SWARM_WAIT_NS) {
-                    atomicOr(flag, 8);
-                    ok = 0;
-                    break;
-                }
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        // The timer is read on every 32nd poll only: a read costs as much as
+        // a poll.
+        const unsigned target = round * gridDim.x;
+        const unsigned long long t0 = global_ns();
+        for (unsigned n = 1;; ++n) {
+            unsigned seen;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+            if (seen >= target) break;
+            if ((n & 31u) == 0u && global_ns() - t0 > SWARM_WAIT_NS) {
+                atomicOr(flag, 8);
+                ok = 0;
+                break;
             }
         }
-        __threadfence();
         s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
+}
+
+// After a launch's last barrier: the last CTA to leave zeroes the counters for
+// the next launch.
+__device__ void grid_barrier_leave(unsigned* bar) {
+    if (threadIdx.x == 0 && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+        bar[0] = 0u;
+        bar[1] = 0u;
+    }
 }
 
 // Sum over the CTA (fixed order), returned in every thread.
@@ -1489,23 +1658,6 @@ __device__ __forceinline__ int block_sum_int(int v, int* red) {
     return t;
 }
 
-// The tiles bubble b's window touches, per axis (ascending), as k_bin finds
-// them; returns false for a bubble that is not selected.
-__device__ __forceinline__ bool bubble_tiles(const Geo& g, const BubbleDev& B, const int* select,
-                                             int pad, int b, int tl[3][MAX_AXIS_TILES],
-                                             int nt[3]) {
-    if (!__ldcg(select + b)) return false;
-    const int L[3] = {g.nx, g.ny, g.nz};
-    const int T[3] = {TX, TY, TZ};
-    const float nh = B.k[b].nh, nl = B.k[b].nl;
-    for (int a = 0; a < 3; ++a) {
-        int lo, hi;
-        support_cells(F2{__ldcg(B.xh + 3 * b + a), __ldcg(B.xl + 3 * b + a)}, nh, nl, lo, hi);
-        nt[a] = axis_tiles(lo - pad, hi + pad, L[a], !(g.walls & (1u << (2 * a))), T[a], tl[a]);
-    }
-    return true;
-}
-
 __global__ void __launch_bounds__(SWARM_THREADS)
 k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__ select,
             int* __restrict__ flag) {
@@ -1517,36 +1669,28 @@ k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__
     const int gtid = blockIdx.x * SWARM_THREADS + tid;
     const int T = bins.T;
 
+    pdl_wait();
+    // A wait that ran out in an earlier launch left the counters part-way:
+    // nothing more is binned until the host has reset them.
+    if (__ldcg(flag) & 8) return;
+    unsigned round = 0;
     // 1. Count; and the z tile layers the lists reach (for the next steps'
     // split of the sweep).
-    int zlo = INT_MAX, zhi = -1;
-    for (int b = gtid; b < B.nb; b += nthreads) {
-        int tl[3][MAX_AXIS_TILES], nt[3];
-        int n = 0;
-        if (bubble_tiles(g, B, select, sw.pad, b, tl, nt)) {
-            for (int iz = 0; iz < nt[2]; ++iz) {
-                zlo = min(zlo, tl[2][iz]);
-                zhi = max(zhi, tl[2][iz]);
-                for (int iy = 0; iy < nt[1]; ++iy)
-                    for (int ix = 0; ix < nt[0]; ++ix)
-                        atomicAdd(&bins.cnt[(tl[2][iz] * g.nty + tl[1][iy]) * g.ntx + tl[0][ix]], 1);
+    if (select != nullptr) {
+        int zlo = INT_MAX, zhi = -1;
+        for (int b = gtid; b < B.nb; b += nthreads) {
+            int n = 0;
+            if (__ldcg(select + b)) {
+                const TileRuns r = tile_runs(g, B, b, sw.pad);
+                count_tiles(g, r, bins.cnt, zlo, zhi);
+                n = r.n;
             }
-            n = nt[0] * nt[1] * nt[2];
+            sw.ntile[b] = n;
         }
-        sw.ntile[b] = n;
+        __syncwarp();
+        if (sw.zrange) merge_zrange(zlo, zhi, sw.zrange);
+        if (!grid_barrier(sw.bar, ++round, flag)) return;
     }
-    if (sw.zrange) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            zlo = min(zlo, __shfl_xor_sync(0xffffffffu, zlo, o));
-            zhi = max(zhi, __shfl_xor_sync(0xffffffffu, zhi, o));
-        }
-        if (lane == 0 && zhi >= 0) {
-            atomicMin(sw.zrange, zlo);
-            atomicMax(sw.zrange + 1, zhi);
-        }
-    }
-    if (!grid_barrier(sw.bar, flag)) return;
 
     // 2. Scan, chunk totals.
     const int chunk = (T + gridDim.x - 1) / gridDim.x;
@@ -1555,7 +1699,7 @@ k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__
     for (int t = c0 + tid; t < c1; t += SWARM_THREADS) part += __ldcg(bins.cnt + t);
     part = block_sum_int(part, s_red);
     if (tid == 0) sw.chunk_sums[blockIdx.x] = part;
-    if (!grid_barrier(sw.bar, flag)) return;
+    if (!grid_barrier(sw.bar, ++round, flag)) return;
 
     // Scan, offsets (and the fill cursors).
     int prefix = 0;
@@ -1585,36 +1729,38 @@ k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__
         }
         if (c1 == T && c0 < c1 && tid == 0) bins.off[T] = carry;
     }
-    if (!grid_barrier(sw.bar, flag)) return;
+    if (!grid_barrier(sw.bar, ++round, flag)) return;
 
-    // 3. Fill.
-    for (int b = gtid; b < B.nb; b += nthreads) {
-        int tl[3][MAX_AXIS_TILES], nt[3];
-        if (!bubble_tiles(g, B, select, sw.pad, b, tl, nt)) continue;
-        int k = 0;
-        for (int iz = 0; iz < nt[2]; ++iz)
-            for (int iy = 0; iy < nt[1]; ++iy)
-                for (int ix = 0; ix < nt[0]; ++ix, ++k) {
-                    const int t = (tl[2][iz] * g.nty + tl[1][iy]) * g.ntx + tl[0][ix];
-                    const int at = atomicAdd(&sw.cursor[t], 1);
-                    if (at < bins.cap) {
-                        bins.items[at] = b;
-                        sw.kidx[at] = k;
-                    } else {
-                        atomicOr(bins.overflow, 1);
-                    }
-                }
+    // 3. Fill: FILL_LANES lanes per bubble, a tile each, so that the cursors'
+    // round trips overlap.
+    constexpr int FILL_LANES = 8;
+    if (select == nullptr) select = B.spread;
+    for (int i = gtid; i < B.nb * FILL_LANES; i += nthreads) {
+        const int b = i / FILL_LANES;
+        if (!__ldcg(select + b)) continue;
+        const TileRuns r = tile_runs(g, B, b, sw.pad);
+        for (int k = i % FILL_LANES; k < r.n; k += FILL_LANES) {
+            const int at = atomicAdd(&sw.cursor[r.tile(g, k)], 1);
+            if (at < bins.cap) {
+                bins.items[at] = b;
+                sw.kidx[at] = k;
+            } else {
+                atomicOr(bins.overflow, 1);
+            }
+        }
     }
-    if (!grid_barrier(sw.bar, flag)) return;
+    if (!grid_barrier(sw.bar, ++round, flag)) return;
+    grid_barrier_leave(sw.bar);
 
     // 4. Each tile's list in bubble order, and each bubble's list positions.
     // A bubble is listed at most once per tile, so the ids of a list are
     // distinct and their ranks are the positions.
     int* ids = s_id[warp];
     int* ks = s_k[warp];
-    for (int t = blockIdx.x * SWARM_WARPS + warp; t < T; t += gridDim.x * SWARM_WARPS) {
+    const int ncover = __ldcg(sw.ncover);
+    for (int i0 = blockIdx.x * SWARM_WARPS + warp; i0 < ncover; i0 += gridDim.x * SWARM_WARPS) {
+        const int t = __ldcg(sw.cover + i0);
         const int n = __ldcg(bins.cnt + t);
-        if (n == 0) continue;   // uniform over the warp
         const int beg = __ldcg(bins.off + t);
         const int end = min(beg + n, bins.cap);
         const int m = end - beg;
@@ -1671,15 +1817,27 @@ cudaError_t launch_bubble_records(const Geo& g, const BubbleDev& b, cudaStream_t
     return cudaGetLastError();
 }
 
-int swarm_grid(int /*storage*/) {
+int swarm_grid(int* sms_out) {
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_swarm_bin, SWARM_THREADS, 0) !=
             cudaSuccess || per < 1)
         return 0;
+    *sms_out = sms;
     return sms * std::min(per, LBM_SWARM_CTAS_PER_SM);
 }
+
+namespace {
+// CTAs of the binning: 64 bubbles and 2,048 tiles to scan per CTA, at
+// least one CTA per SM (the lists are ordered a warp per covered tile), at most
+// what is resident.  Fewer CTAs make each grid barrier shorter.
+int swarm_bin_grid(const SwarmBins& sw, int nb, int T) {
+    const int need = std::max(sw.sms, std::max((nb + SWARM_THREADS / 4 - 1) / (SWARM_THREADS / 4),
+                                               (T + 2047) / 2048));
+    return std::min(sw.grid, need);
+}
+}  // namespace
 
 int interp_grid(int storage) {
     int dev = 0, sms = 0, per = 0;
@@ -1703,7 +1861,7 @@ cudaError_t launch_interp_as(const void* f, const Geo& g, const CollideParams& c
     using T = typename Store<ST>::T;
     k_tile_interp<ST, PAIR, LIFT><<<sw.interp_grid, INTERP_THREADS, 0, st>>>(
         (const T*)f, g, cp, bins.cnt, bins.off, bins.items, bins.cap, b.rec, b.nb, sw.cover,
-        sw.ncover, sw.partial);
+        sw.ncover, sw.partial, sw.cnt_next, bins.T, sw.zrange);
     return cudaGetLastError();
 }
 
@@ -1721,7 +1879,8 @@ cudaError_t launch_interp(const void* f, const Geo& g, const CollideParams& cp, 
 
 bool swarm_ready(const SwarmBins& sw) {
     return sw.grid >= 1 && sw.interp_grid >= 1 && sw.bar && sw.cursor && sw.kidx && sw.slots &&
-           sw.ntile && sw.per >= 1 && sw.partial && sw.cover && sw.ncover && sw.chunk_sums;
+           sw.ntile && sw.per >= 1 && sw.partial && sw.cover && sw.ncover && sw.chunk_sums &&
+           sw.cnt_next;
 }
 }  // namespace
 
@@ -1738,18 +1897,34 @@ cudaError_t launch_swarm_update(int storage, const void* f, const Geo& g,
         default: e = launch_interp<2>(f, g, cp, bins, b, sw, bc.lift != 0, st); break;
     }
     if (e != cudaSuccess) return e;
-    k_swarm_tail<<<(b.nb + TAIL_THREADS - 1) / TAIL_THREADS, TAIL_THREADS, 0, st>>>(g, b, bc, flag,
-                                                                                   bins, sw);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_swarm_binning(g, b, bins, sw, b.spread, flag, st);
+    // The update and the binning are launched while the launch before drains
+    // (each waits for it before it reads anything).
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((b.nb + TAIL_THREADS - 1) / TAIL_THREADS);
+    cfg.blockDim = dim3(TAIL_THREADS);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    Bins next = bins;
+    next.cnt = sw.cnt_next;
+    e = bc.lift ? cudaLaunchKernelEx(&cfg, k_swarm_tail<true>, g, b, bc, flag, next, sw)
+                : cudaLaunchKernelEx(&cfg, k_swarm_tail<false>, g, b, bc, flag, next, sw);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3(swarm_bin_grid(sw, b.nb, bins.T));
+    cfg.blockDim = dim3(SWARM_THREADS);
+    return cudaLaunchKernelEx(&cfg, k_swarm_bin, g, b, next, sw, (const int*)nullptr, flag);
 }
 
 cudaError_t launch_swarm_binning(const Geo& g, const BubbleDev& b, const Bins& bins,
                                  const SwarmBins& sw, const int* select, int* flag,
                                  cudaStream_t st) {
     if (b.nb == 0) return cudaSuccess;
-    if (!swarm_ready(sw)) return cudaErrorInvalidValue;
-    k_swarm_bin<<<sw.grid, SWARM_THREADS, 0, st>>>(g, b, bins, sw, select, flag);
+    if (!swarm_ready(sw) || !select) return cudaErrorInvalidValue;
+    k_swarm_bin<<<swarm_bin_grid(sw, b.nb, bins.T), SWARM_THREADS, 0, st>>>(g, b, bins, sw, select,
+                                                                          flag);
     return cudaGetLastError();
 }
 

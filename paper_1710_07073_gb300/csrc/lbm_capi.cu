@@ -175,7 +175,7 @@ void free_bubbles(lbm_ctx* c) {
                     b.active, b.spread, b.cell, b.rec, c->bins.items, sb.start, sb.count, sb.items,
                     sb.prev_tiles, sb.prev_n, sb.overflow, sb.done, sb.part, sb.arrive, sb.safe,
                     sb.zperm, sb.zrange, sw.bar, sw.cursor, sw.kidx, sw.slots, sw.ntile, sw.partial, sw.cover,
-                    sw.ncover, sw.chunk_sums, sw.zrange};
+                    sw.ncover, sw.chunk_sums, sw.zrange, sw.cnt_next};
     for (void* p : ptrs) dfree(c, p);
     c->cover_valid = false;
     b = BubbleDev{};
@@ -221,8 +221,14 @@ int alloc_guard(lbm_ctx* c, unsigned** safe, int** zperm, int* nbz, int** zrange
 // Interpolation CTAs per SM while the sweep of the blocks no bubble reaches
 // runs beside it (GB300, swarm 384x384x768: 2 gives the shortest step; 4,
 // the interpolation's own occupancy, leaves the sweep no room; 1 starves it).
+// Only where that sweep is the longer of the two: in smaller lattices the
+// bubble side is the step's critical path and keeps the whole grid (GB300,
+// 128x128x256 with 3,704 bubbles and lift: 0.153 ms a step against 0.165 at 2).
 #ifndef LBM_SPLIT_INTERP_PER_SM
 #define LBM_SPLIT_INTERP_PER_SM 2
+#endif
+#ifndef LBM_SPLIT_SHARE_MIN_SITES
+#define LBM_SPLIT_SHARE_MIN_SITES (1LL << 24)
 #endif
 
 // Few bubbles: the split pays only where the sweep is long against the
@@ -394,11 +400,12 @@ int enqueue_one_step(lbm_ctx* c) {
             sw.pad = pad;
             // Split: the persistent interpolation leaves room on every SM for
             // the sweep of the blocks bubbles do not reach.
-            if (split && c->sms > 0)
+            if (split && c->sms > 0 && g.S >= LBM_SPLIT_SHARE_MIN_SITES)
                 sw.interp_grid = std::min(sw.interp_grid, c->sms * LBM_SPLIT_INTERP_PER_SM);
             LBM_CUDA(launch_swarm_update(c->storage, c->f[c->cur], g, cp, c->bub, bubble_const(c),
                                          c->flag_d, c->bins, sw, st),
                      "bubble update");
+            std::swap(c->bins.cnt, c->swarm.cnt_next);   // the counts just made
             c->launches += SWARM_LAUNCHES;   // interpolation by tiles; update; binning
             c->cover_valid = true;
         }
@@ -818,7 +825,7 @@ int lbm_set_bubbles(lbm_ctx* c, int n, const double* pos3, const double* vel3,
         c->bins.cap = (int)cap;
         c->bins.items = (int*)dalloc(c, sizeof(int) * (size_t)cap);
         SwarmBins& sw = c->swarm;
-        sw.grid = swarm_grid(c->storage);
+        sw.grid = swarm_grid(&sw.sms);
         if (sw.grid < 1) {
             free_bubbles(c);
             return fail(c, LBM_ERR_CUDA, "occupancy of the bubble binning");
@@ -834,13 +841,15 @@ int lbm_set_bubbles(lbm_ctx* c, int n, const double* pos3, const double* vel3,
         sw.kidx = (int*)dalloc(c, sizeof(int) * (size_t)cap);
         sw.slots = (int*)dalloc(c, sizeof(int) * (size_t)cap);   // n * per
         sw.ntile = (int*)dalloc(c, sizeof(int) * (size_t)n);
-        sw.partial = (float*)dalloc(c, WIN_VALS_LIFT * sizeof(float) * (size_t)cap);
+        sw.partial = (float*)dalloc(c, PARTIAL_STRIDE_MAX * sizeof(float) * (size_t)cap);
         sw.cover = (int*)dalloc(c, sizeof(int) * (size_t)c->bins.T);
         sw.ncover = (int*)dalloc(c, sizeof(int));
         sw.chunk_sums = (int*)dalloc(c, sizeof(int) * (size_t)sw.grid);
         sw.zrange = (int*)dalloc(c, 2 * sizeof(int));
+        sw.cnt_next = (int*)dalloc(c, sizeof(int) * (size_t)c->bins.T);
         lists_ok = c->bins.items && sw.bar && sw.cursor && sw.kidx && sw.slots && sw.ntile &&
-                   sw.partial && sw.cover && sw.ncover && sw.chunk_sums && sw.zrange;
+                   sw.partial && sw.cover && sw.ncover && sw.chunk_sums && sw.zrange &&
+                   sw.cnt_next;
         if (lists_ok)
             LBM_CUDA(cudaMemsetAsync(sw.bar, 0, 2 * sizeof(unsigned), c->stream), "barrier");
     }

@@ -776,64 +776,66 @@ __device__ __forceinline__ QuadSlot fill_slot(uint2* s_raw, const unsigned A[Q],
     return slot;
 }
 
-// Eq. 21 at the quad (x0 .. x0 + 3), (y, z) of a tile with long lists: as
-// gather_force_tab (same products and order), over the whole tile.  A warp is
-// one z-plane, so it visits only the listed bubbles whose z weight there is
-// not zero.  Every thread of the CTA calls it.
-template <int ST>
-__device__ __forceinline__ void gather_force_quad(const Geo& g, const int* __restrict__ items,
+// Eq. 21 of a tile with long lists, as gather_force_tab (same products and
+// order) over the whole tile, in two parts per chunk of FORCE_CHUNK listed
+// bubbles.  The first stages the records and tabulates their per-axis weights
+// over the tile (every thread of the CTA calls it; the caller synchronises).
+constexpr int QUAD_NAX = TX + TY + TZ;   // x: [0, TX), y: [TX, TX + TY), z: the rest
+static_assert(FORCE_CHUNK == 32 && QX * TY == 32, "a lane per staged bubble, a warp per plane");
+
+__device__ __forceinline__ void quad_force_tables(const Geo& g, const int* __restrict__ items,
                                                   const BubbleRec* __restrict__ recs, int nb,
-                                                  int beg, int end, int bx, int by, int bz,
-                                                  bool point, BubbleRec* srec, float2 F[6]) {
-    constexpr int FB = FORCE_CHUNK, NAX = TX + TY + TZ;
-    static_assert(FB == 32 && QX * TY == 32, "a lane per staged bubble, a warp per plane");
-    __shared__ __align__(16) float s_w[FB][NAX];   // x: [0, TX), y: [TX, TX + TY), z: the rest
+                                                  int c0, int cnt, int bx, int by, int bz,
+                                                  bool point, BubbleRec* srec,
+                                                  float (*s_w)[QUAD_NAX]) {
     const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
     const int xb0 = bx * TX, yb0 = by * TY, zb0 = bz * TZ;
-    for (int c0 = beg; c0 < end; c0 += FB) {
-        const int cnt = min(FB, end - c0);
-        __syncthreads();
-        if (tid < cnt) {
-            const int id = __ldcg(items + c0 + tid);
-            if (id >= 0 && id < nb) srec[tid] = load_rec(recs + id);
-            else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        }
-        __syncthreads();
-        auto tabulate = [&](auto mode) {
-            constexpr int PM = decltype(mode)::value;
-            for (int e = tid; e < cnt * NAX; e += QUAD_THREADS) {
-                const int k = e / NAX, q = e - k * NAX;
-                const BubbleRec& r = srec[k];
-                if (q < TX)
-                    s_w[k][q] = axis_weight<PM>(r, xb0 + q, r.ax, r.fx, g.nx, !(g.walls & 0x01));
-                else if (q < TX + TY)
-                    s_w[k][q] = axis_weight<PM>(r, yb0 + q - TX, r.ay, r.fy, g.ny, !(g.walls & 0x04));
-                else
-                    s_w[k][q] =
-                        axis_weight<PM>(r, zb0 + q - TX - TY, r.az, r.fz, g.nz, !(g.walls & 0x10));
-            }
-        };
-        if (point) tabulate(MapMode<MAP_POINT>{});
-        else tabulate(MapMode<MAP_CELL>{});
-        __syncthreads();
-        const int lane = tid & 31, yi = TX + threadIdx.y, zi = TX + TY + threadIdx.z;
-        unsigned todo = __ballot_sync(0xffffffffu, lane < cnt && s_w[lane < cnt ? lane : 0][zi] != 0.0f);
-        while (todo) {
-            const int k = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const float wyz = s_w[k][yi] * s_w[k][zi];
-            if (wyz == 0.0f) continue;
-            const float4 wx = *reinterpret_cast<const float4*>(&s_w[k][4 * threadIdx.x]);
+    if (tid < cnt) {
+        const int id = __ldcg(items + c0 + tid);
+        if (id >= 0 && id < nb) srec[tid] = load_rec(recs + id);
+        else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    }
+    __syncthreads();
+    auto tabulate = [&](auto mode) {
+        constexpr int PM = decltype(mode)::value;
+        for (int e = tid; e < cnt * QUAD_NAX; e += QUAD_THREADS) {
+            const int k = e / QUAD_NAX, q = e - k * QUAD_NAX;
             const BubbleRec& r = srec[k];
-            const float2 wa = make_float2(wx.x * wyz, wx.y * wyz);
-            const float2 wb = make_float2(wx.z * wyz, wx.w * wyz);
-            F[0] = fma2(wa, f2(r.px), F[0]);
-            F[1] = fma2(wa, f2(r.py), F[1]);
-            F[2] = fma2(wa, f2(r.pz), F[2]);
-            F[3] = fma2(wb, f2(r.px), F[3]);
-            F[4] = fma2(wb, f2(r.py), F[4]);
-            F[5] = fma2(wb, f2(r.pz), F[5]);
+            if (q < TX)
+                s_w[k][q] = axis_weight<PM>(r, xb0 + q, r.ax, r.fx, g.nx, !(g.walls & 0x01));
+            else if (q < TX + TY)
+                s_w[k][q] = axis_weight<PM>(r, yb0 + q - TX, r.ay, r.fy, g.ny, !(g.walls & 0x04));
+            else
+                s_w[k][q] =
+                    axis_weight<PM>(r, zb0 + q - TX - TY, r.az, r.fz, g.nz, !(g.walls & 0x10));
         }
+    };
+    if (point) tabulate(MapMode<MAP_POINT>{});
+    else tabulate(MapMode<MAP_CELL>{});
+}
+
+// The second adds the chunk to the force F on the thread's quad.  A warp is
+// one z-plane, so it visits only the bubbles whose z weight there is not zero.
+__device__ __forceinline__ void quad_force_add(int cnt, const BubbleRec* srec,
+                                               const float (*s_w)[QUAD_NAX], float2 F[6]) {
+    const int lane = threadIdx.y * QX + threadIdx.x;
+    const int yi = TX + threadIdx.y, zi = TX + TY + threadIdx.z;
+    unsigned todo = __ballot_sync(0xffffffffu, lane < cnt && s_w[lane < cnt ? lane : 0][zi] != 0.0f);
+    while (todo) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const float wyz = s_w[k][yi] * s_w[k][zi];
+        if (wyz == 0.0f) continue;
+        const float4 wx = *reinterpret_cast<const float4*>(&s_w[k][4 * threadIdx.x]);
+        const BubbleRec& r = srec[k];
+        const float2 wa = make_float2(wx.x * wyz, wx.y * wyz);
+        const float2 wb = make_float2(wx.z * wyz, wx.w * wyz);
+        F[0] = fma2(wa, f2(r.px), F[0]);
+        F[1] = fma2(wa, f2(r.py), F[1]);
+        F[2] = fma2(wa, f2(r.pz), F[2]);
+        F[3] = fma2(wb, f2(r.px), F[3]);
+        F[4] = fma2(wb, f2(r.py), F[4]);
+        F[5] = fma2(wb, f2(r.pz), F[5]);
     }
 }
 
@@ -872,6 +874,7 @@ __device__ __forceinline__ void quad_block(const typename Store<ST>::T* __restri
         pdl_wait();
         n_t = __ldcg(tile_count + t);
     }
+    __shared__ __align__(16) float s_w[TAB ? FORCE_CHUNK : 1][QUAD_NAX];
     const QuadSlot slot = fill_slot(s_raw, A, B);
     const unsigned S = (unsigned)g.S;
     const unsigned site0 = (unsigned)site_index(g, xa, ya, za);
@@ -880,7 +883,13 @@ __device__ __forceinline__ void quad_block(const typename Store<ST>::T* __restri
         const int beg = __ldcg(tile_start + t);
         const int end = min(beg + n_t, cap);
         if (TAB) {
-            gather_force_quad<ST>(g, items, recs, nb, beg, end, bx, by, bz, cp.point != 0, srec, F);
+            for (int c0 = beg; c0 < end; c0 += FORCE_CHUNK) {
+                const int cnt = min(FORCE_CHUNK, end - c0);
+                __syncthreads();
+                quad_force_tables(g, items, recs, nb, c0, cnt, bx, by, bz, cp.point != 0, srec, s_w);
+                __syncthreads();
+                quad_force_add(cnt, srec, s_w, F);
+            }
         } else {
             const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
             for (int c0 = beg; c0 < end; c0 += FORCE_CHUNK) {

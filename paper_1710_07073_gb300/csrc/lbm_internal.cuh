@@ -169,6 +169,9 @@ struct BubbleConst {
 // weights, are sums of the velocities times per-axis difference weights).
 constexpr int WIN_VALS_LIFT = 9;
 __host__ __device__ constexpr int win_vals(bool lift) { return lift ? WIN_VALS_LIFT : 3; }
+// Floats per (tile, bubble) entry of SwarmBins::partial: whole 16-byte accesses.
+constexpr int PARTIAL_STRIDE_MAX = 12;
+__host__ __device__ constexpr int partial_stride(bool lift) { return lift ? PARTIAL_STRIDE_MAX : 4; }
 
 // A double as two floats (h = v rounded, l = the rest rounded) and back.
 __host__ __device__ inline void split_f2(double v, float& h, float& l) {
@@ -247,18 +250,21 @@ struct SmallBins {
 // in each of its tiles' lists (slots), so that the next step's interpolation
 // can be summed per tile and gathered per bubble in a fixed order.
 struct SwarmBins {
-    unsigned* bar;        // [2] grid barrier: arrivals, generation (zero between launches)
+    unsigned* bar;        // [2] grid barrier: arrivals, departures (zero between launches)
     int* cursor;          // [T] fill cursors of the counting sort
     int* kidx;            // [cap] for each list entry: which of its bubble's tiles it is
     int* slots;           // [nb * per] list position of bubble b's k-th tile
     int* ntile;           // [nb] tiles of bubble b in the last binning (0: not binned)
     int per;              // tiles a bubble's window can touch at most
-    float* partial;       // [WIN_VALS_LIFT * cap] Eq. 20 sums of each (tile, bubble) entry
+    float* partial;       // [PARTIAL_STRIDE_MAX * cap] Eq. 20 sums of each (tile, bubble) entry
     int pad;              // cells the lists reach beyond the supports (1 with lift)
     int* cover;           // [T] the tiles with a non-empty list (any order)
     int* ncover;          // [1] their number
     int* zrange;          // [2] lowest and highest z tile layer of any list (empty: lo > hi)
     int interp_grid;      // CTAs of the interpolation launch
+    int* cnt_next;        // [T] the tile counts the next binning makes; the step after
+                          // reads them as bins.cnt (the context swaps the two)
+    int sms;              // SM count
     int* chunk_sums;      // [grid] per-CTA count totals (scan)
     int grid;             // CTAs of the binning launch (all resident)
 };
@@ -349,7 +355,7 @@ cudaError_t launch_swarm_binning(const Geo& g, const BubbleDev& b, const Bins& b
 cudaError_t launch_bubble_records(const Geo& g, const BubbleDev& b, cudaStream_t st);
 // CTAs of the many-bubble binning launch that are resident at once on this
 // device, and of the interpolation launch (persistent over the covered tiles).
-int swarm_grid(int storage);
+int swarm_grid(int* sms);   // *sms: the SM count
 int interp_grid(int storage);
 // Planes per z block of the sweep that launch_collide_stream takes for these
 // buffers (even nx): a CTA's planes, within one tile layer.
