@@ -311,6 +311,29 @@ __device__ __forceinline__ void add_window_node(const float wt[4], const float u
     }
 }
 
+// Stored pre-collision values at a node none of whose neighbours lies beyond
+// a face: the sources are at fixed offsets from the node.
+template <int ST>
+__device__ __forceinline__ void gather_issue_inner(const typename Store<ST>::T* __restrict__ f,
+                                                   const Geo& g, int x, int y, int z,
+                                                   typename Store<ST>::T raw[Q]) {
+    const unsigned S = (unsigned)g.S, nx = (unsigned)g.nx, nxy = nx * (unsigned)g.ny;
+    const unsigned site = (unsigned)site_index(g, x, y, z);
+#define LBM_IN(J)                                                                               \
+    raw[J] = Store<ST>::ld(f + ((unsigned)J * S + site - ((unsigned)cx(J) + (unsigned)cy(J) * nx + \
+                                                          (unsigned)cz(J) * nxy)))
+    LBM_IN(0); LBM_IN(1); LBM_IN(2); LBM_IN(3); LBM_IN(4); LBM_IN(5); LBM_IN(6); LBM_IN(7);
+    LBM_IN(8); LBM_IN(9); LBM_IN(10); LBM_IN(11); LBM_IN(12); LBM_IN(13); LBM_IN(14);
+    LBM_IN(15); LBM_IN(16); LBM_IN(17); LBM_IN(18);
+#undef LBM_IN
+}
+
+// Whether that holds for every node of the window.
+__device__ __forceinline__ bool window_inner(const Geo& g, const Window& w) {
+    return w.lo[0] >= 1 && w.lo[0] + w.cnt[0] < g.nx && w.lo[1] >= 1 &&
+           w.lo[1] + w.cnt[1] < g.ny && w.lo[2] >= 1 && w.lo[2] + w.cnt[2] < g.nz;
+}
+
 // Eq. 20 partial sums of one chunk: nodes m0 + tid and m0 + tid + nt (below
 // m1), both gathered before either is used so their loads overlap.
 template <int ST, bool LIFT>
@@ -330,8 +353,13 @@ __device__ __forceinline__ void chunk_sum2(const typename Store<ST>::T* __restri
         wb[0] = window_node(g, w, inv_n, hb ? mb : m0, ib, jb, kb);
     }
     typename Store<ST>::T ra[Q], rb[Q];
-    gather_issue<ST>(f, g, ia, ja, ka, ra);
-    gather_issue<ST>(f, g, ib, jb, kb, rb);
+    if (window_inner(g, w)) {   // uniform over the CTA
+        gather_issue_inner<ST>(f, g, ia, ja, ka, ra);
+        gather_issue_inner<ST>(f, g, ib, jb, kb, rb);
+    } else {
+        gather_issue<ST>(f, g, ia, ja, ka, ra);
+        gather_issue<ST>(f, g, ib, jb, kb, rb);
+    }
     float ga[Q], gb[Q];
     gather_finish<ST>(ra, cp, ga);
     gather_finish<ST>(rb, cp, gb);
@@ -380,7 +408,45 @@ __device__ __noinline__ F2 fold_fp64(F2 x, int L) {
     return f2_from(v);
 }
 
-// One thread: everything after the window sums (ax, ay, az) of bubble b.
+// How the three axes of one bubble's update are spread over threads.  NA = 3: a
+// thread holds all three (many bubbles, a thread each).  NA = 1: a warp per
+// bubble, lane a holding axis a (few bubbles; the lanes beyond mirror lane 2
+// and write nothing): the sub-steps are one serial chain of instructions, and
+// a lane issues a third of the per-axis ones.  The operations per axis and
+// their order are the same.
+template <int NA> struct Axes {
+    static __device__ __forceinline__ int axis(int i) { return i; }
+    static __device__ __forceinline__ bool writes() { return true; }
+    static __device__ __forceinline__ bool lead() { return true; }
+    // The values of all three axes.
+    static __device__ __forceinline__ void all(const float* v, float o[3]) {
+        o[0] = v[0];
+        o[1] = v[1];
+        o[2] = v[2];
+    }
+    static __device__ __forceinline__ bool any(bool p) { return p; }
+    // p of axis 2.
+    static __device__ __forceinline__ bool of_z(bool p) { return p; }
+};
+template <> struct Axes<1> {
+    static __device__ __forceinline__ int axis(int) { return min((int)(threadIdx.x & 31), 2); }
+    static __device__ __forceinline__ bool writes() { return (threadIdx.x & 31) < 3; }
+    static __device__ __forceinline__ bool lead() { return (threadIdx.x & 31) == 0; }
+    static __device__ __forceinline__ void all(const float* v, float o[3]) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) o[q] = __shfl_sync(0xffffffffu, v[0], q);
+    }
+    static __device__ __forceinline__ bool any(bool p) { return __any_sync(0xffffffffu, p); }
+    static __device__ __forceinline__ bool of_z(bool p) {
+        return __shfl_sync(0xffffffffu, (int)p, 2) != 0;
+    }
+};
+
+__device__ __forceinline__ float pick(const float v[3], int a) {
+    return a == 0 ? v[0] : (a == 1 ? v[1] : v[2]);
+}
+
+// Everything after the window sums of bubble b.
 // An idle bubble leaves the coupling; a non-finite one is deactivated and
 // flags the instability; a live one takes the Table 1 forces and the Newton
 // update of Eq. 4 with the added mass on the left (m_eff), sub-stepped with
@@ -388,24 +454,29 @@ __device__ __noinline__ F2 fold_fp64(F2 x, int L) {
 // acc: the window sums, acc[0..2] the Eq. 20 velocity and, with lift,
 // acc[3..8] the vorticity sums (add_window_node).
 // Returns whether the bubble spreads in this step (B.spread); x receives the
-// new centre then.
-__device__ bool bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst& bc,
-                            int* __restrict__ flag, int b, int state, const Window& w,
-                            const float* acc, const BubbleIn& in, F2 x[3]) {
+// new centre then, and *stays whether it remains active.
+template <int NA>
+__device__ __forceinline__ bool bubble_tail(const Geo& g, const BubbleDev& B,
+                                            const BubbleConst& bc, int* __restrict__ flag, int b,
+                                            int state, const Window& w, const float* acc,
+                                            const BubbleIn& in, F2 x[3], bool* stays) {
+    using Ax = Axes<NA>;
+    const bool lead = Ax::lead(), writes = Ax::writes();
+    *stays = false;
     if (state != BUBBLE_LIVE) {
-        if (state == BUBBLE_NONFINITE) {
-            B.active[b] = 0;
-            atomicOr(flag, 2);
+        if (lead) {
+            if (state == BUBBLE_NONFINITE) {
+                B.active[b] = 0;
+                atomicOr(flag, 2);
+            }
+            B.spread[b] = 0;
+            B.cell[b] = -1;
         }
-        B.spread[b] = 0;
-        B.cell[b] = -1;
         return false;
     }
-    const int L[3] = {g.nx, g.ny, g.nz};
-    F2 xb[3] = {in.x[0], in.x[1], in.x[2]};
     const BubbleK& K = in.k;
     const float inv_norm = 1.0f / w.norm;
-    const float ul[3] = {acc[0] * inv_norm, acc[1] * inv_norm, acc[2] * inv_norm};
+    const float ul3[3] = {acc[0] * inv_norm, acc[1] * inv_norm, acc[2] * inv_norm};
     // Interpolated vorticity (lift): curl from the difference sums.
     float om[3] = {0.0f, 0.0f, 0.0f};
     if (bc.lift) {
@@ -413,77 +484,99 @@ __device__ bool bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst&
         om[1] = (acc[7] - acc[4]) * inv_norm;   // d(u_x)/dz - d(u_z)/dx
         om[2] = (acc[3] - acc[5]) * inv_norm;   // d(u_y)/dx - d(u_x)/dy
     }
-    // C_A rho_l V_b D_t u_l (virtual mass, liquid part) plus, with the
-    // stress-gradient force, rho_l V_b D_t u_l (F_S).
-    float fvm[3] = {0.0f, 0.0f, 0.0f};
-    if (in.has_prev) {
-        for (int a = 0; a < 3; ++a)
-            fvm[a] = (K.fvm_coef_dt + K.fs_coef_dt) * (ul[a] - in.ulprev[a]);
-    }
     const F2 dt_b{bc.dt_bh, bc.dt_bl};
     const F2 r{K.rh, K.rl};
-    F2 top[3];   // L - r
-    for (int a = 0; a < 3; ++a) top[a] = f2_add(F2{(float)L[a], 0.0f}, -r.h, -r.l);
+    // Per axis: the box length, the centre, L - r, the liquid's and the
+    // bubble's velocity, the buoyancy, and C_A rho_l V_b D_t u_l (virtual
+    // mass, liquid part) plus, with the stress-gradient force, rho_l V_b
+    // D_t u_l (F_S).
+    int L[NA];
+    bool wall[NA];
+    F2 xb[NA], x0[NA], top[NA];
+    float ul[NA], u[NA], fb[NA], fvm[NA], fd_sum[NA];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        const int a = Ax::axis(i);
+        L[i] = a == 0 ? g.nx : (a == 1 ? g.ny : g.nz);
+        wall[i] = g.walls & (1u << (2 * a));
+        x0[i] = a == 0 ? in.x[0] : (a == 1 ? in.x[1] : in.x[2]);
+        xb[i] = x0[i];
+        top[i] = f2_add(F2{(float)L[i], 0.0f}, -r.h, -r.l);
+        ul[i] = pick(ul3, a);
+        u[i] = pick(in.u, a);
+        fb[i] = a == 2 ? K.fb : 0.0f;
+        fvm[i] = in.has_prev ? (K.fvm_coef_dt + K.fs_coef_dt) * (ul[i] - pick(in.ulprev, a)) : 0.0f;
+        fd_sum[i] = 0.0f;
+    }
     const float sn_coeff = (float)bc.sn_coeff, sn_exp = (float)bc.sn_exp;
-    const float fb[3] = {0.0f, 0.0f, K.fb};
-    float u[3] = {in.u[0], in.u[1], in.u[2]};
-    float fd_sum[3] = {0.0f, 0.0f, 0.0f};
     bool wrap_far = false;   // a periodic coordinate left [-L, 2L): folded through FP64 below
     for (int k = 0; k < bc.substeps; ++k) {
-        const float v0 = u[0] - ul[0], v1 = u[1] - ul[1], v2 = u[2] - ul[2];
+        float v[NA], va[3];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) v[i] = u[i] - ul[i];
+        Ax::all(v, va);
+        const float v0 = va[0], v1 = va[1], v2 = va[2];
         const float speed = sqrtf(v0 * v0 + v1 * v1 + v2 * v2);
         const float re = speed * K.re_per_speed;
         // Re^b with the accurate powf (the adjoint replays the same value).
         const float visc_a = K.visc_a0 * (1.0f + sn_coeff * powf(re, sn_exp));
         const float cdv = fmaxf(fminf(visc_a, K.visc_b), K.eo_term * speed);   // C_D |v|
         const float kd = -K.drag_pref * cdv;
-        float fd[3] = {kd * v0, kd * v1, kd * v2};
+        float kl = 0.0f;
         if (bc.lift) {
             // F_L = -C_L rho_l V_b v x omega (Table 1), with the drag in the
             // reaction (Algorithm 1 step 6).
             const float cl = K.cl_tanh ? fminf(0.288f * tanhf(0.121f * re), K.cl_f) : K.cl_f;
-            const float kl = -cl * K.lift_pref;
-            fd[0] = fmaf(kl, v1 * om[2] - v2 * om[1], fd[0]);
-            fd[1] = fmaf(kl, v2 * om[0] - v0 * om[2], fd[1]);
-            fd[2] = fmaf(kl, v0 * om[1] - v1 * om[0], fd[2]);
+            kl = -cl * K.lift_pref;
         }
-        for (int a = 0; a < 3; ++a) {
-            fd_sum[a] += fd[a];
-            u[a] = fmaf(fb[a] + fd[a] + fvm[a], K.kdt, u[a]);
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            const int a = Ax::axis(i);
+            float fd = kd * v[i];
+            if (bc.lift) {
+                const float vn = a == 0 ? v1 : (a == 1 ? v2 : v0);   // axis a + 1
+                const float vp = a == 0 ? v2 : (a == 1 ? v0 : v1);   // axis a + 2
+                const float on = a == 0 ? om[1] : (a == 1 ? om[2] : om[0]);
+                const float op = a == 0 ? om[2] : (a == 1 ? om[0] : om[1]);
+                fd = fmaf(kl, vn * op - vp * on, fd);
+            }
+            fd_sum[i] += fd;
+            u[i] = fmaf(fb[i] + fd + fvm[i], K.kdt, u[i]);
             // x += u dt_b: the product as hi + lo (FMA error term), then TwoSum.
-            const float ph = u[a] * dt_b.h;
-            const float pl = fmaf(u[a], dt_b.h, -ph) + u[a] * dt_b.l;
-            xb[a] = f2_add(xb[a], ph, pl);
-            if (g.walls & (1u << (2 * a))) {
-                if (f2_lt(xb[a], r)) {
-                    xb[a] = r;
-                    u[a] = fmaxf(u[a], 0.0f);
+            const float ph = u[i] * dt_b.h;
+            const float pl = fmaf(u[i], dt_b.h, -ph) + u[i] * dt_b.l;
+            xb[i] = f2_add(xb[i], ph, pl);
+            if (wall[i]) {
+                if (f2_lt(xb[i], r)) {
+                    xb[i] = r;
+                    u[i] = fmaxf(u[i], 0.0f);
                 }
-                if (f2_lt(top[a], xb[a])) {
-                    xb[a] = top[a];
-                    u[a] = fminf(u[a], 0.0f);
+                if (f2_lt(top[i], xb[i])) {
+                    xb[i] = top[i];
+                    u[i] = fminf(u[i], 0.0f);
                 }
             } else {
-                const float La = (float)L[a];
-                if (f2_lt(xb[a], F2{0.0f, 0.0f})) xb[a] = f2_add(xb[a], La, 0.0f);
-                else if (!f2_lt(xb[a], F2{La, 0.0f})) xb[a] = f2_add(xb[a], -La, 0.0f);
-                if (!(xb[a].h >= 0.0f && xb[a].h <= La)) wrap_far = true;
+                const float La = (float)L[i];
+                if (f2_lt(xb[i], F2{0.0f, 0.0f})) xb[i] = f2_add(xb[i], La, 0.0f);
+                else if (!f2_lt(xb[i], F2{La, 0.0f})) xb[i] = f2_add(xb[i], -La, 0.0f);
+                if (!(xb[i].h >= 0.0f && xb[i].h <= La)) wrap_far = true;
             }
         }
     }
-    if (wrap_far) {
+    if (Ax::any(wrap_far)) {
         // Only reachable with runaway or non-finite velocities: fold in FP64.
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-            if (!(g.walls & (1u << (2 * a)))) xb[a] = fold_fp64(xb[a], L[a]);
+        for (int i = 0; i < NA; ++i)
+            if (!wall[i]) xb[i] = fold_fp64(xb[i], L[i]);
     }
     // A bubble that moved more than GUARD_CELLS cells along an axis in one
     // step (lattice speed > 4) flags the instability.
     bool too_fast = false;
-    for (int a = 0; a < 3; ++a) {
-        float d = (xb[a].h - in.x[a].h) + (xb[a].l - in.x[a].l);
-        if (!(g.walls & (1u << (2 * a)))) {
-            const float La = (float)L[a];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        float d = (xb[i].h - x0[i].h) + (xb[i].l - x0[i].l);
+        if (!wall[i]) {
+            const float La = (float)L[i];
             if (d > 0.5f * La) d -= La;
             else if (d < -0.5f * La) d += La;
         }
@@ -496,41 +589,87 @@ __device__ bool bubble_tail(const Geo& g, const BubbleDev& B, const BubbleConst&
     // F_D + F_L + F_S + C_A rho_l V_b D_t u_l its sub-step mean is
     // react_mb (mean F_D + F_L + fvm) - react_ca F_B, fvm = F_S + C_A rho_l
     // V_b D_t u_l.
-    float psi[3];
+    float psi[NA];
     const float inv_sub = 1.0f / (float)bc.substeps;
-    for (int a = 0; a < 3; ++a) {
-        psi[a] = bc.reaction_all
-                     ? K.react_ca * fb[a] - K.react_mb * fmaf(fd_sum[a], inv_sub, fvm[a])
-                     : -fd_sum[a] * inv_sub;
-        B.xh[3 * b + a] = xb[a].h;
-        B.xl[3 * b + a] = xb[a].l;
-        B.u[3 * b + a] = u[a];
-        B.ul[3 * b + a] = ul[a];
-        B.ulprev[3 * b + a] = ul[a];
-        B.psi[3 * b + a] = psi[a];
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        psi[i] = bc.reaction_all
+                     ? K.react_ca * fb[i] - K.react_mb * fmaf(fd_sum[i], inv_sub, fvm[i])
+                     : -fd_sum[i] * inv_sub;
+        bad = bad || !(isfinite(xb[i].h) && isfinite(u[i]) && isfinite(psi[i]));
+        if (writes) {
+            const int at = 3 * b + Ax::axis(i);
+            B.xh[at] = xb[i].h;
+            B.xl[at] = xb[i].l;
+            B.u[at] = u[i];
+            B.ul[at] = ul[i];
+            B.ulprev[at] = ul[i];
+            B.psi[at] = psi[i];
+        }
     }
-    B.has_prev[b] = 1;
-    if (!(isfinite(xb[0].h) && isfinite(xb[1].h) && isfinite(xb[2].h) && isfinite(u[0]) &&
-          isfinite(u[1]) && isfinite(u[2]) && isfinite(psi[0]) && isfinite(psi[1]) &&
-          isfinite(psi[2]))) {
-        B.active[b] = 0;
-        B.spread[b] = 0;
-        B.cell[b] = -1;
-        atomicOr(flag, 2);
+    if (lead) B.has_prev[b] = 1;
+    if (Ax::any(bad)) {
+        if (lead) {
+            B.active[b] = 0;
+            B.spread[b] = 0;
+            B.cell[b] = -1;
+            atomicOr(flag, 2);
+        }
         return false;
     }
-    B.spread[b] = 1;
-    int ci[3];
-    for (int a = 0; a < 3; ++a) {
-        float fr;
-        ci[a] = min(max(f2_floor(xb[a], fr), 0), L[a] - 1);
-    }
-    B.cell[b] = (ci[2] * g.ny + ci[1]) * g.nx + ci[0];
-    make_record(xb, K, g, psi, B.rec[b]);
-    // Algorithm 1: the bubble stops once it reaches the top of the liquid.
-    if ((g.walls & 0x20) && !f2_lt(xb[2], top[2])) B.active[b] = 0;
+    // The new centre, the cell that holds it and the spreading record.
+    float nrm[NA];
+    float fr[NA];
+    int anc[NA], ci[NA];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) x[a] = xb[a];
+    for (int i = 0; i < NA; ++i) {
+        anc[i] = f2_floor(xb[i], fr[i]);
+        ci[i] = min(max(anc[i], 0), L[i] - 1);
+        nrm[i] = axis_norm(xb[i], anc[i], fr[i], K.inv_nf, K.hmap, L[i], !wall[i]);
+    }
+    float n3[3];
+    Ax::all(nrm, n3);
+    const float inv_rec = 1.0f / (n3[0] * n3[1] * n3[2]);
+    int cell[3];
+    if constexpr (NA == 3) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            x[a] = xb[a];
+            cell[a] = ci[a];
+        }
+    } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            x[a] = F2{__shfl_sync(0xffffffffu, xb[0].h, a), __shfl_sync(0xffffffffu, xb[0].l, a)};
+            cell[a] = __shfl_sync(0xffffffffu, ci[0], a);
+        }
+    }
+    BubbleRec& rec = B.rec[b];
+    if (writes) {
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            const int a = Ax::axis(i);
+            (&rec.ax)[a] = anc[i];
+            (&rec.fx)[a] = fr[i];
+            (&rec.px)[a] = psi[i] * inv_rec;
+        }
+    }
+    // Algorithm 1: the bubble stops once it reaches the top of the liquid.
+    bool at_top = false;
+#pragma unroll
+    for (int i = 0; i < NA; ++i)
+        if (Ax::axis(i) == 2) at_top = (g.walls & 0x20) && !f2_lt(xb[i], top[i]);
+    at_top = Ax::of_z(at_top);
+    if (lead) {
+        rec.pad = 0;
+        rec.inv_n = K.inv_nf;
+        rec.h = K.hmap;
+        B.spread[b] = 1;
+        B.cell[b] = (cell[2] * g.ny + cell[1]) * g.nx + cell[0];
+        if (at_top) B.active[b] = 0;
+    }
+    *stays = !at_top;
     return true;
 }
 
@@ -955,30 +1094,35 @@ __device__ void write_zperm(int nbz, int planes, const unsigned* lay, int* __res
     }
 }
 
-// The z tile layers the support of an active bubble, widened by GUARD_CELLS
-// cells, reaches: bits of `lay` (atomicOr; shared or global memory).
-__device__ __forceinline__ void mark_guarded_layers(const Geo& g, F2 z, float nh, float nl,
-                                                    unsigned* lay) {
-    const int ntz = g.ntz;
+// The z tile layers the support of a bubble, widened by GUARD_CELLS cells,
+// reaches: [l0, l1], to be wrapped on a periodic axis (l1 < l0: none).
+__device__ __forceinline__ void guarded_layers(const Geo& g, F2 z, float nh, float nl, int& l0,
+                                               int& l1) {
     const bool periodic = !(g.walls & 0x10);
     int lo, hi;
     support_cells(z, nh, nl, lo, hi);
     lo = max(lo, -2 * g.nz) - GUARD_CELLS;
     hi = min(hi, 3 * g.nz) + GUARD_CELLS;
-    int l0, l1;
     if (!periodic) {
         lo = max(lo, 0);
         hi = min(hi, g.nz - 1);
-        if (hi < lo) return;
         l0 = lo / TZ;
-        l1 = hi / TZ;
+        l1 = hi < lo ? l0 - 1 : hi / TZ;
     } else if (hi - lo + 1 >= g.nz) {
         l0 = 0;
-        l1 = ntz - 1;
+        l1 = g.ntz - 1;
     } else {
         l0 = floor_div(lo, TZ);
         l1 = floor_div(hi, TZ);
     }
+}
+
+// The same as bits of `lay` (atomicOr; shared or global memory).
+__device__ __forceinline__ void mark_guarded_layers(const Geo& g, F2 z, float nh, float nl,
+                                                    unsigned* lay) {
+    const int ntz = g.ntz;
+    int l0, l1;
+    guarded_layers(g, z, nh, nl, l0, l1);
     for (int l = l0; l <= l1; ++l) {
         int lw = l % ntz;
         if (lw < 0) lw += ntz;
@@ -1032,6 +1176,57 @@ __device__ void write_safe_layers(const Geo& g, const BubbleDev& B, const SmallB
     }
 }
 
+// A column's only bubble: the tile list of bin_small_block and the guard of
+// write_safe_layers in closed form.  The list is written by the first warp (a
+// lane per tile), the guard by the others (every thread of the CTA calls it).
+// Its guarded layers are one run, or two that meet across the periodic
+// boundary, so every sweep block's place in the order follows from counting:
+// no sort, scan or synchronisation.  For one bubble the two general routines
+// took 8,700 of the update's 29,000 cycles.
+__device__ void bin_single(const Geo& g, const SmallBins& sb, const F2 c[3], float nh, float nl,
+                           int pad, bool spread, bool active) {
+    const int tid = threadIdx.x;
+    if (tid < 32) {
+        TileRuns r;
+        r.n = 0;
+        if (spread) r = tile_runs(g, c, nh, nl, pad);
+        for (int k = tid; k < r.n; k += 32) {
+            const int t = r.tile(g, k);
+            sb.items[k] = 0;
+            sb.prev_tiles[k] = t;
+            sb.start[t] = k;
+            sb.count[t] = 1;
+        }
+        if (tid == 0) *sb.prev_n = r.n;
+        return;
+    }
+    if (sb.safe == nullptr) return;
+    const int ntz = g.ntz, at = tid - 32, nt = (int)blockDim.x - 32;
+    int l0 = 0, l1 = -1;
+    if (active) guarded_layers(g, c[2], nh, nl, l0, l1);
+    const int n = min(l1 - l0 + 1, ntz);
+    l0 = n == ntz ? 0 : l0 % ntz;
+    if (l0 < 0) l0 += ntz;
+    // Guarded: [l0, e0) and, wrapped, [0, e1).
+    const int e0 = min(l0 + n, ntz), e1 = l0 + n - e0;
+    for (int l = at; l < ntz; l += nt)
+        if (!((l >= l0 && l < e0) || l < e1)) sb.safe[l] = sb.safe_epoch;
+    if (sb.zperm != nullptr) {
+        const int per = TZ / sb.planes, nbz = sb.nbz;   // sweep blocks per layer
+        const int b0 = min(l0 * per, nbz), b1 = min(e0 * per, nbz), w1 = min(e1 * per, nbz);
+        const int clear = nbz - (b1 - b0) - w1;
+        for (int bz = at; bz < nbz; bz += nt) {
+            const int before = min(max(bz - b0, 0), b1 - b0) + min(bz, w1);
+            const bool guarded = (bz >= b0 && bz < b1) || bz < w1;
+            sb.zperm[guarded ? clear + before : bz - before] = bz;
+        }
+    }
+    if (sb.zrange != nullptr && at == 0) {
+        sb.zrange[0] = n <= 0 ? INT_MAX : (e1 > 0 ? 0 : l0);
+        sb.zrange[1] = n <= 0 ? -1 : e0 - 1;
+    }
+}
+
 // Bubble update with the few-pair binning fused behind it.
 //
 // The window of a bubble is cut into chunks of WINDOW_CHUNK nodes (node m of
@@ -1051,6 +1246,13 @@ __device__ void write_safe_layers(const Geo& g, const BubbleDev& B, const SmallB
 // then lets the next sweep start: that sweep runs alongside the rest of the
 // update and waits for it only in the z layers the guard does not clear.
 // LIFT: the window carries the vorticity halo and nine sums (add_window_node).
+//
+// Bound by latency: in a small column the update is the step (32x32x64: 29,000
+// of its cycles ran after the sweep before had ended).  So the window's nodes
+// take fixed offsets where no face is near, the sub-steps run an axis per lane
+// (Axes<1>), and a column's only bubble is binned in closed form (bin_single):
+// 32x32x64 17.9 -> 11.9 us a step, 127x127x255 (update and sweep in stream
+// order) 136 -> 126 us.
 template <int ST, bool LIFT>
 __global__ void __launch_bounds__(BUBBLE_THREADS, 1)
 k_bubbles_binned(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp,
@@ -1059,14 +1261,16 @@ k_bubbles_binned(const typename Store<ST>::T* __restrict__ f, Geo g, CollidePara
     constexpr int NV = win_vals(LIFT);
     __shared__ float red[NV][BUBBLE_THREADS / 32];
     __shared__ unsigned long long keys[SMALL_MAX_PAIRS];
-    __shared__ int s_n, s_last;
+    __shared__ int s_n, s_last, s_spread, s_active;
+    __shared__ F2 s_x[3];
     const int parts = sb.parts;
     const int b = blockIdx.x / parts, p = blockIdx.x - b * parts;
     const bool alone = gridDim.x == 1;   // one bubble, one CTA: nothing to publish
+    const bool single = B.nb == 1 && cols == nullptr;
     pdl_wait();
     pdl_trigger();
     BubbleIn in;
-    load_bubble(B, b, threadIdx.x == 0, in);
+    load_bubble(B, b, threadIdx.x < 32, in);   // the first warp will integrate
     if (blockIdx.x == 0) {
         clear_prev_tiles(sb);
         if (!alone) __threadfence();
@@ -1105,9 +1309,9 @@ k_bubbles_binned(const typename Store<ST>::T* __restrict__ f, Geo g, CollidePara
         __syncthreads();   // `red` is reused by the next chunk
     }
     __syncthreads();       // CTA 0's clearing is complete before thread 0 arrives
-    if (threadIdx.x == 0) {
-        bool mine = true;
-        if (parts > 1) {
+    if (threadIdx.x < 32) {
+        int mine = 1;
+        if (threadIdx.x == 0 && parts > 1) {
             __threadfence();                                 // publish this CTA's chunk sums
             mine = atomicAdd(sb.arrive + b, 1) == parts - 1;
             if (mine) {
@@ -1119,21 +1323,39 @@ k_bubbles_binned(const typename Store<ST>::T* __restrict__ f, Geo g, CollidePara
                 sb.arrive[b] = 0;                            // ready for the next launch
             }
         }
-        s_last = 0;
+        mine = __shfl_sync(0xffffffffu, mine, 0);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) sum[q] = __shfl_sync(0xffffffffu, sum[q], 0);
+        int last = 0;
         if (mine) {
-            F2 x_new[3];
-            bubble_tail(g, B, bc, flag, b, state, w, sum, in, x_new);
-            if (alone) {
-                s_last = 1;
+            F2 x[3];
+            bool stays;
+            const bool spread =
+                bubble_tail<1>(g, B, bc, flag, b, state, w, sum, in, x, &stays);
+            if (single) {
+                last = 1;
+                if (threadIdx.x == 0) {
+                    s_spread = spread;
+                    s_active = stays;
+                    if (spread)
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) s_x[a] = x[a];
+                }
             } else {
                 __threadfence();                             // publish this bubble's state
-                s_last = atomicAdd(sb.done, 1) == B.nb - 1;
+                __syncwarp();
+                if (threadIdx.x == 0) last = alone || atomicAdd(sb.done, 1) == B.nb - 1;
             }
         }
+        if (threadIdx.x == 0) s_last = last;
     }
     __syncthreads();
     if (!s_last) return;
-    if (!alone) __threadfence();
+    if (single) {
+        bin_single(g, sb, s_x, in.k.nh, in.k.nl, LIFT ? 1 : 0, s_spread != 0, s_active != 0);
+        return;
+    }
+    __threadfence();
     bin_small_block(g, B, sb, keys, &s_n, LIFT ? 1 : 0, cols, bubble_col);
     if (sb.safe != nullptr && cols == nullptr) write_safe_layers(g, B, sb);
     if (threadIdx.x == 0 && !alone) *sb.done = 0;        // ready for the next launch
@@ -1566,7 +1788,8 @@ k_swarm_tail(Geo g, BubbleDev B, BubbleConst bc, int* __restrict__ flag, Bins bi
         const int state = bubble_window(g, in, w);
         F2 x[3];
         int nt = 0;
-        if (bubble_tail(g, B, bc, flag, b, state, w, acc, in, x)) {
+        bool stays;
+        if (bubble_tail<3>(g, B, bc, flag, b, state, w, acc, in, x, &stays)) {
             const TileRuns r = tile_runs(g, x, in.k.nh, in.k.nl, sw.pad);
             count_tiles(g, r, bins.cnt, zlo, zhi);
             nt = r.n;
