@@ -333,9 +333,9 @@ int lbm_get_kernel_time(lbm_ctx* ctx, double* ms, int* launches);
  * (LBM_TOP_FREE_SLIP), the optional forces (lbm_params.forces), point-sampled
  * mapping and the -sum F reaction are not covered: lbm_adj_forward returns
  * LBM_ERR_STATE.
- * Each reverse step runs the bubbles' spreading adjoint and sub-step reverse
- * (a CTA per bubble) on a second, library-owned stream alongside the per-node
- * sweep, and joins them through events before the interpolation adjoint.
+ * Each reverse step runs the bubbles' part (a CTA per bubble) and then the
+ * nodes of their interpolation windows on a second, library-owned stream
+ * alongside the per-node sweep of the other nodes.
  * Memory: one state per
  * checkpoint plus checkpoint_every states during the backward.  With kernel
  * timing on (lbm_set_kernel_timing), lbm_adj_backward times each launch of

@@ -15,12 +15,15 @@
 //   liquid          f^{n+1} = Stream(Collide(f^n, F)) (Eq. 12-16).
 // The reverse step (step n, newest first):
 //   k_adj_liquid    Lambda^n = C_f^T S^T Lambda^{n+1} per node (transposed
-//                   streaming with bounce-back, linearised forced BGK);
-//   k_adj_bubbles_ab (a CTA per bubble, on a second stream alongside
+//                   streaming with bounce-back, linearised forced BGK) at
+//                   every node outside the bubbles' interpolation windows;
+//   k_adj_bubbles   (a CTA per bubble, on a second stream alongside
 //                   k_adj_liquid: both read only Lambda^{n+1} and f^n)
-//                   spreading adjoint and the reverse of the sub-steps;
-//   k_adj_bubbles_c (after both, one CTA, bubbles in order)
-//                   the interpolation adjoint.
+//                   spreading adjoint, reverse of the sub-steps and the
+//                   interpolation's adjoint with respect to the bubble;
+//   k_adj_window    (after k_adj_bubbles, same stream) Lambda^n at the
+//                   windows' nodes: as k_adj_liquid plus the interpolation's
+//                   adjoint with respect to the liquid.
 //   In all:         per bubble: spreading adjoint (Lambda_psi, Lambda_x^{n+1},
 //                   Lambda_n from the force adjoint at the window nodes),
 //                   reverse of the sub-steps, interpolation adjoint (adds to
@@ -38,7 +41,7 @@ using namespace lbm;
 namespace {
 
 constexpr int ADJ_MAX_BUBBLES = 256;
-constexpr int ADJ_THREADS = 256;
+constexpr int ADJ_THREADS = 256;   // worker threads of k_adj_bubbles
 constexpr int ADJ_MAX_SUB = 64;
 
 // Bubble state snapshot: before a step (x, u, q = u_l history, h, active) and
@@ -47,6 +50,7 @@ struct BubbleSnap {
     double x[3], u[3], q[3], ul[3], psi[3];
     float xh[3], xl[3];   // the centre as stored (x = xh + xl), for an exact restore
     int h, active;
+    int lo[3], cnt[3];    // before a step: the interpolation window's cells
     BubbleRec rec;
 };
 
@@ -61,31 +65,6 @@ struct AdjConst {
     double rho_l, rho_b, g, sigma, c_am;
     int substeps, two_way;
 };
-
-__global__ void k_snapshot(BubbleDev B, BubbleSnap* out, int post) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B.nb) return;
-    BubbleSnap& s = out[b];
-    for (int a = 0; a < 3; ++a) {
-        s.xh[a] = B.xh[3 * b + a];
-        s.xl[a] = B.xl[3 * b + a];
-        s.x[a] = join_f2(s.xh[a], s.xl[a]);
-        s.u[a] = B.u[3 * b + a];
-        if (post) {
-            s.ul[a] = B.ul[3 * b + a];
-            s.psi[a] = B.psi[3 * b + a];
-        } else {
-            s.q[a] = B.ulprev[3 * b + a];
-        }
-    }
-    if (post) {
-        s.rec = B.rec[b];
-        s.active = B.spread[b];   // 1 if it took part in the step
-    } else {
-        s.h = B.has_prev[b];
-        s.active = B.active[b];
-    }
-}
 
 __global__ void k_restore(BubbleDev B, const BubbleSnap* in) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -153,17 +132,10 @@ __device__ __forceinline__ AxisW axis_norm_d(double x, int L, float inv_n, bool 
     return axis_weight((float)(-x), (float)((double)L - x), inv_n);
 }
 
-// Window of one bubble at centre x: cells per axis and the normalisation.
-struct Window {
-    int lo[3], cnt[3];
-    double x[3];
-    float inv_n;
-    AxisW norm[3];
-};
-
-__device__ __forceinline__ void make_window(const Geo& g, const double* x, double n, Window& w) {
+// The cells of a window at centre x, half-width n, per axis.
+__device__ __forceinline__ void window_cells(const Geo& g, const double* x, double n, int lo[3],
+                                             int cnt[3]) {
     const int L[3] = {g.nx, g.ny, g.nz};
-    w.inv_n = (float)(1.0 / n);
     for (int a = 0; a < 3; ++a) {
         const bool periodic = !(g.walls & (1u << (2 * a)));
         int l = (int)floor(x[a] - n);
@@ -172,10 +144,71 @@ __device__ __forceinline__ void make_window(const Geo& g, const double* x, doubl
             l = max(l, 0);
             h = min(h, L[a] - 1);
         }
-        w.lo[a] = l;
-        w.cnt[a] = min(max(h - l + 1, 0), 2 * (int)MAX_HALF_WIDTH + 2);
-        w.x[a] = x[a];
-        w.norm[a] = axis_norm_d(x[a], L[a], w.inv_n, periodic);
+        lo[a] = l;
+        cnt[a] = min(max(h - l + 1, 0), 2 * (int)MAX_HALF_WIDTH + 2);
+    }
+}
+
+// Window of one bubble: its cells, the centre as stored (two floats), 1/n, the
+// reciprocal of the normalisation and, per axis, its derivative over itself
+// with respect to the centre (rx) and, summed, to n (rn).
+struct Window {
+    int lo[3], cnt[3];
+    float xh[3], xl[3];
+    float inv_n, inv_norm, rx[3], rn;
+    bool inner;   // no node has a neighbour beyond a face
+};
+
+__device__ __forceinline__ void make_window(const Geo& g, const double* x, const float* xh,
+                                            const float* xl, double n, Window& w) {
+    const int L[3] = {g.nx, g.ny, g.nz};
+    window_cells(g, x, n, w.lo, w.cnt);
+    w.inv_n = (float)(1.0 / n);
+    float nrm = 1.0f;
+    w.rn = 0.0f;
+    w.inner = true;
+    for (int a = 0; a < 3; ++a) {
+        w.xh[a] = xh[a];
+        w.xl[a] = xl[a];
+        const AxisW q = axis_norm_d(x[a], L[a], w.inv_n, !(g.walls & (1u << (2 * a))));
+        nrm *= q.w;
+        w.rx[a] = q.dx / q.w;
+        w.rn += q.dn / q.w;
+        w.inner = w.inner && w.lo[a] >= 1 && w.lo[a] + w.cnt[a] < L[a];
+    }
+    w.inv_norm = 1.0f / nrm;
+}
+
+// The left end of cell c relative to the centre on axis a.
+__device__ __forceinline__ float cell_left(const Window& w, int a, int c) {
+    return ((float)c - w.xh[a]) - w.xl[a];
+}
+
+__device__ __forceinline__ int wrap1(int c, int L) { return c < 0 ? c + L : (c >= L ? c - L : c); }
+
+__global__ void k_snapshot(Geo g, BubbleDev B, BubbleSnap* out, int post) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= B.nb) return;
+    BubbleSnap& s = out[b];
+    for (int a = 0; a < 3; ++a) {
+        s.xh[a] = B.xh[3 * b + a];
+        s.xl[a] = B.xl[3 * b + a];
+        s.x[a] = join_f2(s.xh[a], s.xl[a]);
+        s.u[a] = B.u[3 * b + a];
+        if (post) {
+            s.ul[a] = B.ul[3 * b + a];
+            s.psi[a] = B.psi[3 * b + a];
+        } else {
+            s.q[a] = B.ulprev[3 * b + a];
+        }
+    }
+    if (post) {
+        s.rec = B.rec[b];
+        s.active = B.spread[b];   // 1 if it took part in the step
+    } else {
+        s.h = B.has_prev[b];
+        s.active = B.active[b];
+        window_cells(g, s.x, B.n[b], s.lo, s.cnt);
     }
 }
 
@@ -183,27 +216,49 @@ __device__ __forceinline__ void make_window(const Geo& g, const double* x, doubl
 // node's wrapped lattice coordinates in (i, j, k).
 __device__ __forceinline__ float window_node(const Geo& g, const Window& w, int m, float dWdx[3],
                                              float& dWdn, int& i, int& j, int& k) {
-    const int ix = m % w.cnt[0], rest = m / w.cnt[0];
-    const int iy = rest % w.cnt[1], iz = rest / w.cnt[1];
-    const int c[3] = {w.lo[0] + ix, w.lo[1] + iy, w.lo[2] + iz};
+    const int rest = m / w.cnt[0], iz = rest / w.cnt[1];
+    const int c[3] = {w.lo[0] + m - rest * w.cnt[0], w.lo[1] + rest - iz * w.cnt[1], w.lo[2] + iz};
     AxisW ax[3];
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float s0 = (float)((double)c[a] - w.x[a]);
+        const float s0 = cell_left(w, a, c[a]);
         ax[a] = axis_weight(s0, s0 + 1.0f, w.inv_n);
     }
-    const float nrm = w.norm[0].w * w.norm[1].w * w.norm[2].w;
-    const float W = ax[0].w * ax[1].w * ax[2].w / nrm;
-    dWdn = 0.0f;
+    const float W = ax[0].w * ax[1].w * ax[2].w * w.inv_norm;
+    dWdn = -W * w.rn;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-        const float others = ax[b1].w * ax[b2].w / nrm;
-        dWdx[a] = ax[a].dx * others - W * w.norm[a].dx / w.norm[a].w;
-        dWdn += ax[a].dn * others - W * w.norm[a].dn / w.norm[a].w;
+        const float others = ax[(a + 1) % 3].w * ax[(a + 2) % 3].w * w.inv_norm;
+        dWdx[a] = ax[a].dx * others - W * w.rx[a];
+        dWdn = fmaf(ax[a].dn, others, dWdn);
     }
-    i = (c[0] % g.nx + g.nx) % g.nx;
-    j = (c[1] % g.ny + g.ny) % g.ny;
-    k = (c[2] % g.nz + g.nz) % g.nz;
+    i = wrap1(c[0], g.nx);
+    j = wrap1(c[1], g.ny);
+    k = wrap1(c[2], g.nz);
     return W;
+}
+
+// Whether node (i, j, k) lies in a bubble's window, and its weight W there
+// (window_node's).
+__device__ __forceinline__ bool in_window(const Geo& g, const int lo[3], const int cnt[3], int i,
+                                          int j, int k) {
+    const int c[3] = {i, j, k}, L[3] = {g.nx, g.ny, g.nz};
+    bool in = true;
+#pragma unroll
+    for (int a = 2; a >= 0; --a) in = in && wrap1(c[a] - lo[a], L[a]) < cnt[a];
+    return in;
+}
+
+__device__ __forceinline__ float window_weight(const Geo& g, const Window& w, int i, int j,
+                                               int k) {
+    const int c[3] = {i, j, k}, L[3] = {g.nx, g.ny, g.nz};
+    float v[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float s0 = cell_left(w, a, w.lo[a] + wrap1(c[a] - w.lo[a], L[a]));
+        v[a] = axis_weight(s0, s0 + 1.0f, w.inv_n).w;
+    }
+    return v[0] * v[1] * v[2] * w.inv_norm;
 }
 
 __device__ __forceinline__ int node_index(const Geo& g, int i, int j, int k) {
@@ -278,6 +333,21 @@ __device__ __forceinline__ void force_at(const Geo& g, const BubbleRec* recs, co
         F[1] = fmaf(w, r.py, F[1]);
         F[2] = fmaf(w, r.pz, F[2]);
     }
+}
+
+// Bare Eq. 10 velocity and 1 / rho of shifted populations.
+__device__ __forceinline__ void node_moments(const float gv[Q], float rho0, float u[3],
+                                             float& inv_rho) {
+    float drho = 0.0f, m[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        drho += gv[q];
+        m[0] += (float)cx(q) * gv[q];
+        m[1] += (float)cy(q) * gv[q];
+        m[2] += (float)cz(q) * gv[q];
+    }
+    inv_rho = 1.0f / (rho0 + drho);
+    for (int d = 0; d < 3; ++d) u[d] = m[d] * inv_rho;
 }
 
 // Linearised forced BGK at one node, transposed.  g: shifted pre-collision
@@ -355,55 +425,251 @@ __device__ __forceinline__ void collide_adjoint(const float g[Q], const float F[
     }
 }
 
-// Lambda^n = C_f^T S^T Lambda^{n+1} at every node.
+// ---- two nodes per thread (even nx) -----------------------------------------
+// Lambda^{n+1} of direction J at the places a row's pair (x0, x0 + 1) streams
+// to: the row at (y, z) + c_J shifted against c_x, one aligned 2-wide load and,
+// for the population leaving the pair, one scalar load; a row that bounces off
+// a y or z wall takes the opposite plane of its own nodes.
+template <int J>
+__device__ __forceinline__ float2 push_pair(const float* __restrict__ lam, const Geo& g, int x0,
+                                            int y, int z) {
+    int ty = y + cy(J), tz = z + cz(J);
+    bool bounce = false;
+    if (cy(J) != 0) {
+        const bool out = (unsigned)ty >= (unsigned)g.ny;
+        bounce = out && (g.walls & 0x04);
+        ty = out ? (ty < 0 ? ty + g.ny : ty - g.ny) : ty;
+    }
+    if (cz(J) != 0) {
+        const bool out = (unsigned)tz >= (unsigned)g.nz;
+        bounce = bounce || (out && (g.walls & 0x10));
+        tz = out ? (tz < 0 ? tz + g.nz : tz - g.nz) : tz;
+    }
+    const unsigned S = (unsigned)g.S, nx = (unsigned)g.nx;
+    const unsigned own = (unsigned)opp(J) * S + (unsigned)node_index(g, x0, y, z);
+    const unsigned row = bounce ? own : (unsigned)J * S + (unsigned)node_index(g, x0, ty, tz);
+    const float2 P = __ldg(reinterpret_cast<const float2*>(lam + row));
+    if (cx(J) == 0) return P;
+    const bool wallx = (g.walls & 0x01) != 0;
+    unsigned e;
+    if (cx(J) == 1) {   // node x0 sends to x0 + 1, node x0 + 1 to x0 + 2
+        e = row + 2u;
+        if ((unsigned)x0 + 2u >= nx) e = wallx ? own + 1u : row - (unsigned)x0;
+    } else {            // node x0 sends to x0 - 1, node x0 + 1 to x0
+        e = row - 1u;
+        if (x0 == 0) e = wallx ? own : row + nx - 1u;
+    }
+    if (bounce) return P;
+    const float v = __ldg(lam + e);
+    return cx(J) == 1 ? make_float2(P.y, v) : make_float2(v, P.x);
+}
+
+// collide_adjoint without the force's adjoint on a pair of nodes, by sums s
+// and differences d of opposite directions: S1 = sum aw c from the d, the
+// second moments M = sum aw c c from the s, S2 = M u, S3 = M F, Su = S1 . u,
+// Su2 = u . S2.
+template <class Put>
+__device__ __forceinline__ void collide_adjoint_pair(float2 drho, float2 jx, float2 jy, float2 jz,
+                                                     const float2 F[3], float rho0, float omega,
+                                                     float pref, const float2 a[Q], Put put) {
+    const float2 rho = add2(f2(rho0), drho);
+    const float2 inv_rho = make_float2(1.0f / rho.x, 1.0f / rho.y);
+    const float2 u[3] = {mul2(fma2(f2(0.5f), F[0], jx), inv_rho),
+                         mul2(fma2(f2(0.5f), F[1], jy), inv_rho),
+                         mul2(fma2(f2(0.5f), F[2], jz), inv_rho)};
+    const float2 usq = fma2(u[0], u[0], fma2(u[1], u[1], mul2(u[2], u[2])));
+    float2 s[9], d[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        s[k] = add2(a[2 * k + 1], a[2 * k + 2]);
+        d[k] = sub2(a[2 * k + 1], a[2 * k + 2]);
+    }
+    // Pairs: 0 x, 1 y, 2 z, 3 (1,1,0), 4 (1,-1,0), 5 (1,0,1), 6 (1,0,-1),
+    // 7 (0,1,1), 8 (0,1,-1).
+    const float2 wa = f2(wf(1)), we = f2(wf(7));
+    const float2 exy = add2(s[3], s[4]), exz = add2(s[5], s[6]), eyz = add2(s[7], s[8]);
+    const float2 S0 = fma2(f2(wf(0)), a[0],
+                           fma2(wa, add2(add2(s[0], s[1]), s[2]), mul2(we, add2(add2(exy, exz), eyz))));
+    const float2 S1[3] = {
+        fma2(wa, d[0], mul2(we, add2(add2(d[3], d[4]), add2(d[5], d[6])))),
+        fma2(wa, d[1], mul2(we, add2(sub2(d[3], d[4]), add2(d[7], d[8])))),
+        fma2(wa, d[2], mul2(we, add2(sub2(d[5], d[6]), sub2(d[7], d[8]))))};
+    const float2 Mxx = fma2(wa, s[0], mul2(we, add2(exy, exz)));
+    const float2 Myy = fma2(wa, s[1], mul2(we, add2(exy, eyz)));
+    const float2 Mzz = fma2(wa, s[2], mul2(we, add2(exz, eyz)));
+    const float2 Mxy = mul2(we, sub2(s[3], s[4])), Mxz = mul2(we, sub2(s[5], s[6])),
+                 Myz = mul2(we, sub2(s[7], s[8]));
+    const float2 S2[3] = {fma2(Mxx, u[0], fma2(Mxy, u[1], mul2(Mxz, u[2]))),
+                          fma2(Mxy, u[0], fma2(Myy, u[1], mul2(Myz, u[2]))),
+                          fma2(Mxz, u[0], fma2(Myz, u[1], mul2(Mzz, u[2])))};
+    const float2 S3[3] = {fma2(Mxx, F[0], fma2(Mxy, F[1], mul2(Mxz, F[2]))),
+                          fma2(Mxy, F[0], fma2(Myy, F[1], mul2(Myz, F[2]))),
+                          fma2(Mxz, F[0], fma2(Myz, F[1], mul2(Mzz, F[2])))};
+    const float2 Su = fma2(S1[0], u[0], fma2(S1[1], u[1], mul2(S1[2], u[2])));
+    const float2 Su2 = fma2(S2[0], u[0], fma2(S2[1], u[1], mul2(S2[2], u[2])));
+    const float2 A_rho = mul2(f2(omega), fma2(S0, fma2(f2(-1.5f), usq, f2(1.0f)),
+                                              fma2(f2(3.0f), Su, mul2(f2(4.5f), Su2))));
+    const float2 wr = mul2(f2(omega), rho);
+    float2 Au[3], base = A_rho;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float2 eq = fma2(f2(9.0f), S2[k], mul2(f2(3.0f), sub2(S1[k], mul2(u[k], S0))));
+        const float2 guo = fma2(f2(9.0f), S3[k], mul2(f2(-3.0f), mul2(F[k], S0)));
+        Au[k] = mul2(fma2(wr, eq, mul2(f2(pref), guo)), inv_rho);
+        base = sub2(base, mul2(u[k], Au[k]));
+    }
+    // lam_k = (1 - omega) a_k + A_rho + (c_k - u) . A_u / rho
+    const float2 om1 = f2(1.0f - omega);
+    put(0, fma2(om1, a[0], base));
+    const float2 cA[9] = {Au[0], Au[1], Au[2], add2(Au[0], Au[1]), sub2(Au[0], Au[1]),
+                          add2(Au[0], Au[2]), sub2(Au[0], Au[2]), add2(Au[1], Au[2]),
+                          sub2(Au[1], Au[2])};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        put(2 * k + 1, fma2(om1, a[2 * k + 1], add2(base, cA[k])));
+        put(2 * k + 2, fma2(om1, a[2 * k + 2], sub2(base, cA[k])));
+    }
+}
+
+// What the per-node kernels need of the bubbles, in dynamic shared memory sized
+// by their number (256 of them would hold back the CTAs of one): the spreading
+// records, which bubbles spread, and the interpolation windows.
+struct AdjBox {
+    int lo[3], cnt[3];   // cnt = 0: not active
+};
+
+struct AdjView {
+    BubbleRec* rec;
+    AdjBox* box;
+    int* spread;
+    int nb;
+    __device__ __forceinline__ AdjView(unsigned char* s, int n)
+        : rec(reinterpret_cast<BubbleRec*>(s)), box(reinterpret_cast<AdjBox*>(rec + n)),
+          spread(reinterpret_cast<int*>(box + n)), nb(n) {}
+    __device__ __forceinline__ void load(const BubbleSnap* pre, const BubbleSnap* post,
+                                         int two_way) {
+        for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+            rec[b] = post[b].rec;
+            spread[b] = two_way ? post[b].active : 0;
+            for (int a = 0; a < 3; ++a) {
+                box[b].lo[a] = pre[b].lo[a];
+                box[b].cnt[a] = pre[b].active ? pre[b].cnt[a] : 0;
+            }
+        }
+        __syncthreads();
+    }
+    static size_t bytes(int nb) { return (sizeof(BubbleRec) + sizeof(AdjBox) + sizeof(int)) * (size_t)nb; }
+};
+
+// Lambda^{n+1} at the places a node's populations stream to, for a node none of
+// whose neighbours lies beyond a face.
+__device__ __forceinline__ void gather_push_inner(const float* __restrict__ lam, const Geo& g,
+                                                  int x, int y, int z, float a[Q]) {
+    const unsigned S = (unsigned)g.S, nx = (unsigned)g.nx, nxy = nx * (unsigned)g.ny;
+    const unsigned site = (unsigned)node_index(g, x, y, z);
+#define LBM_PI(J)                                                                               \
+    a[J] = __ldg(lam + ((unsigned)J * S + site + ((unsigned)cx(J) + (unsigned)cy(J) * nx +      \
+                                                  (unsigned)cz(J) * nxy)))
+    LBM_PI(0); LBM_PI(1); LBM_PI(2); LBM_PI(3); LBM_PI(4); LBM_PI(5); LBM_PI(6); LBM_PI(7);
+    LBM_PI(8); LBM_PI(9); LBM_PI(10); LBM_PI(11); LBM_PI(12); LBM_PI(13); LBM_PI(14);
+    LBM_PI(15); LBM_PI(16); LBM_PI(17); LBM_PI(18);
+#undef LBM_PI
+}
+
+// One node of the reverse step: Lambda^n (out), the force's adjoint, and the
+// bare Eq. 10 velocity with 1 / rho (the interpolation's adjoint).
+__device__ __forceinline__ void adjoint_at(const float* __restrict__ fn,
+                                           const float* __restrict__ lam_next, const Geo& g,
+                                           const CollideParams& cp, const BubbleRec* recs,
+                                           const int* spread, int nb, int x, int y, int z,
+                                           bool inner, float out[Q], float lamF[3], float u[3],
+                                           float& inv_rho) {
+    float gv[Q], a[Q], F[3];
+    if (inner) {
+        gather_issue_inner<0>(fn, g, x, y, z, gv);   // FP32 storage: the values themselves
+        gather_push_inner(lam_next, g, x, y, z, a);
+    } else {
+        gather<0>(fn, g, cp, x, y, z, gv);
+        gather_push(lam_next, g, x, y, z, a);
+    }
+    force_at(g, recs, spread, nb, x, y, z, F);
+    collide_adjoint(gv, F, cp.rho0, cp.omega, cp.pref, a, out, lamF);
+    node_moments(gv, cp.rho0, u, inv_rho);
+}
+
+#ifndef LBM_ADJ_MINB
+#define LBM_ADJ_MINB 4
+#endif
+// Lambda^n = C_f^T S^T Lambda^{n+1} at every node outside the bubbles'
+// interpolation windows, whose nodes k_adj_window writes.
+//
+// Bound by HBM (228 B per node: f^n and Lambda^{n+1} read, Lambda^n written).
+// A node per thread was bound by issue (0.172 ms on 128 x 128 x 256, 82 % of
+// the copy peak, 1,200 warp instructions per 32 nodes); on even rows a thread
+// takes an x-pair with 2-wide loads and packed arithmetic: 0.157 ms at 4 CTAs
+// per SM (124 registers; 5 and 6 spill and lose).
+__global__ void __launch_bounds__(128, LBM_ADJ_MINB)
+k_adj_liquid_pair(const float* __restrict__ fn, const float* __restrict__ lam_next,
+                  float* __restrict__ lam, Geo g, CollideParams cp,
+                  const BubbleSnap* __restrict__ pre, const BubbleSnap* __restrict__ post, int nb,
+                  int two_way) {
+    extern __shared__ unsigned char s_dyn[];
+    AdjView sh(s_dyn, nb);
+    sh.load(pre, post, two_way);
+    const unsigned half = (unsigned)g.nx / 2u;
+    const unsigned p = blockIdx.x * blockDim.x + threadIdx.x;   // 19 S < 2^32
+    if (p >= (unsigned)g.S / 2u) return;
+    const unsigned xy = p / half;
+    const int x0 = 2 * (int)(p - xy * half), y = (int)(xy % (unsigned)g.ny),
+              z = (int)(xy / (unsigned)g.ny);
+    float2 rv[Q], a[Q];
+    gather_pair<0>(fn, g, x0, y, z, rv);
+#define LBM_PP(J) a[J] = push_pair<J>(lam_next, g, x0, y, z)
+    LBM_PP(0); LBM_PP(1); LBM_PP(2); LBM_PP(3); LBM_PP(4); LBM_PP(5); LBM_PP(6); LBM_PP(7);
+    LBM_PP(8); LBM_PP(9); LBM_PP(10); LBM_PP(11); LBM_PP(12); LBM_PP(13); LBM_PP(14);
+    LBM_PP(15); LBM_PP(16); LBM_PP(17); LBM_PP(18);
+#undef LBM_PP
+    float Fa[3], Fb[3];
+    force_at(g, sh.rec, sh.spread, nb, x0, y, z, Fa);
+    force_at(g, sh.rec, sh.spread, nb, x0 + 1, y, z, Fb);
+    bool skip_a = false, skip_b = false;
+    for (int b = 0; b < nb; ++b) {
+        skip_a = skip_a || in_window(g, sh.box[b].lo, sh.box[b].cnt, x0, y, z);
+        skip_b = skip_b || in_window(g, sh.box[b].lo, sh.box[b].cnt, x0 + 1, y, z);
+    }
+    const float2 F[3] = {make_float2(Fa[0], Fb[0]), make_float2(Fa[1], Fb[1]),
+                         make_float2(Fa[2], Fb[2])};
+    float2 drho, jx, jy, jz;
+    pair_moments<0>(rv, cp, drho, jx, jy, jz);
+    const unsigned S = (unsigned)g.S, site0 = (unsigned)node_index(g, x0, y, z);
+    collide_adjoint_pair(drho, jx, jy, jz, F, cp.rho0, cp.omega, cp.pref, a,
+                         [&](int j, float2 v) {
+                             float* const at = lam + ((unsigned)j * S + site0);
+                             if (!skip_a && !skip_b) *reinterpret_cast<float2*>(at) = v;
+                             else if (!skip_a) at[0] = v.x;
+                             else if (!skip_b) at[1] = v.y;
+                         });
+}
+
+// The same, a node per thread (odd rows).
 __global__ void __launch_bounds__(128)
 k_adj_liquid(const float* __restrict__ fn, const float* __restrict__ lam_next,
-             float* __restrict__ lam, Geo g, CollideParams cp, const BubbleSnap* __restrict__ post,
-             int nb, int two_way) {
-    __shared__ BubbleRec srec[ADJ_MAX_BUBBLES];
-    __shared__ int sspread[ADJ_MAX_BUBBLES];
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        srec[b] = post[b].rec;
-        sspread[b] = two_way ? post[b].active : 0;
-    }
-    __syncthreads();
+             float* __restrict__ lam, Geo g, CollideParams cp, const BubbleSnap* __restrict__ pre,
+             const BubbleSnap* __restrict__ post, int nb, int two_way) {
+    extern __shared__ unsigned char s_dyn[];
+    AdjView sh(s_dyn, nb);
+    sh.load(pre, post, two_way);
     const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;   // 19 S < 2^32
     if (s >= (unsigned)g.S) return;
     const unsigned xy = s / (unsigned)g.nx;
     const int x = (int)(s - xy * (unsigned)g.nx), y = (int)(xy % (unsigned)g.ny),
               z = (int)(xy / (unsigned)g.ny);
-    float gv[Q], a[Q], out[Q], F[3], lamF[3];
-    gather<0>(fn, g, cp, x, y, z, gv);
-    gather_push(lam_next, g, x, y, z, a);
-    force_at(g, srec, sspread, nb, x, y, z, F);
-    collide_adjoint(gv, F, cp.rho0, cp.omega, cp.pref, a, out, lamF);
+    for (int b = 0; b < nb; ++b)
+        if (in_window(g, sh.box[b].lo, sh.box[b].cnt, x, y, z)) return;
+    float out[Q], lamF[3], u[3], inv_rho;
+    adjoint_at(fn, lam_next, g, cp, sh.rec, sh.spread, nb, x, y, z, false, out, lamF, u, inv_rho);
 #pragma unroll
     for (int j = 0; j < Q; ++j) lam[(size_t)j * g.S + s] = out[j];
-}
-
-// Sums of N values over the CTA, in thread 0 only (per value: warp shuffles,
-// then the warps in order).  The N chains interleave, so the FP64 latency is
-// paid once rather than N times.
-template <int N>
-__device__ __forceinline__ void block_sum_dn(double v[N], double (*sh)[8]) {
-    static_assert(N <= 8, "at most 8 values");
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    __syncthreads();   // the previous user of sh is done
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < N; ++i) sh[wid][i] = v[i];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) v[i] = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-#pragma unroll
-            for (int i = 0; i < N; ++i) v[i] += sh[w][i];
-    }
 }
 
 // One replayed sub-step (FP32, like the forward): slip v = u - u_l, |v|, Re,
@@ -416,292 +682,330 @@ struct SubRec {
     int xclamp[3], uclamp[3];
 };
 
-// Phases A and B of one reverse step, a CTA per bubble (blockIdx.x).  They
-// read f^n, Lambda^{n+1} and the step's snapshots only, so they run alongside
+// The bubble part of one reverse step, a CTA per bubble (blockIdx.x).  It reads
+// f^n, Lambda^{n+1} and the step's snapshots only, so it runs alongside
 // k_adj_liquid; each CTA writes its own bubble's adjoint state, diameter
 // gradient, drag-scale gradient part and interpolation seed lul_out.
-__global__ void __launch_bounds__(ADJ_THREADS)
-k_adj_bubbles_ab(const float* __restrict__ fn, const float* __restrict__ lam_next, Geo g,
-                 CollideParams cp, const BubbleSnap* __restrict__ pre,
-                 const BubbleSnap* __restrict__ post, const double* __restrict__ diam, int nb,
-                 AdjConst ac, BubbleAdj* __restrict__ adj, double* __restrict__ grad_sD,
-                 double* __restrict__ grad_d, double* __restrict__ lul_out, double loss_seed) {
-    __shared__ BubbleRec srec[ADJ_MAX_BUBBLES];
-    __shared__ int sspread[ADJ_MAX_BUBBLES];
-    __shared__ double shn[ADJ_THREADS / 32][8];
+//
+// Bound by latency (one CTA's chain of dependent loads and FP64 arithmetic), and
+// in a small column it is the reverse step.  So what does not wait for
+// something runs at once: the worker warps sum the spreading adjoint over the
+// window at x^{n+1} and the interpolation's velocity moments over the window
+// at x^n, while the last warp forms the closure constants and replays the
+// sub-steps, an axis per lane; then that warp adds up the workers' sums, a
+// value per lane, and runs the sub-steps in reverse.  With the windows' nodes
+// beside the sweep too, a reverse step of one bubble went from 0.252 to 0.157 ms
+// on 128 x 128 x 256 (the sweep's own time) and from 0.080 to 0.041 ms on 32 x
+// 32 x 64.
+constexpr int ADJ_WORKERS = ADJ_THREADS;
+constexpr int ADJ_BUBBLE_THREADS = ADJ_WORKERS + 32;
+// The workers' sums: the spreading adjoint of psi (3), of x (3) and of n, the
+// interpolation's sum u_c dW/dx_d (9) and sum u_c dW/dn (3).
+constexpr int ADJ_SUMS = 19;
+
+__device__ __forceinline__ float lane3_sum(float v) {
+    const float a = __shfl_sync(0xffffffffu, v, 0), b = __shfl_sync(0xffffffffu, v, 1),
+                c = __shfl_sync(0xffffffffu, v, 2);
+    return a + b + c;
+}
+
+__device__ __forceinline__ double lane3_sum(double v) {
+    const double a = __shfl_sync(0xffffffffu, v, 0), b = __shfl_sync(0xffffffffu, v, 1),
+                 c = __shfl_sync(0xffffffffu, v, 2);
+    return a + b + c;
+}
+
+__global__ void __launch_bounds__(ADJ_BUBBLE_THREADS)
+k_adj_bubbles(const float* __restrict__ fn, const float* __restrict__ lam_next, Geo g,
+              CollideParams cp, const BubbleSnap* __restrict__ pre,
+              const BubbleSnap* __restrict__ post, const double* __restrict__ diam, int nb,
+              AdjConst ac, BubbleAdj* __restrict__ adj, double* __restrict__ grad_sD,
+              double* __restrict__ grad_d, double* __restrict__ lul_out, double loss_seed) {
+    extern __shared__ unsigned char s_dyn[];
+    __shared__ double s_sum[ADJ_WORKERS / 32][ADJ_SUMS];
     __shared__ SubRec sub[ADJ_MAX_SUB];
-    const int tid = threadIdx.x;
+    __shared__ Window s_win[2];   // at x^{n+1} and at x^n
+    const int tid = threadIdx.x, lane = tid & 31;
     const int b = blockIdx.x;
     if (!pre[b].active) {
         // Not updated this step: its adjoint state passes through unchanged.
         if (tid == 0 && loss_seed != 0.0) adj[b].lu[2] += loss_seed;
         return;
     }
-    for (int k = tid; k < nb; k += blockDim.x) {
-        srec[k] = post[k].rec;
-        sspread[k] = ac.two_way ? post[k].active : 0;
-    }
-    __syncthreads();
-    {
-        const double d = diam[b];
-        const double n = ac.width_factor * d;
+    const double d = diam[b];
+    const double n = ac.width_factor * d;
+    AdjView sh(s_dyn, nb);
+    if (tid == 0) make_window(g, post[b].x, post[b].xh, post[b].xl, n, s_win[0]);
+    if (tid == 32) make_window(g, pre[b].x, pre[b].xh, pre[b].xl, n, s_win[1]);
+    sh.load(pre, post, ac.two_way);   // synchronises the CTA
 
-        // -- Phase A: spreading adjoint at x^{n+1} ------------------------------
-        double lpsi[3] = {0.0, 0.0, 0.0}, gx[3] = {0.0, 0.0, 0.0}, gn = 0.0;
-        if (sspread[b]) {
-            Window w;
-            make_window(g, post[b].x, n, w);
-            const double psi[3] = {post[b].psi[0], post[b].psi[1], post[b].psi[2]};
+    if (tid < ADJ_WORKERS) {
+        double sum[ADJ_SUMS];
+#pragma unroll
+        for (int i = 0; i < ADJ_SUMS; ++i) sum[i] = 0.0;
+        if (sh.spread[b]) {
+            const Window& w = s_win[0];
+            const float psi[3] = {(float)post[b].psi[0], (float)post[b].psi[1],
+                                  (float)post[b].psi[2]};   // FP32 in the forward
             const int M = w.cnt[0] * w.cnt[1] * w.cnt[2];
-            for (int m = tid; m < M; m += blockDim.x) {
-                float dWdx[3], dWdn;
+            for (int m = tid; m < M; m += ADJ_WORKERS) {
+                float dWdx[3], dWdn, out[Q], lamF[3], u[3], inv_rho;
                 int i, j, k;
                 const float W = window_node(g, w, m, dWdx, dWdn, i, j, k);
-                float gv[Q], a[Q], out[Q], F[3], lamF[3];
-                gather<0>(fn, g, cp, i, j, k, gv);
-                gather_push(lam_next, g, i, j, k, a);
-                force_at(g, srec, sspread, nb, i, j, k, F);
-                collide_adjoint(gv, F, cp.rho0, cp.omega, cp.pref, a, out, lamF);
-                const double pl = psi[0] * lamF[0] + psi[1] * lamF[1] + psi[2] * lamF[2];
+                adjoint_at(fn, lam_next, g, cp, sh.rec, sh.spread, nb, i, j, k, w.inner, out, lamF,
+                           u, inv_rho);
+                const double pl = (double)psi[0] * lamF[0] + (double)psi[1] * lamF[1] +
+                                  (double)psi[2] * lamF[2];
+#pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    lpsi[c] += (double)W * lamF[c];
-                    gx[c] += pl * dWdx[c];
+                    sum[c] += (double)W * lamF[c];
+                    sum[3 + c] += pl * dWdx[c];
                 }
-                gn += pl * dWdn;
+                sum[6] += pl * dWdn;
             }
         }
         {
-            double sums[7] = {lpsi[0], lpsi[1], lpsi[2], gx[0], gx[1], gx[2], gn};
-            block_sum_dn<7>(sums, shn);   // results in thread 0, which runs Phase B
-            for (int c = 0; c < 3; ++c) {
-                lpsi[c] = sums[c];
-                gx[c] = sums[3 + c];
+            const Window& w = s_win[1];
+            const int M = w.cnt[0] * w.cnt[1] * w.cnt[2];
+            for (int m = tid; m < M; m += ADJ_WORKERS) {
+                float dWdx[3], dWdn, gv[Q], u[3], inv_rho;
+                int i, j, k;
+                window_node(g, w, m, dWdx, dWdn, i, j, k);
+                if (w.inner) gather_issue_inner<0>(fn, g, i, j, k, gv);
+                else gather<0>(fn, g, cp, i, j, k, gv);
+                node_moments(gv, cp.rho0, u, inv_rho);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const double uc = u[c];
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) sum[7 + 3 * c + e] += uc * dWdx[e];
+                    sum[16 + c] += uc * dWdn;
+                }
             }
-            gn = sums[6];
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < ADJ_SUMS; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < ADJ_SUMS; ++i) s_sum[tid >> 5][i] = sum[i];
+        __syncthreads();
+        return;
+    }
 
-        // -- Phase B: reverse of the sub-stepped update (thread 0) ---------------
-        // The closure constants and their d-derivatives are FP64, once per step.
-        // The sub-step replay and the per-sub-step terms of its reverse run in
-        // FP32, the precision of the forward they differentiate, because FP64
-        // issue is slow on this GPU.  The centre (wall clamps) and the adjoint
-        // state carried between sub-steps and steps stay FP64.
-        if (tid == 0) {
-            const int K = min(ac.substeps, ADJ_MAX_SUB);
-            const double r = 0.5 * d, vol = M_PI * d * d * d / 6.0, dvol = 0.5 * M_PI * d * d;
-            const double meff = (ac.rho_b + ac.c_am * ac.rho_l) * vol;
-            const double kdt = ac.dt_b / meff, dkdt = -kdt / vol * dvol;
-            const double fb = (ac.rho_l - ac.rho_b) * vol * ac.g, dfb = (ac.rho_l - ac.rho_b) * ac.g * dvol;
-            const double P = 0.5 * ac.rho_l * M_PI * r * r * ac.drag_scale;
-            const double dP = 0.25 * ac.rho_l * M_PI * d * ac.drag_scale;
-            const double A0 = 24.0 * ac.nu / d, dA0 = -A0 / d;
-            const double Bv = 48.0 * ac.nu / d, dBv = -Bv / d;
-            const double Eo = (ac.rho_l - ac.rho_b) * ac.g * d * d / ac.sigma, dEo = 2.0 * Eo / d;
-            const double E = 8.0 / 3.0 * Eo / (Eo + 4.0), dE = 8.0 / 3.0 * 4.0 / ((Eo + 4.0) * (Eo + 4.0)) * dEo;
-            const double Cf = ac.c_am * ac.rho_l * vol / ac.dt_l, dCf = ac.c_am * ac.rho_l * dvol / ac.dt_l;
-            const float kdt_f = (float)kdt, fb_f = (float)fb, P_f = (float)P, A0_f = (float)A0,
-                        Bv_f = (float)Bv, E_f = (float)E;
-            const float sn_coeff = (float)ac.sn_coeff, sn_exp = (float)ac.sn_exp;
-            const float re_per_s = (float)(d / ac.nu), nu_over_d = (float)(ac.nu / d),
-                        inv_nu = (float)(1.0 / ac.nu), inv_K = 1.0f / (float)K;
-            const double* ul = post[b].ul;
-            const double* q = pre[b].q;
-            const int h = pre[b].h;
-            float ulf[3], fvm[3];
-            for (int c = 0; c < 3; ++c) {
-                ulf[c] = (float)ul[c];
-                fvm[c] = h ? (float)(Cf * (ul[c] - q[c])) : 0.0f;
+    // The last warp: lane c holds axis c (the lanes beyond mirror axis 2 and
+    // write nothing).  The closure constants and their d-derivatives are
+    // FP64, once per step.  The sub-step replay and the per-sub-step terms of
+    // its reverse run in FP32, the precision of the forward they
+    // differentiate; the centre (wall clamps) and the adjoint state carried
+    // between sub-steps and steps stay FP64.
+    const int c = min(lane, 2);
+    const bool mine = lane < 3;
+    const int K = min(ac.substeps, ADJ_MAX_SUB);
+    const double r = 0.5 * d, vol = M_PI * d * d * d / 6.0, dvol = 0.5 * M_PI * d * d;
+    const double meff = (ac.rho_b + ac.c_am * ac.rho_l) * vol;
+    const double kdt = ac.dt_b / meff, dkdt = -kdt / vol * dvol;
+    const double fb = (ac.rho_l - ac.rho_b) * vol * ac.g, dfb = (ac.rho_l - ac.rho_b) * ac.g * dvol;
+    const double P = 0.5 * ac.rho_l * M_PI * r * r * ac.drag_scale;
+    const double dP = 0.25 * ac.rho_l * M_PI * d * ac.drag_scale;
+    const double A0 = 24.0 * ac.nu / d, dA0 = -A0 / d;
+    const double Bv = 48.0 * ac.nu / d, dBv = -Bv / d;
+    const double Eo = (ac.rho_l - ac.rho_b) * ac.g * d * d / ac.sigma, dEo = 2.0 * Eo / d;
+    const double E = 8.0 / 3.0 * Eo / (Eo + 4.0), dE = 8.0 / 3.0 * 4.0 / ((Eo + 4.0) * (Eo + 4.0)) * dEo;
+    const double Cf = ac.c_am * ac.rho_l * vol / ac.dt_l, dCf = ac.c_am * ac.rho_l * dvol / ac.dt_l;
+    const float kdt_f = (float)kdt, fb_f = (float)fb, P_f = (float)P, A0_f = (float)A0,
+                Bv_f = (float)Bv, E_f = (float)E;
+    const float sn_coeff = (float)ac.sn_coeff, sn_exp = (float)ac.sn_exp;
+    const float re_per_s = (float)(d / ac.nu), nu_over_d = (float)(ac.nu / d),
+                inv_nu = (float)(1.0 / ac.nu), inv_K = 1.0f / (float)K;
+    const double ul = post[b].ul[c], q = pre[b].q[c];
+    const int h = pre[b].h;
+    const float ulf = (float)ul, fvm = h ? (float)(Cf * (ul - q)) : 0.0f;
+    const float fz = c == 2 ? fb_f : 0.0f;
+    const double top = (double)(c == 0 ? g.nx : (c == 1 ? g.ny : g.nz)) - r;
+    const bool wall = g.walls & (1u << (2 * c));
+    // forward replay
+    {
+        float u = (float)pre[b].u[c];
+        double x = pre[b].x[c];
+        for (int kk = 0; kk < K; ++kk) {
+            SubRec& sr = sub[kk];
+            const float v = u - ulf;
+            float s2 = 0.0f;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                const float ve = __shfl_sync(0xffffffffu, v, e);
+                s2 = fmaf(ve, ve, s2);
             }
-            const int L[3] = {g.nx, g.ny, g.nz};
-            // forward replay
-            float u[3] = {(float)pre[b].u[0], (float)pre[b].u[1], (float)pre[b].u[2]};
-            double x[3] = {pre[b].x[0], pre[b].x[1], pre[b].x[2]};
-            for (int kk = 0; kk < K; ++kk) {
-                SubRec& sr = sub[kk];
-                float s2 = 0.0f;
-                for (int c = 0; c < 3; ++c) {
-                    sr.v[c] = u[c] - ulf[c];
-                    s2 = fmaf(sr.v[c], sr.v[c], s2);
+            const float sp = sqrtf(s2);
+            const float re = sp * re_per_s;
+            const float pw = re > 0.0f ? powf(re, sn_exp) : 0.0f;
+            const float A = A0_f * (1.0f + sn_coeff * pw);
+            const float vis = fminf(A, Bv_f);
+            const bool eo = E_f * sp >= vis;
+            const float cdv = eo ? E_f * sp : vis;
+            const float fd = -P_f * cdv * v;
+            u = u + (fz + fd + fvm) * kdt_f;
+            x = x + (double)u * ac.dt_b;
+            int xclamp = 0, uclamp = 0;
+            if (wall) {
+                if (x < r) {
+                    x = r;
+                    xclamp = 1;
+                    if (u < 0.0f) { u = 0.0f; uclamp = 1; }
                 }
-                sr.s = sqrtf(s2);
-                sr.inv_s = sr.s > 0.0f ? 1.0f / sr.s : 0.0f;
-                sr.re = sr.s * re_per_s;
-                sr.pw = sr.re > 0.0f ? powf(sr.re, sn_exp) : 0.0f;
-                const float A = A0_f * (1.0f + sn_coeff * sr.pw);
-                const float vis = fminf(A, Bv_f);
-                if (E_f * sr.s >= vis) {
-                    sr.cdv = E_f * sr.s;
-                    sr.branch = 0;
-                } else {
-                    sr.cdv = vis;
-                    sr.branch = A <= Bv_f ? 1 : 2;
-                }
-                for (int c = 0; c < 3; ++c) {
-                    sr.fd[c] = -P_f * sr.cdv * sr.v[c];
-                    const float fz = c == 2 ? fb_f : 0.0f;
-                    u[c] = u[c] + (fz + sr.fd[c] + fvm[c]) * kdt_f;
-                    x[c] = x[c] + (double)u[c] * ac.dt_b;
-                    sr.xclamp[c] = 0;
-                    sr.uclamp[c] = 0;
-                    if (g.walls & (1u << (2 * c))) {
-                        if (x[c] < r) {
-                            x[c] = r;
-                            sr.xclamp[c] = 1;
-                            if (u[c] < 0.0f) { u[c] = 0.0f; sr.uclamp[c] = 1; }
-                        }
-                        if (x[c] > (double)L[c] - r) {
-                            x[c] = (double)L[c] - r;
-                            sr.xclamp[c] = 1;
-                            if (u[c] > 0.0f) { u[c] = 0.0f; sr.uclamp[c] = 1; }
-                        }
-                    }
+                if (x > top) {
+                    x = top;
+                    xclamp = 1;
+                    if (u > 0.0f) { u = 0.0f; uclamp = 1; }
                 }
             }
-            // reverse
-            double lx[3], lu[3], lul[3], lq[3];
-            float lfvm[3] = {0.0f, 0.0f, 0.0f}, lpsi_f[3];
-            float lP = 0.0f, lkdt = 0.0f, lfb = 0.0f, lA0 = 0.0f, lB = 0.0f, lE = 0.0f, ld_re = 0.0f;
-            for (int c = 0; c < 3; ++c) {
-                lx[c] = adj[b].lx[c] + gx[c];
-                lu[c] = adj[b].lu[c];
-                lul[c] = adj[b].lq[c];   // u_l of this step is the next step's history
-                lq[c] = 0.0;
-                lpsi_f[c] = (float)lpsi[c];
+            if (mine) {
+                sr.v[c] = v;
+                sr.fd[c] = fd;
+                sr.xclamp[c] = xclamp;
+                sr.uclamp[c] = uclamp;
             }
-            lu[2] += loss_seed;
-            for (int kk = K - 1; kk >= 0; --kk) {
-                const SubRec& sr = sub[kk];
-                double lpre[3];
-                for (int c = 0; c < 3; ++c) {
-                    // x_{k+1} = clamp(x_k + u_{k+1} dt_b), u_{k+1} = clamp(u_k + du)
-                    double lu_next = lu[c];
-                    if (!sr.xclamp[c]) lu_next += lx[c] * ac.dt_b;
-                    else lx[c] = 0.0;
-                    lpre[c] = sr.uclamp[c] ? 0.0 : lu_next;
-                }
-                float lfd[3];
-                for (int c = 0; c < 3; ++c) {
-                    const float lp = (float)lpre[c];
-                    lfd[c] = lp * kdt_f - lpsi_f[c] * inv_K;
-                    lfvm[c] += lp * kdt_f;
-                    lkdt += lp * ((c == 2 ? fb_f : 0.0f) + sr.fd[c] + fvm[c]);
-                    if (c == 2) lfb += lp * kdt_f;
-                    lu[c] = lpre[c];
-                }
-                // fd = -P cdv v
-                const float lfd_v = lfd[0] * sr.v[0] + lfd[1] * sr.v[1] + lfd[2] * sr.v[2];
-                const float lcdv = -P_f * lfd_v;
-                lP += -sr.cdv * lfd_v;
-                float lv[3] = {-P_f * sr.cdv * lfd[0], -P_f * sr.cdv * lfd[1], -P_f * sr.cdv * lfd[2]};
-                float ls = 0.0f;
-                if (sr.branch == 0) {
-                    lE += lcdv * sr.s;
-                    ls += lcdv * E_f;
-                } else if (sr.branch == 1) {
-                    lA0 += lcdv * (1.0f + sn_coeff * sr.pw);
-                    if (sr.re > 0.0f) {
-                        // d(Re^e)/dRe = e Re^e / Re, with 1/Re = nu / (d |v|)
-                        const float lre = lcdv * A0_f * sn_coeff * sn_exp * sr.pw * nu_over_d * sr.inv_s;
-                        ls += lre * re_per_s;
-                        ld_re += lre * sr.s * inv_nu;
-                    }
-                } else {
-                    lB += lcdv;
-                }
-                if (sr.s > 0.0f)
-                    for (int c = 0; c < 3; ++c) lv[c] += ls * sr.v[c] * sr.inv_s;
-                for (int c = 0; c < 3; ++c) {
-                    lu[c] += lv[c];
-                    lul[c] -= lv[c];
-                }
-            }
-            double lCf = 0.0;
-            if (h)
-                for (int c = 0; c < 3; ++c) {
-                    lul[c] += lfvm[c] * Cf;
-                    lq[c] -= lfvm[c] * Cf;
-                    lCf += lfvm[c] * (ul[c] - q[c]);
-                }
-            const double gdd = lP * dP + lkdt * dkdt + lfb * dfb + lA0 * dA0 + lB * dBv + lE * dE +
-                               ld_re + lCf * dCf + gn * ac.width_factor;
-            grad_d[b] += gdd;
-            grad_sD[b] += lP * P / ac.drag_scale;   // summed over bubbles at the end
-            for (int c = 0; c < 3; ++c) {
-                adj[b].lx[c] = lx[c];
-                adj[b].lu[c] = lu[c];
-                adj[b].lq[c] = lq[c];
-                lul_out[3 * b + c] = lul[c];
+            if (lane == 0) {
+                sr.s = sp;
+                sr.inv_s = sp > 0.0f ? 1.0f / sp : 0.0f;
+                sr.re = re;
+                sr.pw = pw;
+                sr.cdv = cdv;
+                sr.branch = eo ? 0 : (A <= Bv_f ? 1 : 2);
             }
         }
+    }
+    __syncthreads();   // the workers' sums (and, within the warp, the replay)
+    // The sums over the workers' warps, a value per lane.
+    double tot = 0.0;
+    if (lane < ADJ_SUMS)
+        for (int w = 0; w < ADJ_WORKERS / 32; ++w) tot += s_sum[w][lane];
+    const double lpsi = __shfl_sync(0xffffffffu, tot, c), gx = __shfl_sync(0xffffffffu, tot, 3 + c),
+                 gn = __shfl_sync(0xffffffffu, tot, 6);
+    // reverse
+    const float lpsi_f = (float)lpsi;
+    double lx = adj[b].lx[c] + gx, lu = adj[b].lu[c];
+    double lul = adj[b].lq[c];   // u_l of this step is the next step's history
+    double lq = 0.0;
+    float lfvm = 0.0f, lkdt = 0.0f, lfb = 0.0f;   // this axis' parts
+    float lP = 0.0f, lA0 = 0.0f, lB = 0.0f, lE = 0.0f, ld_re = 0.0f;
+    if (c == 2) lu += loss_seed;
+    for (int kk = K - 1; kk >= 0; --kk) {
+        const SubRec& sr = sub[kk];
+        // x_{k+1} = clamp(x_k + u_{k+1} dt_b), u_{k+1} = clamp(u_k + du)
+        double lu_next = lu;
+        if (!sr.xclamp[c]) lu_next += lx * ac.dt_b;
+        else lx = 0.0;
+        const double lpre = sr.uclamp[c] ? 0.0 : lu_next;
+        const float lp = (float)lpre, v = sr.v[c];
+        const float lfd = lp * kdt_f - lpsi_f * inv_K;
+        lfvm += lp * kdt_f;
+        lkdt += lp * (fz + sr.fd[c] + fvm);
+        if (c == 2) lfb += lp * kdt_f;
+        // fd = -P cdv v
+        const float lfd_v = lane3_sum(lfd * v);
+        const float lcdv = -P_f * lfd_v;
+        lP += -sr.cdv * lfd_v;
+        float lv = -P_f * sr.cdv * lfd, ls = 0.0f;
+        if (sr.branch == 0) {
+            lE += lcdv * sr.s;
+            ls += lcdv * E_f;
+        } else if (sr.branch == 1) {
+            lA0 += lcdv * (1.0f + sn_coeff * sr.pw);
+            if (sr.re > 0.0f) {
+                // d(Re^e)/dRe = e Re^e / Re, with 1/Re = nu / (d |v|)
+                const float lre = lcdv * A0_f * sn_coeff * sn_exp * sr.pw * nu_over_d * sr.inv_s;
+                ls += lre * re_per_s;
+                ld_re += lre * sr.s * inv_nu;
+            }
+        } else {
+            lB += lcdv;
+        }
+        if (sr.s > 0.0f) lv += ls * v * sr.inv_s;
+        lu = lpre + lv;
+        lul -= lv;
+    }
+    double lCf = 0.0;
+    if (h) {
+        lul += lfvm * Cf;
+        lq -= lfvm * Cf;
+        lCf = lfvm * (ul - q);
+    }
+    lCf = lane3_sum(lCf);
+    lkdt = lane3_sum(lkdt);
+    lfb = __shfl_sync(0xffffffffu, lfb, 2);
+    // The interpolation adjoint's part of the bubble: sum_c lul_c sum_nodes u_c
+    // dW/dx_d (and dW/dn).
+    double gx0 = 0.0, gn0 = 0.0;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const double le = __shfl_sync(0xffffffffu, lul, e);
+        gx0 += le * __shfl_sync(0xffffffffu, tot, 7 + 3 * e + c);
+        gn0 += le * __shfl_sync(0xffffffffu, tot, 16 + e);
+    }
+    if (mine) {
+        adj[b].lx[c] = lx + gx0;
+        adj[b].lu[c] = lu;
+        adj[b].lq[c] = lq;
+        lul_out[3 * b + c] = lul;
+    }
+    if (lane == 0) {
+        grad_d[b] += lP * dP + lkdt * dkdt + lfb * dfb + lA0 * dA0 + lB * dBv + lE * dE + ld_re +
+                     lCf * dCf + (gn + gn0) * ac.width_factor;
+        grad_sD[b] += lP * P / ac.drag_scale;   // summed over bubbles at the end
     }
 }
 
-// Phase C of one reverse step, after k_adj_liquid and k_adj_bubbles_ab: the
-// interpolation adjoint of every active bubble, one bubble after another in
-// one CTA (windows may overlap, and Lambda^n is updated in place in bubble
-// order).
-__global__ void __launch_bounds__(ADJ_THREADS)
-k_adj_bubbles_c(const float* __restrict__ fn, float* __restrict__ lam, Geo g, CollideParams cp,
-                const BubbleSnap* __restrict__ pre, const double* __restrict__ diam, int nb,
-                AdjConst ac, BubbleAdj* __restrict__ adj, double* __restrict__ grad_d,
-                const double* __restrict__ lul_in) {
-    __shared__ double shn[ADJ_THREADS / 32][8];
-    const int tid = threadIdx.x;
-    for (int b = 0; b < nb; ++b) {
-        if (!pre[b].active) continue;
-        const double n = ac.width_factor * diam[b];
-        // -- Phase C: interpolation adjoint at x^n --------------------------------
-        {
+// Lambda^n at the nodes of the interpolation windows, after k_adj_bubbles,
+// ADJ_WINDOW_CTAS CTAs per bubble.  A node in several windows belongs to the first active
+// bubble whose window holds it; the interpolation adjoints of all of them are
+// added to the collision's in bubble order: u(j) = m / rho, du / df_k = (c_k -
+// u) / rho.  (One CTA after k_adj_liquid, bubble after bubble, took 20 us of
+// every reverse step.)
+constexpr int ADJ_WINDOW_CTAS = 8, ADJ_WINDOW_THREADS = 64;
+
+__global__ void __launch_bounds__(ADJ_WINDOW_THREADS)
+k_adj_window(const float* __restrict__ fn, const float* __restrict__ lam_next,
+             float* __restrict__ lam, Geo g, CollideParams cp, const BubbleSnap* __restrict__ pre,
+             const BubbleSnap* __restrict__ post, const double* __restrict__ diam, int nb,
+             AdjConst ac, const double* __restrict__ lul_in) {
+    extern __shared__ unsigned char s_dyn[];
+    const int self = blockIdx.x / ADJ_WINDOW_CTAS, part = blockIdx.x % ADJ_WINDOW_CTAS;
+    if (!pre[self].active) return;
+    AdjView sh(s_dyn, nb);
+    sh.load(pre, post, ac.two_way);
+    const AdjBox& box = sh.box[self];
+    const int M = box.cnt[0] * box.cnt[1] * box.cnt[2];
+    for (int m = part * ADJ_WINDOW_THREADS + threadIdx.x; m < M;
+         m += ADJ_WINDOW_CTAS * ADJ_WINDOW_THREADS) {
+        const int r = m / box.cnt[0], ix = m - r * box.cnt[0];
+        const int i = wrap1(box.lo[0] + ix, g.nx), j = wrap1(box.lo[1] + r % box.cnt[1], g.ny),
+                  k = wrap1(box.lo[2] + r / box.cnt[1], g.nz);
+        bool mine = true;
+        for (int b = 0; b < self; ++b)
+            mine = mine && !in_window(g, sh.box[b].lo, sh.box[b].cnt, i, j, k);
+        if (!mine) continue;
+        float out[Q], lamF[3], uj[3], inv_rho;
+        const bool inner = i > 0 && i < g.nx - 1 && j > 0 && j < g.ny - 1 && k > 0 && k < g.nz - 1;
+        adjoint_at(fn, lam_next, g, cp, sh.rec, sh.spread, nb, i, j, k, inner, out, lamF, uj, inv_rho);
+        for (int b = self; b < nb; ++b) {
+            if (!in_window(g, sh.box[b].lo, sh.box[b].cnt, i, j, k)) continue;
             Window w;
-            make_window(g, pre[b].x, n, w);
-            const double lul[3] = {lul_in[3 * b], lul_in[3 * b + 1], lul_in[3 * b + 2]};
-            double gx0[3] = {0.0, 0.0, 0.0}, gn0 = 0.0;
-            const int M = w.cnt[0] * w.cnt[1] * w.cnt[2];
-            for (int m = tid; m < M; m += blockDim.x) {
-                float dWdx[3], dWdn;
-                int i, j, k;
-                const float W = window_node(g, w, m, dWdx, dWdn, i, j, k);
-                float gv[Q];
-                gather<0>(fn, g, cp, i, j, k, gv);
-                float drho = 0.0f, mm[3] = {0.0f, 0.0f, 0.0f};
+            make_window(g, pre[b].x, pre[b].xh, pre[b].xl, ac.width_factor * diam[b], w);
+            const float W = window_weight(g, w, i, j, k);
+            const float lw[3] = {(float)(W * lul_in[3 * b]) * inv_rho,
+                                 (float)(W * lul_in[3 * b + 1]) * inv_rho,
+                                 (float)(W * lul_in[3 * b + 2]) * inv_rho};
 #pragma unroll
-                for (int q2 = 0; q2 < Q; ++q2) {
-                    drho += gv[q2];
-                    mm[0] += (float)cx(q2) * gv[q2];
-                    mm[1] += (float)cy(q2) * gv[q2];
-                    mm[2] += (float)cz(q2) * gv[q2];
-                }
-                const float rho = cp.rho0 + drho, inv_rho = 1.0f / rho;
-                const float uj[3] = {mm[0] * inv_rho, mm[1] * inv_rho, mm[2] * inv_rho};
-                const double lu_u = lul[0] * uj[0] + lul[1] * uj[1] + lul[2] * uj[2];
-                for (int c = 0; c < 3; ++c) gx0[c] += lu_u * dWdx[c];
-                gn0 += lu_u * dWdn;
-                // u(j) = m/rho: d u / d f_k = (c_k - u) / rho
-                const int node = node_index(g, i, j, k);
-                const float lw[3] = {(float)(W * lul[0]) * inv_rho, (float)(W * lul[1]) * inv_rho,
-                                     (float)(W * lul[2]) * inv_rho};
-                // Each window node belongs to one thread: load its 19 values
-                // first, so that the read-modify-writes do not serialise.
-                float cur[Q];
-#pragma unroll
-                for (int q2 = 0; q2 < Q; ++q2) cur[q2] = lam[(size_t)q2 * g.S + node];
-#pragma unroll
-                for (int q2 = 0; q2 < Q; ++q2) {
-                    const float add = ((float)cx(q2) - uj[0]) * lw[0] + ((float)cy(q2) - uj[1]) * lw[1] +
-                                      ((float)cz(q2) - uj[2]) * lw[2];
-                    lam[(size_t)q2 * g.S + node] = cur[q2] + add;
-                }
-            }
-            double sums[4] = {gx0[0], gx0[1], gx0[2], gn0};
-            block_sum_dn<4>(sums, shn);   // results in thread 0
-            for (int c = 0; c < 3; ++c) gx0[c] = sums[c];
-            gn0 = sums[3];
-            if (tid == 0) {
-                for (int c = 0; c < 3; ++c) adj[b].lx[c] += gx0[c];
-                grad_d[b] += gn0 * ac.width_factor;
-            }
+            for (int q = 0; q < Q; ++q)
+                out[q] += ((float)cx(q) - uj[0]) * lw[0] + ((float)cy(q) - uj[1]) * lw[1] +
+                          ((float)cz(q) - uj[2]) * lw[2];
         }
-        __syncthreads();
+        const int node = node_index(g, i, j, k);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) lam[(size_t)q * g.S + node] = out[q];
     }
 }
 
@@ -714,23 +1018,50 @@ __global__ void k_adj_init(const float* __restrict__ f0, const float* __restrict
     const unsigned xy = s / (unsigned)g.nx;
     const int x = (int)(s - xy * (unsigned)g.nx), y = (int)(xy % (unsigned)g.ny),
               z = (int)(xy / (unsigned)g.ny);
+    // FP64 issues at 2 FMAs per clock and SM here, so the sums over directions
+    // run on opposite pairs in two floats (two_sum: about 48 bits), scaled by
+    // 36 so that the weights are 12, 2 and 1, and FP64 only combines them
+    // (all in FP64, 545 operations per node, took 3.97 ms on 128 x 128 x 256).
     float gv[Q];
     gather<0>(f0, g, cp, x, y, z, gv);
-    double drho = 0.0, m[3] = {0.0, 0.0, 0.0};
-    for (int j = 0; j < Q; ++j) {
-        drho += gv[j];
-        m[0] += cx(j) * (double)gv[j];
-        m[1] += cy(j) * (double)gv[j];
-        m[2] += cz(j) * (double)gv[j];
+    F2 r = F2{gv[0], 0.0f}, m[3], S0, S1[3], M[3], Mo[3];
+    for (int d = 0; d < 3; ++d) m[d] = S1[d] = M[d] = Mo[d] = F2{0.0f, 0.0f};
+    const float l0 = lam[s], l12 = __fmul_rn(l0, 12.0f);
+    S0 = F2{l12, fmaf(l0, 12.0f, -l12)};
+#pragma unroll
+    for (int j = 1; j < Q; j += 2) {
+        const F2 gs = two_sum(gv[j], gv[j + 1]), gd = two_sum(gv[j], -gv[j + 1]);
+        r = f2_add(r, gs.h, gs.l);
+        const float k = j < 7 ? 2.0f : 1.0f;
+        const float la = k * lam[(size_t)j * g.S + s], lb = k * lam[(size_t)(j + 1) * g.S + s];
+        const F2 ls = two_sum(la, lb), ld = two_sum(la, -lb);
+        S0 = f2_add(S0, ls.h, ls.l);
+        const int c[3] = {cx(j), cy(j), cz(j)};
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (c[d] != 0) {
+                const float sg = (float)c[d];
+                m[d] = f2_add(m[d], sg * gd.h, sg * gd.l);
+                S1[d] = f2_add(S1[d], sg * ld.h, sg * ld.l);
+                M[d] = f2_add(M[d], ls.h, ls.l);
+            }
+        // Off-diagonal: Mo[0] yz, Mo[1] xz, Mo[2] xy.
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float sg = (float)(c[(d + 1) % 3] * c[(d + 2) % 3]);
+            if (c[(d + 1) % 3] * c[(d + 2) % 3] != 0) Mo[d] = f2_add(Mo[d], sg * ls.h, sg * ls.l);
+        }
     }
-    const double rho = (double)cp.rho0 + drho;
-    const double u[3] = {m[0] / rho, m[1] / rho, m[2] / rho};
-    double out[3] = {0.0, 0.0, 0.0};
-    for (int j = 0; j < Q; ++j) {
-        const double c[3] = {(double)cx(j), (double)cy(j), (double)cz(j)};
-        const double cu = c[0] * u[0] + c[1] * u[1] + c[2] * u[2];
-        const double lw = (double)lam[(size_t)j * g.S + s] * wd(j) * rho;
-        for (int d = 0; d < 3; ++d) out[d] += lw * (3.0 * c[d] + 9.0 * cu * c[d] - 3.0 * u[d]);
+    auto dbl = [](F2 v) { return (double)v.h + (double)v.l; };
+    const double rho = (double)cp.rho0 + dbl(r), inv = 1.0 / rho;
+    const double u[3] = {dbl(m[0]) * inv, dbl(m[1]) * inv, dbl(m[2]) * inv};
+    const double s0 = dbl(S0);
+    const double mo[3] = {dbl(Mo[0]), dbl(Mo[1]), dbl(Mo[2])};
+    double out[3];
+    for (int d = 0; d < 3; ++d) {
+        const int e = (d + 1) % 3, f = (d + 2) % 3;
+        const double mu = dbl(M[d]) * u[d] + mo[f] * u[e] + mo[e] * u[f];
+        out[d] = rho * (1.0 / 12.0) * (dbl(S1[d]) + 3.0 * mu - u[d] * s0);
     }
     for (int d = 0; d < 3; ++d) du0[(size_t)d * g.S + s] = out[d];
 }
@@ -827,7 +1158,7 @@ extern "C" int lbm_adj_forward(lbm_ctx* c, int nsteps, int checkpoint_every, int
             t->ck_b.push_back(cb);
             LBM_CUDA(cudaMemcpyAsync(ck, c->f[c->cur], t->fbytes, cudaMemcpyDeviceToDevice, s),
                      "checkpoint");
-            k_snapshot<<<sb, 128, 0, s>>>(c->bub, cb, 0);
+            k_snapshot<<<sb, 128, 0, s>>>(g, c->bub, cb, 0);
             c->launches += 1;
         }
         rc = enqueue_one_step(c);
@@ -837,7 +1168,7 @@ extern "C" int lbm_adj_forward(lbm_ctx* c, int nsteps, int checkpoint_every, int
     }
     LBM_CUDA(cudaMemcpyAsync(t->final_f, c->f[c->cur], t->fbytes, cudaMemcpyDeviceToDevice, s),
              "final state");
-    k_snapshot<<<sb, 128, 0, s>>>(c->bub, t->final_b, 0);
+    k_snapshot<<<sb, 128, 0, s>>>(g, c->bub, t->final_b, 0);
     t->final_cur = c->cur;
     k_adj_loss<<<1, 32, 0, s>>>(t->uz, nsteps, nb, window, target, t->lossbuf);
     c->launches += 2;   // the final snapshot and the loss
@@ -921,11 +1252,14 @@ extern "C" int lbm_adj_backward(lbm_ctx* c, double dloss, double* grad_drag_scal
     step_rc(cudaMemsetAsync(lam[lc], 0, fb, s), "lambda");
     step_rc(cudaMemsetAsync(adj, 0, sizeof(BubbleAdj) * nb, s), "bubble adjoint");
     step_rc(cudaMemsetAsync(grads, 0, sizeof(double) * 2 * (size_t)nb, s), "grads");
-    // Phases A and B of the bubble adjoint run on a second stream alongside
-    // the liquid adjoint; phase C joins both.
+    // The bubble adjoint and the windows' nodes run on a second stream
+    // alongside the liquid adjoint of the other nodes; the step joins both.
     cudaStream_t s2 = nullptr;
     cudaEvent_t ev_in = nullptr, ev_ab = nullptr;
-    step_rc(cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking), "adjoint stream");
+    // (High priority: their few CTAs take the first slots the sweep frees.)
+    int least = 0, greatest = 0;
+    step_rc(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
+    step_rc(cudaStreamCreateWithPriority(&s2, cudaStreamNonBlocking, greatest), "adjoint stream");
     step_rc(cudaEventCreateWithFlags(&ev_in, cudaEventDisableTiming), "event");
     step_rc(cudaEventCreateWithFlags(&ev_ab, cudaEventDisableTiming), "event");
     struct Side {
@@ -942,6 +1276,8 @@ extern "C" int lbm_adj_backward(lbm_ctx* c, double dloss, double* grad_drag_scal
         }
     } side{s2, ev_in, ev_ab};
     const unsigned blocks = (unsigned)((g.S + 127) / 128);
+    const unsigned pair_blocks = (unsigned)((g.S / 2 + 127) / 128);
+    const size_t shared = AdjView::bytes(nb);
     const int nseg = (N + K - 1) / K;
     for (int seg = nseg - 1; seg >= 0 && rc == LBM_OK; --seg) {
         const int n0 = seg * K, n1 = std::min(N, n0 + K);
@@ -959,10 +1295,10 @@ extern "C" int lbm_adj_backward(lbm_ctx* c, double dloss, double* grad_drag_scal
             c->cur = 0;
             c->f[0] = seg_f[n - n0];
             c->f[1] = n + 1 < n1 ? seg_f[n + 1 - n0] : f_ctx[0];
-            k_snapshot<<<sb, 128, 0, s>>>(c->bub, seg_pre + (size_t)(n - n0) * nb, 0);
+            k_snapshot<<<sb, 128, 0, s>>>(g, c->bub, seg_pre + (size_t)(n - n0) * nb, 0);
             int r2 = enqueue_one_step(c);
             if (r2) rc = r2;
-            k_snapshot<<<sb, 128, 0, s>>>(c->bub, seg_post + (size_t)(n - n0) * nb, 1);
+            k_snapshot<<<sb, 128, 0, s>>>(g, c->bub, seg_post + (size_t)(n - n0) * nb, 1);
             c->launches += 2;   // the two snapshots around the recomputed step
         }
         c->f[0] = f_ctx[0];
@@ -987,16 +1323,25 @@ extern "C" int lbm_adj_backward(lbm_ctx* c, double dloss, double* grad_drag_scal
             const double ls = n >= N - t->window ? seed : 0.0;
             step_rc(cudaEventRecord(ev_in, s), "event");
             step_rc(cudaStreamWaitEvent(s2, ev_in, 0), "event wait");
-            k_adj_bubbles_ab<<<nb, ADJ_THREADS, 0, s2>>>(fn, lam[lc], g, cp, pre, post, c->bub.d, nb,
-                                                          ac, adj, grads + nb, grads, lul, ls);
+            k_adj_bubbles<<<nb, ADJ_BUBBLE_THREADS, shared, s2>>>(fn, lam[lc], g, cp, pre, post, c->bub.d,
+                                                                  nb, ac, adj, grads + nb, grads, lul, ls);
             step_rc(cudaGetLastError(), "bubble adjoint");
-            step_rc(cudaEventRecord(ev_ab, s2), "event");
-            k_adj_liquid<<<blocks, 128, 0, s>>>(fn, lam[lc], lam[lc ^ 1], g, cp, post, nb, ac.two_way);
+            if (g.nx & 1)
+                k_adj_liquid<<<blocks, 128, shared, s>>>(fn, lam[lc], lam[lc ^ 1], g, cp, pre, post, nb,
+                                                         ac.two_way);
+            else
+                k_adj_liquid_pair<<<pair_blocks, 128, shared, s>>>(fn, lam[lc], lam[lc ^ 1], g, cp, pre,
+                                                                   post, nb, ac.two_way);
             if (e1) step_rc(cudaEventRecord(e1, s), "event");
-            step_rc(cudaStreamWaitEvent(s, ev_ab, 0), "event wait");
-            k_adj_bubbles_c<<<1, ADJ_THREADS, 0, s>>>(fn, lam[lc ^ 1], g, cp, pre, c->bub.d, nb, ac, adj,
-                                                       grads, lul);
             step_rc(cudaGetLastError(), "adjoint step");
+            // Enqueued after the sweep it runs beside: ahead of it, its wait
+            // for the bubble adjoint can hold the sweep back where the two
+            // streams share a hardware queue.
+            k_adj_window<<<nb * ADJ_WINDOW_CTAS, ADJ_WINDOW_THREADS, shared, s2>>>(fn, lam[lc], lam[lc ^ 1], g, cp, pre, post,
+                                                          c->bub.d, nb, ac, lul);
+            step_rc(cudaGetLastError(), "window adjoint");
+            step_rc(cudaEventRecord(ev_ab, s2), "event");
+            step_rc(cudaStreamWaitEvent(s, ev_ab, 0), "event wait");
             c->launches += 3;
             lc ^= 1;
         }

@@ -35,28 +35,12 @@ namespace lbm {
 // FP32 pipe: FP64 issue is slow on this GPU and the bubble update is one
 // serial thread.  Sums use Knuth's TwoSum; the product error of u dt_b comes
 // from one FMA (the exact-product property of fused multiply-add).
-struct F2 {
-    float h, l;
-};
-
 __device__ __forceinline__ F2 f2_from(double v) {
     const float h = (float)v;
     return F2{h, (float)(v - (double)h)};
 }
 
 __device__ __forceinline__ double f2_to(F2 a) { return (double)a.h + (double)a.l; }
-
-__device__ __forceinline__ F2 two_sum(float a, float b) {
-    const float s = a + b;
-    const float bb = s - a;
-    return F2{s, (a - (s - bb)) + (b - bb)};
-}
-
-// (a.h + a.l) + (bh + bl)
-__device__ __forceinline__ F2 f2_add(F2 a, float bh, float bl) {
-    const F2 s = two_sum(a.h, bh);
-    return two_sum(s.h, s.l + (a.l + bl));
-}
 
 __device__ __forceinline__ bool f2_lt(F2 a, F2 b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
 
@@ -309,23 +293,6 @@ __device__ __forceinline__ void add_window_node(const float wt[4], const float u
         acc[7] = fmaf(wt[3], u[0], acc[7]);
         acc[8] = fmaf(wt[3], u[1], acc[8]);
     }
-}
-
-// Stored pre-collision values at a node none of whose neighbours lies beyond
-// a face: the sources are at fixed offsets from the node.
-template <int ST>
-__device__ __forceinline__ void gather_issue_inner(const typename Store<ST>::T* __restrict__ f,
-                                                   const Geo& g, int x, int y, int z,
-                                                   typename Store<ST>::T raw[Q]) {
-    const unsigned S = (unsigned)g.S, nx = (unsigned)g.nx, nxy = nx * (unsigned)g.ny;
-    const unsigned site = (unsigned)site_index(g, x, y, z);
-#define LBM_IN(J)                                                                               \
-    raw[J] = Store<ST>::ld(f + ((unsigned)J * S + site - ((unsigned)cx(J) + (unsigned)cy(J) * nx + \
-                                                          (unsigned)cz(J) * nxy)))
-    LBM_IN(0); LBM_IN(1); LBM_IN(2); LBM_IN(3); LBM_IN(4); LBM_IN(5); LBM_IN(6); LBM_IN(7);
-    LBM_IN(8); LBM_IN(9); LBM_IN(10); LBM_IN(11); LBM_IN(12); LBM_IN(13); LBM_IN(14);
-    LBM_IN(15); LBM_IN(16); LBM_IN(17); LBM_IN(18);
-#undef LBM_IN
 }
 
 // Whether that holds for every node of the window.

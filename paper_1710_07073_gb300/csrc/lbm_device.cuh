@@ -17,6 +17,25 @@ __device__ __forceinline__ void pdl_trigger() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// ---- two floats ------------------------------------------------------------------
+// hi + lo with |lo| <= ulp(hi)/2, about 48 significant bits: sums by Knuth's
+// TwoSum.  (A product as an argument may be contracted into the sum.)
+struct F2 {
+    float h, l;
+};
+
+__device__ __forceinline__ F2 two_sum(float a, float b) {
+    const float s = a + b;
+    const float bb = s - a;
+    return F2{s, (a - (s - bb)) + (b - bb)};
+}
+
+// (a.h + a.l) + (bh + bl)
+__device__ __forceinline__ F2 f2_add(F2 a, float bh, float bl) {
+    const F2 s = two_sum(a.h, bh);
+    return two_sum(s.h, s.l + (a.l + bl));
+}
+
 // ---- population storage ------------------------------------------------------
 // Stored value of population j is the shifted deviation g_j = f_j - w_j rho0:
 // as is for FP32, times scale / w_j for the 16-bit formats.  load/store convert
@@ -193,6 +212,23 @@ __device__ __forceinline__ void gather_issue(const typename Store<ST>::T* __rest
 #undef LBM_OFF
 #pragma unroll
     for (int q = 0; q < Q; ++q) raw[q] = Store<ST>::ld(f + o[q]);
+}
+
+// Stored pre-collision values at a node none of whose neighbours lies beyond
+// a face: the sources are at fixed offsets from the node.
+template <int ST>
+__device__ __forceinline__ void gather_issue_inner(const typename Store<ST>::T* __restrict__ f,
+                                                   const Geo& g, int x, int y, int z,
+                                                   typename Store<ST>::T raw[Q]) {
+    const unsigned S = (unsigned)g.S, nx = (unsigned)g.nx, nxy = nx * (unsigned)g.ny;
+    const unsigned site = (unsigned)site_index(g, x, y, z);
+#define LBM_IN(J)                                                                               \
+    raw[J] = Store<ST>::ld(f + ((unsigned)J * S + site - ((unsigned)cx(J) + (unsigned)cy(J) * nx + \
+                                                          (unsigned)cz(J) * nxy)))
+    LBM_IN(0); LBM_IN(1); LBM_IN(2); LBM_IN(3); LBM_IN(4); LBM_IN(5); LBM_IN(6); LBM_IN(7);
+    LBM_IN(8); LBM_IN(9); LBM_IN(10); LBM_IN(11); LBM_IN(12); LBM_IN(13); LBM_IN(14);
+    LBM_IN(15); LBM_IN(16); LBM_IN(17); LBM_IN(18);
+#undef LBM_IN
 }
 
 // Stored values to shifted populations f_j - w_j rho0.
