@@ -256,10 +256,9 @@ int lbm_set_bubbles(lbm_ctx* ctx, int n, const double* pos3, const double* vel3,
  *      applies Eq. 13, 6, 14, 12, 15 and streams (Eq. 16) with bounce-back;
  *   4. a bubble whose centre reached nz - r_b under a +z wall is deactivated
  *      (Algorithm 1, stop at the top) after spreading this step.
- * With few bubbles (the single-launch binning) on even-nx lattices, a step's
- * sweep may start while its bubble update still runs: lattice z layers that
- * no bubble can reach this step (support widened by 4 cells) do not wait for
- * it.  Results are the same bits as with the two in stream order (which the
+ * With few bubbles (the single-launch binning), a step's sweep may start
+ * while its bubble update still runs: lattice z layers that no bubble can
+ * reach this step (support widened by 4 cells) do not wait for it.  Results are the same bits as with the two in stream order (which the
  * library keeps while kernel timing is on).  With many bubbles, or few
  * bubbles in a lattice of 2^24 sites or more, on even-nx lattices whose z
  * axis is wall-bounded, a step forks from the context stream into two

@@ -54,6 +54,7 @@ struct lbm_batch {
     SmallBins small{};
 
     // launch shape (autotuned)
+    bool quad = false;       // four nodes per thread in the sweep (set on first device use)
     int planes = SWEEP_PZ;   // z-planes per CTA: the CTA tile is 32 x 4 x planes nodes
     int depth = 2;           // z-blocks (of `planes` planes) per work item
     int grid = 0;            // persistent CTAs
@@ -242,7 +243,10 @@ int ensure_device(lbm_batch* b) {
     int dev = 0, sms = 0;
     LBM_BCUDA(cudaGetDevice(&dev), "device");
     LBM_BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    if (!b->grid_fixed) b->grid = sms * batch_min_blocks(b->storage, b->planes);
+    b->quad = true;
+    for (int c = 0; c < b->ncols; ++c)
+        b->quad = b->quad && sweep_planes(b->storage, b->dims[3 * c], b->f[0], b->f[1]) != SWEEP_PZ;
+    if (!b->grid_fixed) b->grid = sms * batch_min_blocks(b->storage, b->planes, b->quad);
     b->dev_ready = true;
     return LBM_OK;
 }
@@ -275,7 +279,7 @@ int enqueue_step(lbm_batch* b, bool time_it) {
     const bool two_way = bubbles && b->p.two_way;
     TileLists none{nullptr, nullptr, nullptr, 0};
     LBM_BCUDA(launch_collide_batch(b->storage, b->f[b->cur], b->f[b->cur ^ 1], b->cols_d, b->ncols,
-                                   b->total_items, b->depth, b->grid, b->planes,
+                                   b->total_items, b->depth, b->grid, b->planes, b->quad,
                                    b->work_counter,
                                    two_way ? tl : none, b->bub.rec, b->bub.nb, b->flag_d, s),
               "batch collide-stream");
@@ -652,7 +656,7 @@ int lbm_batch_tune(lbm_batch* b, int trial_steps, int* depth_out, int* grid_out)
     const bool timing = b->timing;
     b->timing = false;
     for (int pl : planes_c) {
-        const int maxb = batch_min_blocks(b->storage, pl);
+        const int maxb = batch_min_blocks(b->storage, pl, b->quad);
         const int per_sm[] = {maxb / 2, maxb, 2 * maxb};
         for (int d : depths) {
             for (int k : per_sm) {
@@ -726,7 +730,7 @@ int lbm_batch_set_launch_shape(lbm_batch* b, int planes, int depth, int grid) {
         int dev = 0, sms = 0;
         LBM_BCUDA(cudaGetDevice(&dev), "device");
         LBM_BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-        b->grid = sms * batch_min_blocks(b->storage, planes);
+        b->grid = sms * batch_min_blocks(b->storage, planes, b->quad);
     }
     if (b->dev_ready) {
         layout_columns(b);

@@ -314,14 +314,14 @@ int enqueue_one_step(lbm_ctx* c) {
     const CollideParams cp = collide_params(c);
     const bool bubbles = c->bub.nb > 0;
     const bool two_way = bubbles && c->p.two_way;
-    // Two-way coupling on even rows: the update and the sweep overlap
+    // Two-way coupling: the update and the sweep overlap
     // (programmatic dependent launches), guarded by the tags the update before
     // wrote.  Timed launches keep plain stream order so that the sweep's
     // events time the sweep alone.
     unsigned* const safe = c->use_small ? c->small.safe : nullptr;
     int* const zperm = c->use_small ? c->small.zperm : nullptr;
     const int nbz = c->small.nbz;
-    const bool overlap = two_way && safe != nullptr && !c->timing && (g.nx & 1) == 0;
+    const bool overlap = two_way && safe != nullptr && !c->timing;
     if (c->epoch >= 0xFFFFFF00u) {
         // Before the step number wraps: no stored tag may match a later one.
         if (safe)

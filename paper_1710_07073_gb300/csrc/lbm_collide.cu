@@ -186,56 +186,73 @@ __device__ __forceinline__ void collide_store(typename Store<ST>::T* __restrict_
 #undef LBM_PAIR
 }
 
+// Odd rows: a CTA is 32 x 4 nodes of one z-plane, a node per thread (rows of odd
+// length leave no aligned 2-wide access).  127 x 127 x 255, FP32: 0.115 ms, 80 %
+// of the copy peak.  Two planes per thread, all rows loaded first, took 0.122 ms:
+// it is not the loads in flight that bound it but the sectors that unaligned
+// rows share between warps.  Overlapped with the bubble update as the even
+// rows' sweep is (126 us a step before, in stream order).
+constexpr int ODD_PZ = 1;
+constexpr int ODD_CHUNK = 32;   // bubble records staged per pass
+
 template <int ST>
 __global__ void __launch_bounds__(TX * TY, 8)
 k_collide_stream(const typename Store<ST>::T* __restrict__ fin,
                  typename Store<ST>::T* __restrict__ fout, Geo g, CollideParams cp,
-                 const int* __restrict__ tile_start, const int* __restrict__ tile_count,
-                 const int* __restrict__ items, int cap, const BubbleRec* __restrict__ recs,
-                 int nb, int* __restrict__ flag) {
-    __shared__ BubbleRec srec[TX * TY];
+                 const int* tile_start, const int* tile_count, const int* items, int cap,
+                 const BubbleRec* recs, int nb, int* __restrict__ flag, const unsigned* safe,
+                 unsigned epoch, const int* zperm) {
+    __shared__ BubbleRec srec[ODD_CHUNK];
+    pdl_trigger();
+    const int z = zperm != nullptr ? __ldcg(zperm + blockIdx.z) : (int)blockIdx.z;
+    const bool lead = (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
     const int x = blockIdx.x * TX + threadIdx.x;
     const int y = blockIdx.y * TY + threadIdx.y;
-    const int z = blockIdx.z;
     const bool inside = (x < g.nx) && (y < g.ny);
-
-    float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
-    bool forced = false;   // uniform over the CTA
+    const int t = ((z / TZ) * g.nty + blockIdx.y) * g.ntx + blockIdx.x;
+    // The order of the tile count, the population loads and the wait for an
+    // overlapped update is sweep_block's.
+    int n_t = 0;
+    bool skip = false;
     if (tile_count != nullptr) {
-        const int t = ((z / TZ) * g.nty + blockIdx.y) * g.ntx + blockIdx.x;
-        const int n_t = tile_count[t];
-        if (n_t > 0) {
-            forced = true;
-            const int beg = tile_start[t];
-            const int end = min(beg + n_t, cap);
-            const int tid = threadIdx.y * TX + threadIdx.x;
-            for (int c0 = beg; c0 < end; c0 += TX * TY) {
-                const int cnt = min(TX * TY, end - c0);
-                __syncthreads();
-                if (tid < cnt) {
-                    const int id = items[c0 + tid];
-                    if (id >= 0 && id < nb) srec[tid] = recs[id];
-                    else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                }
-                __syncthreads();
-                if (inside)
-                    for (int k = 0; k < cnt; ++k) add_bubble_force(srec[k], g, x, y, z, Fx, Fy, Fz);
+        if (safe == nullptr) n_t = __ldcg(tile_count + t);
+        else skip = !lead && __ldcg(safe + z / TZ) == epoch;
+    }
+    const unsigned S = (unsigned)g.S;
+    const unsigned nx = (unsigned)g.nx, nxy = (unsigned)g.nx * (unsigned)g.ny;
+    // Threads beyond the box gather at a valid node and store nothing.
+    const int xa = min(x, g.nx - 1), ya = min(y, g.ny - 1);
+    const unsigned site = (unsigned)z * nxy + (unsigned)ya * nx + (unsigned)xa;
+    float rv[Q];
+    // Rows away from the y and z faces (uniform over a warp, which is one row).
+    if (ya > 0 && ya < g.ny - 1 && z > 0 && z < g.nz - 1)
+        gather_rows<ST>(fin, S, site, nx, nxy, xa == 0, xa == g.nx - 1, (g.walls & 0x01) != 0, rv);
+    else
+        gather_any<ST>(fin, g, xa, ya, z, rv);
+    if (tile_count != nullptr && safe != nullptr && !skip) {
+        pdl_wait();
+        n_t = __ldcg(tile_count + t);
+    }
+    float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
+    if (n_t > 0) {   // uniform over the CTA (one tile)
+        const int beg = __ldcg(tile_start + t);
+        const int end = min(beg + n_t, cap);
+        const int tid = threadIdx.y * TX + threadIdx.x;
+        for (int c0 = beg; c0 < end; c0 += ODD_CHUNK) {
+            const int cnt = min(ODD_CHUNK, end - c0);
+            __syncthreads();
+            if (tid < cnt) {
+                const int id = __ldcg(items + c0 + tid);
+                if (id >= 0 && id < nb) srec[tid] = load_rec(recs + id);
+                else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             }
+            __syncthreads();
+            if (inside)
+                for (int k = 0; k < cnt; ++k) add_bubble_force(srec[k], g, x, y, z, Fx, Fy, Fz);
         }
     }
     if (!inside) return;
-
-    const unsigned S = (unsigned)g.S;
-    const unsigned nx = (unsigned)g.nx, nxy = (unsigned)g.nx * (unsigned)g.ny;
-    const unsigned site = (unsigned)z * nxy + (unsigned)y * nx + (unsigned)x;
-    float rv[Q];
-    // Rows away from the y and z faces (uniform over a warp, which is one row).
-    if (y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 1)
-        gather_rows<ST>(fin, S, site, nx, nxy, x == 0, x == g.nx - 1, (g.walls & 0x01) != 0, rv);
-    else
-        gather_any<ST>(fin, g, x, y, z, rv);
-
-    if (forced) collide_store<ST, true>(fout, S, site, rv, Fx, Fy, Fz, cp, flag);
+    if (n_t > 0) collide_store<ST, true>(fout, S, site, rv, Fx, Fy, Fz, cp, flag);
     else collide_store<ST, false>(fout, S, site, rv, 0.0f, 0.0f, 0.0f, cp, flag);
 }
 
@@ -577,11 +594,11 @@ constexpr int QUAD_THREADS = QX * TY * QUAD_PZ;
 #endif
 // CTA shape and residency of the sweep kernels, by nodes per thread.
 template <int ST, int NODES> struct SweepShape {
-    static constexpr int kThreads = PX * TY * PZ;
+    static constexpr int kThreads = PX * TY * PZ, kPlanes = PZ;
     static constexpr int kMinBlocks = PairOccupancy<ST>::kMinBlocks;
 };
 template <int ST> struct SweepShape<ST, 4> {
-    static constexpr int kThreads = QUAD_THREADS;
+    static constexpr int kThreads = QUAD_THREADS, kPlanes = QUAD_PZ;
     static constexpr int kMinBlocks = LBM_QUAD_MINB;
 };
 
@@ -589,9 +606,10 @@ template <int ST> struct SweepShape<ST, 4> {
 // and the relaxation (a slot per thread, so no synchronisation): held in
 // registers, packed and widened, they spill at any occupancy that hides the
 // load latency.
+template <int PZV>
 struct QuadSlot {
     unsigned at;   // shared-space address of direction 0
-    static constexpr unsigned STRIDE = QUAD_THREADS * 8;
+    static constexpr unsigned STRIDE = QX * TY * PZV * 8;
     template <int J>
     __device__ __forceinline__ void put(unsigned a, unsigned b) const {
         asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(at + J * STRIDE), "r"(a), "r"(b));
@@ -670,14 +688,14 @@ struct PackedPair {
     __device__ __forceinline__ void put(float2 x) { v[(J + 1) & 1] = Raw2<ST>::pack(x); }
 };
 
-template <int ST, int J, bool FORCED>
+template <int ST, int J, bool FORCED, class Slot>
 __device__ __forceinline__ void relax_quad(typename Store<ST>::T* __restrict__ fout, unsigned S,
-                                           unsigned site0, const QuadSlot& slot,
+                                           unsigned site0, const Slot& slot,
                                            const PairState& pa, const PairState& pb,
                                            const float2 F[6], const CollideParams& cp,
                                            bool active) {
     unsigned ra[Q], rb[Q];   // only [J] and [J + 1] are used
-    const Quad q0 = slot.get<J>(), q1 = slot.get<J + 1>();
+    const Quad q0 = slot.template get<J>(), q1 = slot.template get<J + 1>();
     ra[J] = q0.a;
     ra[J + 1] = q1.a;
     rb[J] = q0.b;
@@ -694,20 +712,20 @@ __device__ __forceinline__ void relax_quad(typename Store<ST>::T* __restrict__ f
 
 // Forced relaxation of one pair of a quad: the first pair's results go back
 // into the slot, the second's are stored together with them.
-template <int ST, int J, bool SECOND>
+template <int ST, int J, bool SECOND, class Slot>
 __device__ __forceinline__ void relax_half(typename Store<ST>::T* __restrict__ fout, unsigned S,
-                                           unsigned site0, const QuadSlot& slot,
+                                           unsigned site0, const Slot& slot,
                                            const PairState& p, const float2* F,
                                            const CollideParams& cp, bool active) {
     unsigned r[Q];   // only [J] and [J + 1] are used
-    const Quad q0 = slot.get<J>(), q1 = slot.get<J + 1>();
+    const Quad q0 = slot.template get<J>(), q1 = slot.template get<J + 1>();
     r[J] = SECOND ? q0.b : q0.a;
     r[J + 1] = SECOND ? q1.b : q1.a;
     PackedPair<ST> v;
     relax_pair2<ST, J, true>(v, r, p.k, p.ux, p.uy, p.uz, F[0], F[1], F[2], p.uF, cp);
     if (!SECOND) {
-        slot.put_a<J>(v.v[0]);
-        slot.put_a<J + 1>(v.v[1]);
+        slot.template put_a<J>(v.v[0]);
+        slot.template put_a<J + 1>(v.v[1]);
     } else if (active) {
         __stcs(reinterpret_cast<uint2*>(fout + ((unsigned)J * S + site0)), make_uint2(q0.a, v.v[0]));
         __stcs(reinterpret_cast<uint2*>(fout + ((unsigned)(J + 1) * S + site0)),
@@ -719,17 +737,17 @@ __device__ __forceinline__ void relax_half(typename Store<ST>::T* __restrict__ f
 // force the two pairs' states fit the registers side by side; with it the raw
 // values are read back (none are held through the force gather) and one pair
 // is finished before the other begins.
-template <int ST, bool FORCED>
+template <int ST, bool FORCED, class Slot>
 __device__ __forceinline__ void collide_quad(typename Store<ST>::T* __restrict__ fout, unsigned S,
                                              unsigned site0, const unsigned A[Q],
-                                             const unsigned B[Q], const QuadSlot& slot,
+                                             const unsigned B[Q], const Slot& slot,
                                              const float2 F[6], const CollideParams& cp,
                                              int* flag, bool active) {
     const float2 om1 = f2(1.0f - cp.omega);
     if (!FORCED) {
         const PairState pa = pair_state<ST, false>(A, F[0], F[1], F[2], cp, flag, active);
         const PairState pb = pair_state<ST, false>(B, F[3], F[4], F[5], cp, flag, active);
-        const Quad q = slot.get<0>();
+        const Quad q = slot.template get<0>();
         if (active)
             __stcs(reinterpret_cast<uint2*>(fout + site0),
                    make_uint2(Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(q.a), pa.rest)),
@@ -743,17 +761,17 @@ __device__ __forceinline__ void collide_quad(typename Store<ST>::T* __restrict__
 #define LBM_RH(J, N) relax_half<ST, J, N>(fout, S, site0, slot, p, F + 3 * N, cp, active)
     {
         unsigned v[Q];
-        slot.get_all<0>(v);
+        slot.template get_all<0>(v);
         const PairState p = pair_state<ST, true>(v, F[0], F[1], F[2], cp, flag, active);
-        slot.put_a<0>(Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(slot.get<0>().a), p.rest)));
+        slot.template put_a<0>(Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(slot.template get<0>().a), p.rest)));
         LBM_RH(1, 0); LBM_RH(3, 0); LBM_RH(5, 0); LBM_RH(7, 0); LBM_RH(9, 0);
         LBM_RH(11, 0); LBM_RH(13, 0); LBM_RH(15, 0); LBM_RH(17, 0);
     }
     {
         unsigned v[Q];
-        slot.get_all<1>(v);
+        slot.template get_all<1>(v);
         const PairState p = pair_state<ST, true>(v, F[3], F[4], F[5], cp, flag, active);
-        const Quad q = slot.get<0>();
+        const Quad q = slot.template get<0>();
         if (active)
             __stcs(reinterpret_cast<uint2*>(fout + site0),
                    make_uint2(q.a, Raw2<ST>::pack(fma2(om1, Raw2<ST>::widen(q.b), p.rest))));
@@ -763,12 +781,14 @@ __device__ __forceinline__ void collide_quad(typename Store<ST>::T* __restrict__
 #undef LBM_RH
 }
 
-// The slot of this thread in s_raw[Q][QUAD_THREADS], filled with its raw values.
-__device__ __forceinline__ QuadSlot fill_slot(uint2* s_raw, const unsigned A[Q],
-                                              const unsigned B[Q]) {
+// The slot of this thread in s_raw[Q][threads of the CTA], filled with its raw
+// values.
+template <int PZV>
+__device__ __forceinline__ QuadSlot<PZV> fill_slot(uint2* s_raw, const unsigned A[Q],
+                                                   const unsigned B[Q]) {
     const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
-    const QuadSlot slot{(unsigned)__cvta_generic_to_shared(s_raw + tid)};
-#define LBM_SP(J) slot.put<J>(A[J], B[J])
+    const QuadSlot<PZV> slot{(unsigned)__cvta_generic_to_shared(s_raw + tid)};
+#define LBM_SP(J) slot.template put<J>(A[J], B[J])
     LBM_SP(0); LBM_SP(1); LBM_SP(2); LBM_SP(3); LBM_SP(4); LBM_SP(5); LBM_SP(6);
     LBM_SP(7); LBM_SP(8); LBM_SP(9); LBM_SP(10); LBM_SP(11); LBM_SP(12); LBM_SP(13);
     LBM_SP(14); LBM_SP(15); LBM_SP(16); LBM_SP(17); LBM_SP(18);
@@ -777,24 +797,40 @@ __device__ __forceinline__ QuadSlot fill_slot(uint2* s_raw, const unsigned A[Q],
 }
 
 // Eq. 21 of a tile with long lists, as gather_force_tab (same products and
-// order) over the whole tile, in two parts per chunk of FORCE_CHUNK listed
-// bubbles.  The first stages the records and tabulates their per-axis weights
-// over the tile (every thread of the CTA calls it; the caller synchronises).
+// order) over the whole tile, in three parts per chunk of FORCE_CHUNK listed
+// bubbles.  The first stages the records, straight into shared memory: for
+// the first chunk it runs between the population loads and their use, so that
+// its chain of dependent loads (list start, ids, records) hides behind theirs.
 constexpr int QUAD_NAX = TX + TY + TZ;   // x: [0, TX), y: [TX, TX + TY), z: the rest
 static_assert(FORCE_CHUNK == 32 && QX * TY == 32, "a lane per staged bubble, a warp per plane");
 
-__device__ __forceinline__ void quad_force_tables(const Geo& g, const int* __restrict__ items,
-                                                  const BubbleRec* __restrict__ recs, int nb,
-                                                  int c0, int cnt, int bx, int by, int bz,
-                                                  bool point, BubbleRec* srec,
+__device__ __forceinline__ void quad_force_stage(const int* __restrict__ items,
+                                                 const BubbleRec* __restrict__ recs, int nb,
+                                                 int c0, int cnt, BubbleRec* srec) {
+    const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
+    if (tid < cnt) {
+        const int id = __ldcg(items + c0 + tid);
+        if (id >= 0 && id < nb) {
+            const unsigned to = (unsigned)__cvta_generic_to_shared(srec + tid);
+            const char* from = reinterpret_cast<const char*>(recs + id);
+#pragma unroll
+            for (int k = 0; k < (int)sizeof(BubbleRec); k += 16)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + k),
+                             "l"(from + k) : "memory");
+        } else {
+            srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        }
+    }
+}
+
+// The second tabulates their per-axis weights over the tile.  Every thread of
+// the CTA calls it; the caller synchronises after it.
+__device__ __forceinline__ void quad_force_tables(const Geo& g, int cnt, int bx, int by, int bz,
+                                                  bool point, const BubbleRec* srec,
                                                   float (*s_w)[QUAD_NAX]) {
     const int tid = (threadIdx.z * TY + threadIdx.y) * QX + threadIdx.x;
     const int xb0 = bx * TX, yb0 = by * TY, zb0 = bz * TZ;
-    if (tid < cnt) {
-        const int id = __ldcg(items + c0 + tid);
-        if (id >= 0 && id < nb) srec[tid] = load_rec(recs + id);
-        else srec[tid] = BubbleRec{0, 0, 0, 0, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     auto tabulate = [&](auto mode) {
         constexpr int PM = decltype(mode)::value;
@@ -814,7 +850,7 @@ __device__ __forceinline__ void quad_force_tables(const Geo& g, const int* __res
     else tabulate(MapMode<MAP_CELL>{});
 }
 
-// The second adds the chunk to the force F on the thread's quad.  A warp is
+// The third adds the chunk to the force F on the thread's quad.  A warp is
 // one z-plane, so it visits only the bubbles whose z weight there is not zero.
 __device__ __forceinline__ void quad_force_add(int cnt, const BubbleRec* srec,
                                                const float (*s_w)[QUAD_NAX], float2 F[6]) {
@@ -839,8 +875,9 @@ __device__ __forceinline__ void quad_force_add(int cnt, const BubbleRec* srec,
     }
 }
 
-// One CTA's tile of the sweep (sweep_block with four nodes per thread).
-template <int ST, bool TAB>
+// One CTA's block of the sweep (sweep_block with four nodes per thread): 32 x 4
+// nodes of PZV planes, a whole tile at PZV = 4.
+template <int ST, bool TAB, int PZV = QUAD_PZ>
 __device__ __forceinline__ void quad_block(const typename Store<ST>::T* __restrict__ fin,
                                            typename Store<ST>::T* __restrict__ fout,
                                            const Geo& g, const CollideParams& cp,
@@ -851,22 +888,23 @@ __device__ __forceinline__ void quad_block(const typename Store<ST>::T* __restri
                                            int* __restrict__ flag, int bx, int by, int bz,
                                            BubbleRec* srec, const unsigned* safe,
                                            unsigned epoch, bool lead) {
-    __shared__ uint2 s_raw[Q * QUAD_THREADS];
+    static_assert(TZ % PZV == 0 && (!TAB || PZV == QUAD_PZ), "a block lies in one tile layer");
+    __shared__ uint2 s_raw[Q * QX * TY * PZV];
     const int x0 = bx * TX + 4 * threadIdx.x;
     const int y = by * TY + threadIdx.y;
-    const int z = bz * QUAD_PZ + threadIdx.z;
+    const int z = bz * PZV + threadIdx.z;
     const bool active = (x0 < g.nx) && (y < g.ny) && (z < g.nz);
     // Inactive threads gather at a valid node and store nothing.
     const int xa = active ? x0 : 0;
     const int ya = min(y, g.ny - 1), za = min(z, g.nz - 1);
-    const int t = (bz * g.nty + by) * g.ntx + bx;
+    const int t = (((bz * PZV) / TZ) * g.nty + by) * g.ntx + bx;
     // The order of the tile count, the population loads and the wait for an
     // overlapped update is sweep_block's.
     int n_t = 0;
     bool skip = false;
     if (tile_count != nullptr) {
         if (safe == nullptr) n_t = __ldcg(tile_count + t);
-        else skip = !lead && __ldcg(safe + bz) == epoch;
+        else skip = !lead && __ldcg(safe + (bz * PZV) / TZ) == epoch;
     }
     unsigned A[Q], B[Q];
     gather_quad<ST>(fin, g, xa, ya, za, A, B);
@@ -875,18 +913,25 @@ __device__ __forceinline__ void quad_block(const typename Store<ST>::T* __restri
         n_t = __ldcg(tile_count + t);
     }
     __shared__ __align__(16) float s_w[TAB ? FORCE_CHUNK : 1][QUAD_NAX];
-    const QuadSlot slot = fill_slot(s_raw, A, B);
+    int beg = 0, end = 0;
+    if (n_t > 0) {   // uniform over the CTA (one tile)
+        beg = __ldcg(tile_start + t);
+        end = min(beg + n_t, cap);
+        if (TAB) quad_force_stage(items, recs, nb, beg, min(FORCE_CHUNK, end - beg), srec);
+    }
+    const QuadSlot<PZV> slot = fill_slot<PZV>(s_raw, A, B);
     const unsigned S = (unsigned)g.S;
     const unsigned site0 = (unsigned)site_index(g, xa, ya, za);
     float2 F[6] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
-    if (n_t > 0) {   // uniform over the CTA (one tile)
-        const int beg = __ldcg(tile_start + t);
-        const int end = min(beg + n_t, cap);
+    if (n_t > 0) {
         if (TAB) {
             for (int c0 = beg; c0 < end; c0 += FORCE_CHUNK) {
                 const int cnt = min(FORCE_CHUNK, end - c0);
-                __syncthreads();
-                quad_force_tables(g, items, recs, nb, c0, cnt, bx, by, bz, cp.point != 0, srec, s_w);
+                if (c0 > beg) {
+                    __syncthreads();   // the chunk before is done with
+                    quad_force_stage(items, recs, nb, c0, cnt, srec);
+                }
+                quad_force_tables(g, cnt, bx, by, bz, cp.point != 0, srec, s_w);
                 __syncthreads();
                 quad_force_add(cnt, srec, s_w, F);
             }
@@ -930,7 +975,7 @@ __device__ __forceinline__ void quad_block_free(const typename Store<ST>::T* __r
     unsigned A[Q], B[Q];
     gather_quad<ST>(fin, g, xa, ya, za, A, B);
     const float2 F[6] = {f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f), f2(0.0f)};
-    const QuadSlot slot = fill_slot(s_raw, A, B);
+    const QuadSlot<QUAD_PZ> slot = fill_slot<QUAD_PZ>(s_raw, A, B);
     collide_quad<ST, false>(fout, (unsigned)g.S, (unsigned)site_index(g, xa, ya, za), A, B, slot,
                             F, cp, flag, active);
 }
@@ -944,7 +989,7 @@ k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
                       const int* tile_start, const int* tile_count, const int* items, int cap,
                       const BubbleRec* recs, int nb, int* __restrict__ flag,
                       const unsigned* safe, unsigned epoch, const int* zperm, ZSpan zs) {
-    __shared__ BubbleRec srec[FORCE_CHUNK];
+    __shared__ __align__(16) BubbleRec srec[FORCE_CHUNK];
     // The next bubble update may be scheduled once every CTA of the sweep has
     // started; it waits for the sweep to complete before it reads anything.
     pdl_trigger();
@@ -1002,8 +1047,11 @@ k_collide_stream_free(const typename Store<ST>::T* __restrict__ fin,
 // ---------------------------------------------------------------------------
 constexpr int MAX_BATCH_COLUMNS = 256;
 
-template <int ST, int PZV>
-__global__ void __launch_bounds__(PX * TY * PZV, PairOccupancy<ST>::kMinBlocks * PZ / PZV)
+// NODES: nodes per thread along x, as the single sweep's (four where every
+// column's rows are a multiple of 4 of 16-bit values).
+template <int ST, int PZV, int NODES>
+__global__ void __launch_bounds__(SweepShape<ST, NODES>::kThreads / SweepShape<ST, NODES>::kPlanes * PZV,
+                                  SweepShape<ST, NODES>::kMinBlocks * SweepShape<ST, NODES>::kPlanes / PZV)
 k_collide_batch(const typename Store<ST>::T* __restrict__ fin,
                 typename Store<ST>::T* __restrict__ fout, const BatchColumn* __restrict__ cols,
                 int ncols, int total_items, int depth, int* __restrict__ work_counter,
@@ -1013,8 +1061,8 @@ k_collide_batch(const typename Store<ST>::T* __restrict__ fin,
     __shared__ BubbleRec srec[FORCE_CHUNK];
     __shared__ int s_item_base[MAX_BATCH_COLUMNS + 1];
     __shared__ int s_item;
-    const int tid = (threadIdx.z * TY + threadIdx.y) * PX + threadIdx.x;
-    for (int c = tid; c <= ncols; c += PX * TY * PZV)
+    const int tid = (threadIdx.z * TY + threadIdx.y) * (TX / NODES) + threadIdx.x;
+    for (int c = tid; c <= ncols; c += TX / NODES * TY * PZV)
         s_item_base[c] = c < ncols ? cols[c].item_base : total_items;
     for (;;) {
         __syncthreads();
@@ -1035,22 +1083,52 @@ k_collide_batch(const typename Store<ST>::T* __restrict__ fin,
         const int by = rest % col.g.nty;
         const int bz0 = (rest / col.g.nty) * depth;
         const int nbz = (col.g.nz + PZV - 1) / PZV;
-        for (int bz = bz0; bz < min(bz0 + depth, nbz); ++bz)
-            sweep_block<ST, false, PZV>(fin + col.pop_offset, fout + col.pop_offset, col.g, col.cp,
-                            tile_start + col.tile_base, tile_count + col.tile_base, items, cap,
-                            recs, nb, flag, bx, by, bz, srec);
+        // No lists (no two-way coupling): null stays null.
+        const int* const start = tile_start ? tile_start + col.tile_base : nullptr;
+        const int* const count = tile_count ? tile_count + col.tile_base : nullptr;
+        for (int bz = bz0; bz < min(bz0 + depth, nbz); ++bz) {
+            if constexpr (NODES == 4)
+                quad_block<ST, false, PZV>(fin + col.pop_offset, fout + col.pop_offset, col.g,
+                                           col.cp, start, count, items, cap, recs, nb, flag, bx, by,
+                                           bz, srec, nullptr, 0, false);
+            else
+                sweep_block<ST, false, PZV>(fin + col.pop_offset, fout + col.pop_offset, col.g,
+                                            col.cp, start, count, items, cap, recs, nb, flag, bx,
+                                            by, bz, srec);
+        }
     }
 }
 
 cudaError_t launch_collide_batch(int storage, const void* fin, void* fout,
                                  const BatchColumn* cols, int ncols, int total_items, int depth,
-                                 int grid, int planes, int* work_counter, const TileLists& tl,
-                                 const BubbleRec* recs, int nb, int* flag, cudaStream_t st) {
+                                 int grid, int planes, bool quad, int* work_counter,
+                                 const TileLists& tl, const BubbleRec* recs, int nb, int* flag,
+                                 cudaStream_t st) {
     if (ncols > MAX_BATCH_COLUMNS) return cudaErrorInvalidValue;
+    if (quad && storage != 0) {
+        switch (storage * 8 + planes) {
+#define LBM_LAUNCH_BATCH4(SI, PV, T)                                                              \
+    case SI * 8 + PV:                                                                             \
+        k_collide_batch<SI, PV, 4><<<grid, dim3(QX, TY, PV), 0, st>>>(                            \
+            (const T*)fin, (T*)fout, cols, ncols, total_items, depth, work_counter, tl.start,    \
+            tl.count, tl.items, tl.cap, recs, nb, flag);                                         \
+        break;
+            LBM_LAUNCH_BATCH4(1, 1, __half)
+            LBM_LAUNCH_BATCH4(1, 2, __half)
+            LBM_LAUNCH_BATCH4(1, 4, __half)
+            LBM_LAUNCH_BATCH4(2, 1, __nv_bfloat16)
+            LBM_LAUNCH_BATCH4(2, 2, __nv_bfloat16)
+            LBM_LAUNCH_BATCH4(2, 4, __nv_bfloat16)
+#undef LBM_LAUNCH_BATCH4
+            default:
+                return cudaErrorInvalidValue;
+        }
+        return cudaGetLastError();
+    }
     switch (storage * 8 + planes) {
 #define LBM_LAUNCH_BATCH(SI, PV, T)                                                               \
     case SI * 8 + PV:                                                                             \
-        k_collide_batch<SI, PV><<<grid, dim3(PX, TY, PV), 0, st>>>(                               \
+        k_collide_batch<SI, PV, 2><<<grid, dim3(PX, TY, PV), 0, st>>>(                            \
             (const T*)fin, (T*)fout, cols, ncols, total_items, depth, work_counter, tl.start,    \
             tl.count, tl.items, tl.cap, recs, nb, flag);                                         \
         break;
@@ -1075,9 +1153,10 @@ int sweep_planes(int storage, int nx, const void* fa, const void* fb) {
     // bytes at a time.
     const bool quad = storage != 0 && (nx & 3) == 0 && ((uintptr_t)fa & 7) == 0 &&
                       ((uintptr_t)fb & 7) == 0;
-    return quad ? QUAD_PZ : PZ;
+    return (nx & 1) ? ODD_PZ : (quad ? QUAD_PZ : PZ);
 }
-int batch_min_blocks(int storage, int planes) {
+int batch_min_blocks(int storage, int planes, bool quad) {
+    if (quad) return SweepShape<1, 4>::kMinBlocks * QUAD_PZ / planes;
     const int k = storage == 0 ? PairOccupancy<0>::kMinBlocks : PairOccupancy<1>::kMinBlocks;
     return k * PZ / planes;
 }
@@ -1093,8 +1172,8 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
     const int cap = tl ? tl->cap : 0;
     if (overlap && (safe == nullptr || tl == nullptr)) return cudaErrorInvalidValue;
     if (!overlap) safe = nullptr;
-    const bool quad = sweep_planes(storage, g.nx, fin, fout) == QUAD_PZ;
-    const int planes = quad ? QUAD_PZ : PZ;
+    const int planes = sweep_planes(storage, g.nx, fin, fout);
+    const bool quad = planes == QUAD_PZ;
     const int nbz = (g.nz + planes - 1) / planes;
     ZSpan zs{0, nbz, INT_MAX, 0};
     if (span) {
@@ -1173,25 +1252,29 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
                 return cudaErrorInvalidValue;
         }
     }
-    if (overlap) return cudaErrorInvalidValue;   // odd rows: plain stream order only
-    dim3 block(TX, TY, 1);
-    dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, g.nz);
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(TX, TY, 1);
+    cfg.gridDim = dim3((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (unsigned)nbz);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
     switch (storage) {
         case 0:
-            k_collide_stream<0><<<grid, block, 0, st>>>((const float*)fin, (float*)fout, g, cp,
-                                                        start, count, items, cap, recs, nb, flag);
-            break;
+            return cudaLaunchKernelEx(&cfg, k_collide_stream<0>, (const float*)fin, (float*)fout, g,
+                                      cp, start, count, items, cap, recs, nb, flag, safe, epoch,
+                                      zperm);
         case 1:
-            k_collide_stream<1><<<grid, block, 0, st>>>((const __half*)fin, (__half*)fout, g, cp,
-                                                        start, count, items, cap, recs, nb, flag);
-            break;
+            return cudaLaunchKernelEx(&cfg, k_collide_stream<1>, (const __half*)fin, (__half*)fout,
+                                      g, cp, start, count, items, cap, recs, nb, flag, safe, epoch,
+                                      zperm);
         default:
-            k_collide_stream<2><<<grid, block, 0, st>>>((const __nv_bfloat16*)fin,
-                                                        (__nv_bfloat16*)fout, g, cp, start, count,
-                                                        items, cap, recs, nb, flag);
-            break;
+            return cudaLaunchKernelEx(&cfg, k_collide_stream<2>, (const __nv_bfloat16*)fin,
+                                      (__nv_bfloat16*)fout, g, cp, start, count, items, cap, recs,
+                                      nb, flag, safe, epoch, zperm);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace lbm

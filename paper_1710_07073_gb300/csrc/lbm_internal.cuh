@@ -358,7 +358,7 @@ cudaError_t launch_bubble_records(const Geo& g, const BubbleDev& b, cudaStream_t
 int swarm_grid(int* sms);   // *sms: the SM count
 int interp_grid(int storage);
 // Planes per z block of the sweep that launch_collide_stream takes for these
-// buffers (even nx): a CTA's planes, within one tile layer.
+// buffers: a CTA's planes, within one tile layer.
 int sweep_planes(int storage, int nx, const void* fa, const void* fb);
 // Kernels launched by one launch_binning call (count, 3-pass scan, fill, sort).
 // Bubbles b with select[b] != 0 are binned; select defaults to b.spread.
@@ -377,8 +377,9 @@ cudaError_t launch_totals(int storage, const void* f, const Geo& g, const Collid
                           double* partials, int npartials, double* out4, cudaStream_t st);
 cudaError_t launch_collide_batch(int storage, const void* fin, void* fout,
                                  const BatchColumn* cols, int ncols, int total_items, int depth,
-                                 int grid, int planes, int* work_counter, const TileLists& tl,
-                                 const BubbleRec* recs, int nb, int* flag, cudaStream_t st);
+                                 int grid, int planes, bool quad, int* work_counter,
+                                 const TileLists& tl, const BubbleRec* recs, int nb, int* flag,
+                                 cudaStream_t st);
 cudaError_t launch_bubbles_batch(int storage, const void* f, const BatchColumn* cols,
                                  const int* bubble_col, const BubbleDev& b, const BubbleConst& bc,
                                  int* flag, const SmallBins& sb, cudaStream_t st);
@@ -387,7 +388,8 @@ cudaError_t launch_bubble_constants_batch(const BubbleDev& b, const BubbleConst&
                                           cudaStream_t st);
 // Resident CTAs per SM the batch sweep is compiled for, with `planes` z-planes
 // per CTA (1, 2 or 4; the same threads per SM for each).
-int batch_min_blocks(int storage, int planes);
+// `quad`: four nodes per thread (sweep_planes' rule for every column).
+int batch_min_blocks(int storage, int planes, bool quad);
 int totals_partials(const Geo& g);
 constexpr int TOTALS_PARTIALS_MAX = 304;   // totals_partials' largest value
 int scan_blocks(int T);
