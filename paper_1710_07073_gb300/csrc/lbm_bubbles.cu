@@ -1406,12 +1406,14 @@ constexpr int INTERP_CHUNK = 32;              // listed bubbles per pass
 constexpr int INTERP_ROWS = TY * TZ;          // (y, z) rows of a tile: 16
 static_assert(INTERP_THREADS % INTERP_ROWS == 0 && TX == 32 && TY == 4 && TZ == 4,
               "tile shape of the interpolation: a lane per column");
-// Resident CTAs per SM the interpolation is compiled for: 16-bit storage on
-// even rows at 5 (48 registers; its swarm step ran 1 % shorter than at 4, at
-// 6 longer); FP32 at 4 (at 5 it spills 96 bytes and its step was longer), as
-// odd rows (whose two-node gather spills 172 bytes at 48 registers).
+// Resident CTAs per SM the interpolation is compiled for, and whether it loads
+// a tile's rows a tile ahead (kPipe): with 16-bit storage on even rows the 19
+// packed rows fit beside the tables and sums at 64 registers, and the
+// 384x384x768 swarm's FP16 step took 1.910 ms against 1.923 at 5 CTAs (48
+// registers) without; FP32's 38 do not (3 CTAs: 3.068 ms against 3.036).
 template <int ST, bool PAIR> struct InterpOccupancy {
-    static constexpr int kMinBlocks = (ST != 0 && PAIR) ? 5 : 4;
+    static constexpr bool kPipe = PAIR && ST != 0;
+    static constexpr int kMinBlocks = 4;
 };
 
 // The list head of a covered tile: its list range [beg, end) and this
@@ -1421,6 +1423,19 @@ template <int ST, bool PAIR> struct InterpOccupancy {
 struct TileHead {
     int t, beg, end, id;
 };
+
+// The rows of this thread's pair in tile t (even nx): thread (px, y, z) holds
+// the x-pair (2 px, 2 px + 1) of row (y, z).
+template <int ST>
+__device__ __forceinline__ void interp_rows(const typename Store<ST>::T* __restrict__ f,
+                                            const Geo& g, int t, typename Raw2<ST>::T (&rp)[Q]) {
+    const int tid = threadIdx.x;
+    const int x = (t % g.ntx) * TX + 2 * (tid % (TX / 2));
+    const int y = (t / g.ntx) % g.nty * TY + (tid / (TX / 2)) % TY;
+    const int z = t / (g.ntx * g.nty) * TZ + tid / ((TX / 2) * TY);
+    const bool in = x < g.nx && y < g.ny && z < g.nz;
+    gather_pair<ST>(f, g, in ? x : 0, in ? y : 0, in ? z : 0, rp);
+}
 
 // One covered tile h.t: the Eq. 10 velocity of its nodes, then for each listed
 // bubble the part of its Eq. 20 sum over the tile, written at the bubble's
@@ -1433,7 +1448,9 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
                                             const TileHead& h, TileHead& next,
                                             const int* __restrict__ items,
                                             const BubbleRec* __restrict__ recs, int nb,
-                                            float* __restrict__ partial) {
+                                            float* __restrict__ partial,
+                                            typename Raw2<ST>::T (&rp)[PAIR ? Q : 1]) {
+    constexpr bool PIPE = InterpOccupancy<ST, PAIR>::kPipe;
     const int t = h.t;
     constexpr int NAX = TX + TY + TZ;
     __shared__ float s_u[3][INTERP_ROWS][TX + 1];   // node velocities by (z, y) row, padded
@@ -1454,12 +1471,10 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
     const bool inxy = x < g.nx && y < g.ny;
     const bool ina = inxy && za < g.nz, inb = inxy && zb < g.nz;
     const int ppx = tid % (TX / 2), py2 = (tid / (TX / 2)) % TY, pz2 = tid / ((TX / 2) * TY);
-    const int px0 = xb0 + 2 * ppx, pyy = yb0 + py2, pzz = zb0 + pz2;
-    const bool inp = px0 < g.nx && pyy < g.ny && pzz < g.nz;
+    const bool inp = xb0 + 2 * ppx < g.nx && yb0 + py2 < g.ny && zb0 + pz2 < g.nz;
     typename Store<ST>::T ra[PAIR ? 1 : Q], rb[PAIR ? 1 : Q];
-    typename Raw2<ST>::T rp[PAIR ? Q : 1];
     if (PAIR) {
-        gather_pair<ST>(f, g, inp ? px0 : 0, inp ? pyy : 0, inp ? pzz : 0, rp);
+        if constexpr (PAIR && !PIPE) interp_rows<ST>(f, g, t, rp);
     } else {
         gather_issue<ST>(f, g, ina ? x : 0, ina ? y : 0, ina ? za : 0, ra);
         gather_issue<ST>(f, g, inb ? x : 0, inb ? y : 0, inb ? zb : 0, rb);
@@ -1479,6 +1494,9 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
         s_u[1][row][2 * ppx + 1] = inp ? jy.y * ra1 : 0.0f;
         s_u[2][row][2 * ppx] = inp ? jz.x * ra0 : 0.0f;
         s_u[2][row][2 * ppx + 1] = inp ? jz.y * ra1 : 0.0f;
+        // The next tile's rows arrive during this tile's tables and sums.
+        if constexpr (PIPE)
+            if (next.t >= 0) interp_rows<ST>(f, g, next.t, rp);
     } else {
         // Eq. 10 velocity of the tile's nodes (zero for nodes beyond the box).
         float gv[Q], u[3];
@@ -1648,6 +1666,8 @@ k_tile_interp(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams 
     TileHead h = head(__ldcg(cover + i));
     if (threadIdx.x < min(INTERP_CHUNK, h.end - h.beg)) h.id = __ldcg(items + h.beg + threadIdx.x);
     int tn = i + step < ntiles ? __ldcg(cover + i + step) : -1;
+    typename Raw2<ST>::T rp[PAIR ? Q : 1];
+    if constexpr (InterpOccupancy<ST, PAIR>::kPipe) interp_rows<ST>(f, g, h.t, rp);
     for (; i < ntiles; i += step) {
         // The next tile's count and offset go out now; its first list entry
         // during this tile; the index of the tile after it.
@@ -1655,7 +1675,7 @@ k_tile_interp(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams 
         const int tnn = i + 2 * step < ntiles ? __ldcg(cover + i + 2 * step) : -1;
         if (i + step >= ntiles) pdl_trigger();   // this CTA's last tile
         __syncthreads();   // the shared tables of the previous tile are done with
-        tile_interp<ST, PAIR, LIFT>(f, g, cp, h, next, items, recs, nb, partial);
+        tile_interp<ST, PAIR, LIFT>(f, g, cp, h, next, items, recs, nb, partial, rp);
         h = next;
         tn = tnn;
     }
