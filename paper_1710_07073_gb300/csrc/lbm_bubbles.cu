@@ -80,7 +80,7 @@ __device__ __noinline__ float axis_norm_point(int anc, float fr, float inv_n, fl
     for (int k = -K; k <= K; ++k) {
         const int c = anc + k;
         if (!periodic && (c < 0 || c >= L)) continue;
-        sum += cell_poly(((float)k + 0.5f - fr) * inv_n, h);
+        sum += cell_poly<MAP_POINT>(((float)k + 0.5f - fr) * inv_n, h);
     }
     return sum;
 }
