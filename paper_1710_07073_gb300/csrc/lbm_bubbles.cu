@@ -2298,9 +2298,12 @@ __global__ void k_set_feq(const double* __restrict__ rho, const double* __restri
 // direction over its sites as hi + lo, two floats (Neumaier's compensated
 // summation: TwoSum, the rounding errors collected in lo), 7 FP32 operations
 // per value, and only the per-thread sums go through FP64.  The error is that
-// of about 48 bits against the sum of magnitudes.  lbm_get_totals before and
-// after: 7.01 -> 0.77 ms on 256 x 256 x 512 in FP16, 0.54 -> 0.063 ms on
-// 64 x 64 x 128, 0.101 -> 0.045 ms on 32 x 32 x 64.
+// of about 48 bits against the sum of magnitudes.  On even rows a thread takes
+// an x-pair by aligned row loads and sums its two nodes in packed FP32, half
+// the instructions (odd rows: two sites at a time).  lbm_get_totals in FP64, by
+// scalar sums and by packed ones: 7.01, 0.76, 0.44 ms on 256 x 256 x 512 in
+// FP32 (the reads take 0.38) and 0.43 in FP16; 2.42 and 1.37 ms by scalar and
+// packed sums on 384 x 384 x 768.
 constexpr int TOT_BLOCK = 256;
 // Resident CTAs per SM the kernel is compiled for, and the grid: whole waves
 // of 152 SMs.
@@ -2328,21 +2331,25 @@ __device__ double block_sum(double v, double* sh) {
 
 // The same sums of one thread's sites in FP64: for values whose FP32 sums are
 // not finite (infinities, NaN, sums beyond FP32).
-template <int ST>
+template <int ST, bool PAIR>
 __device__ __noinline__ void totals_fp64(const typename Store<ST>::T* __restrict__ f,
                                          const Geo& g, const CollideParams& cp, unsigned s,
                                          unsigned stride, double acc[4]) {
     for (int k = 0; k < 4; ++k) acc[k] = 0.0;
-    for (; s < (unsigned)g.S; s += stride) {
-        int x, y, z;
-        site_coords(g, s, x, y, z);
-        float gv[Q];
-        gather<ST>(f, g, cp, x, y, z, gv);
-        for (int j = 0; j < Q; ++j) {
-            acc[0] += gv[j];
-            acc[1] += cx(j) * (double)gv[j];
-            acc[2] += cy(j) * (double)gv[j];
-            acc[3] += cz(j) * (double)gv[j];
+    // PAIR: s counts pairs of sites.
+    constexpr unsigned M = PAIR ? 2u : 1u;
+    for (; s < (unsigned)g.S / M; s += stride) {
+        for (unsigned k = 0; k < M; ++k) {
+            int x, y, z;
+            site_coords(g, s * M + k, x, y, z);
+            float gv[Q];
+            gather<ST>(f, g, cp, x, y, z, gv);
+            for (int j = 0; j < Q; ++j) {
+                acc[0] += gv[j];
+                acc[1] += cx(j) * (double)gv[j];
+                acc[2] += cy(j) * (double)gv[j];
+                acc[3] += cz(j) * (double)gv[j];
+            }
         }
     }
 }
@@ -2356,7 +2363,39 @@ __device__ __forceinline__ F2 two_sum_rn(float a, float b) {
     return F2{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
 }
 
+// The same on an x-pair's two nodes at once (packed FP32).
+__device__ __forceinline__ void two_sum_pair(float2& h, float2& l, float2 v) {
+    const float2 s = add2(h, v);
+    const float2 bb = sub2(s, h);
+    l = add2(l, add2(sub2(h, sub2(s, bb)), sub2(v, bb)));
+    h = s;
+}
+
+// Even rows: an x-pair per thread and pass, aligned row loads and packed sums.
 template <int ST>
+__device__ __forceinline__ void totals_pairs(const typename Store<ST>::T* __restrict__ f,
+                                             const Geo& g, const CollideParams& cp, F2 dir[Q]) {
+    float2 h[Q], l[Q];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) h[j] = l[j] = f2(0.0f);
+    const unsigned half = (unsigned)g.nx / 2u, n = (unsigned)g.S / 2u;
+    for (unsigned p = blockIdx.x * TOT_BLOCK + threadIdx.x; p < n; p += gridDim.x * TOT_BLOCK) {
+        const unsigned xy = p / half;
+        typename Raw2<ST>::T rv[Q];
+        gather_pair<ST>(f, g, 2 * (int)(p - xy * half), (int)(xy % (unsigned)g.ny),
+                        (int)(xy / (unsigned)g.ny), rv);
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            float2 v = Raw2<ST>::widen(rv[j]);
+            if (Store<ST>::kScaled) v = mul2(v, f2(wf(j) * cp.inv_scale));
+            two_sum_pair(h[j], l[j], v);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < Q; ++j) dir[j] = f2_add(F2{h[j].x, l[j].x}, h[j].y, l[j].y);
+}
+
+template <int ST, bool PAIR>
 __global__ void __launch_bounds__(TOT_BLOCK, TOT_PER_SM)
 k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, double* partials) {
     __shared__ double sh[32];
@@ -2365,9 +2404,10 @@ k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, d
     for (int j = 0; j < Q; ++j) dir[j] = F2{0.0f, 0.0f};
     const unsigned S = (unsigned)g.S, stride = gridDim.x * TOT_BLOCK;   // 19 S < 2^32
     const unsigned s0 = blockIdx.x * TOT_BLOCK + threadIdx.x;
-    // Two sites at a time, the loads of both issued first (two_sum with zero
-    // changes nothing).
-    for (unsigned s = s0; s < S; s += 2 * stride) {
+    if constexpr (PAIR) totals_pairs<ST>(f, g, cp, dir);
+    // Odd rows: two sites at a time, the loads of both issued first (two_sum
+    // with zero changes nothing).
+    for (unsigned s = PAIR ? S : s0; s < S; s += 2 * stride) {
         const bool two = s + stride < S;
         int x, y, z, x2, y2, z2;
         site_coords(g, s, x, y, z);
@@ -2401,7 +2441,7 @@ k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, d
         acc[k] = f2_to(m[k]);
         finite = finite && isfinite(m[k].h) && isfinite(m[k].l);
     }
-    if (!finite) totals_fp64<ST>(f, g, cp, s0, stride, acc);
+    if (!finite) totals_fp64<ST, PAIR>(f, g, cp, s0, stride, acc);
     for (int k = 0; k < 4; ++k) {
         const double t = block_sum(acc[k], sh);
         if (threadIdx.x == 0) partials[4 * blockIdx.x + k] = t;
@@ -2470,11 +2510,21 @@ cudaError_t launch_set_equilibrium(int storage, const double* rho, const double*
 
 cudaError_t launch_totals(int storage, const void* f, const Geo& g, const CollideParams& cp,
                           double* partials, int npartials, double* out4, cudaStream_t st) {
-    switch (storage) {
-        case 0: k_totals<0><<<npartials, TOT_BLOCK, 0, st>>>((const float*)f, g, cp, partials); break;
-        case 1: k_totals<1><<<npartials, TOT_BLOCK, 0, st>>>((const __half*)f, g, cp, partials); break;
+    const bool pair = (g.nx & 1) == 0;
+    switch (storage * 2 + (pair ? 1 : 0)) {
+#define LBM_TOTALS(SI, PR, T)                                                                  \
+    case SI * 2 + PR:                                                                          \
+        k_totals<SI, PR><<<npartials, TOT_BLOCK, 0, st>>>((const T*)f, g, cp, partials);       \
+        break;
+        LBM_TOTALS(0, 0, float)
+        LBM_TOTALS(0, 1, float)
+        LBM_TOTALS(1, 0, __half)
+        LBM_TOTALS(1, 1, __half)
+        LBM_TOTALS(2, 0, __nv_bfloat16)
+        LBM_TOTALS(2, 1, __nv_bfloat16)
+#undef LBM_TOTALS
         default:
-            k_totals<2><<<npartials, TOT_BLOCK, 0, st>>>((const __nv_bfloat16*)f, g, cp, partials);
+            return cudaErrorInvalidValue;
     }
     k_totals_final<<<1, TOT_BLOCK, 0, st>>>(partials, npartials, (double)g.S * (double)cp.rho0, out4);
     return cudaGetLastError();

@@ -45,6 +45,13 @@ def test_totals_against_exact_sums(dims, walls, storage, scale):
     col.close()
 
 
+@pytest.mark.parametrize("dims", [(2, 1, 1), (2, 3, 1), (64, 1, 5), (514, 3, 33), (515, 3, 33)])
+@pytest.mark.parametrize("walls", [0x00, 0x3F, 0x7F])
+def test_totals_by_pairs_on_thin_and_long_rows(dims, walls):
+    # Rows of one pair, single rows and planes, and passes that end inside a row.
+    test_totals_against_exact_sums(dims, walls, lbm.LBM_STORE_F32, 1.0)
+
+
 def test_totals_beyond_fp32_and_nan():
     col = _column((20, 12, 8), 0x3F, lbm.LBM_STORE_F32, 1.0)
     f = lbm.lbm_get_populations(col.ctx)
