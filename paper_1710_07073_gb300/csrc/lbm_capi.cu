@@ -233,8 +233,8 @@ int alloc_guard(lbm_ctx* c, unsigned** safe, int** zperm, int* nbz, int** zrange
 
 // Few bubbles: the split pays only where the sweep is long against the
 // step's extra host and stream work (fork, join, read-back, a third launch):
-// on GB300 256x256x512 gains (FP16 step 0.460 -> 0.445 ms), 128x128x256
-// loses (0.102 -> 0.120 s for 1000 forward steps).
+// on GB300 256x256x512 gains (step in FP16 411 -> 392 us, in FP32 757 -> 756),
+// 128x128x256 loses in FP32 (96.2 -> 97.6 us), 64x64x128 more (14.6 -> 24.6).
 #ifndef LBM_FEW_SPLIT_MIN_SITES
 #define LBM_FEW_SPLIT_MIN_SITES (1LL << 24)
 #endif

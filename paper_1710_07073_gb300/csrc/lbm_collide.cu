@@ -584,7 +584,8 @@ __device__ __forceinline__ void sweep_block(const typename Store<ST>::T* __restr
 // (80 registers, no spills without force; 4: 0.410, 5: 0.396, 7: 0.427,
 // 8: 0.476 ms) the 256 x 256 x 512 FP16 step takes 0.391 ms against 0.444 ms
 // with two nodes (96 % of the copy peak), the 384 x 384 x 768 swarm's FP16 step
-// 1.953 against 2.116 ms, its whole listed sweep 1.660 against 1.777 ms.
+// 1.953 against 2.116 ms, its whole listed sweep 1.660 against 1.777 ms (1.647
+// with a tile's first records staged before the rows are used).
 // ---------------------------------------------------------------------------
 constexpr int QX = TX / 4;      // threads along x
 constexpr int QUAD_PZ = TZ;     // z-planes per CTA
