@@ -191,12 +191,15 @@ __device__ __forceinline__ void collide_store(typename Store<ST>::T* __restrict_
 // of the copy peak.  Two planes per thread, all rows loaded first, took 0.122 ms:
 // it is not the loads in flight that bound it but the sectors that unaligned
 // rows share between warps.  Overlapped with the bubble update as the even
-// rows' sweep is (126 us a step before, in stream order).
+// rows' sweep is (126 us a step before, in stream order).  The 16-bit formats,
+// whose loads are half as long, take 10 CTAs per SM (48 registers): a step in
+// FP16 82.6 us against 88.1 at 8 (12: 83.8), 201 x 150 x 300 193 against 199;
+// FP32 loses by it (117.5 us at 10, 115.3 at 6).
 constexpr int ODD_PZ = 1;
 constexpr int ODD_CHUNK = 32;   // bubble records staged per pass
 
 template <int ST>
-__global__ void __launch_bounds__(TX * TY, 8)
+__global__ void __launch_bounds__(TX * TY, ST == 0 ? 8 : 10)
 k_collide_stream(const typename Store<ST>::T* __restrict__ fin,
                  typename Store<ST>::T* __restrict__ fout, Geo g, CollideParams cp,
                  const int* tile_start, const int* tile_count, const int* items, int cap,
