@@ -693,6 +693,8 @@ cudaError_t launch_bubble_constants(const BubbleDev& b, const BubbleConst& bc, c
 
 // Tiles of one axis holding at least one window cell, ascending.
 // lo, hi: the first and last support cell, floor(x - n) and ceil(x + n) - 1.
+// (axis_run gives the same tiles in closed form where a window cannot wrap
+// onto itself.)
 __device__ int axis_tiles(int lo, int hi, int L, bool periodic, int T, int out[MAX_AXIS_TILES]) {
     int cnt = 0;
     if (!periodic) {
@@ -716,40 +718,6 @@ __device__ int axis_tiles(int lo, int hi, int L, bool periodic, int T, int out[M
         out[k + 1] = v;
     }
     return cnt;
-}
-
-// The same tiles of one axis as two runs of consecutive ones, [first, first +
-// n0) then [second, ...), n in all, for a window that does not wrap onto
-// itself (2 n + 2 <= L on a periodic axis, as lbm_set_bubbles ensures): no
-// loops, divisions or arrays.  The update and the binning of one bubble are a
-// single thread's or warp's serial code, run once per launch, so their length
-// is paid in instruction fetches: with axis_tiles the counting of a bubble's
-// tiles took 7,900 cycles of k_swarm_tail.
-struct AxisRun {
-    int first, n0, second, n;
-    __device__ __forceinline__ int tile(int i) const {
-        return i < n0 ? first + i : second + (i - n0);
-    }
-};
-
-template <int T>
-__device__ __forceinline__ AxisRun axis_run(int lo, int hi, int L, bool periodic) {
-    static_assert((T & (T - 1)) == 0, "tiles of a power of two");
-    if (periodic) {
-        if (lo < 0) lo += L;
-        if (hi >= L) hi -= L;
-    } else {
-        lo = max(lo, 0);
-        hi = min(hi, L - 1);
-        if (hi < lo) return AxisRun{0, 0, 0, 0};
-    }
-    const int ts = lo / T, te = hi / T;   // lo, hi >= 0
-    if (lo <= hi) return AxisRun{ts, te - ts + 1, 0, te - ts + 1};
-    // The window wraps: the tiles up to te, then those from ts (all of them
-    // when both ends lie in one tile).
-    const int nt = (L + T - 1) / T;
-    if (te >= ts) return AxisRun{0, nt, 0, nt};
-    return AxisRun{0, te + 1, ts, te + 1 + nt - ts};
 }
 
 // The tiles of a bubble's window (widened by pad), numbered x fastest.
@@ -1780,6 +1748,7 @@ k_swarm_tail(Geo g, BubbleDev B, BubbleConst bc, int* __restrict__ flag, Bins bi
             const TileRuns r = tile_runs(g, x, in.k.nh, in.k.nl, sw.pad);
             count_tiles(g, r, bins.cnt, zlo, zhi);
             nt = r.n;
+            if (nt > sw.per) atomicOr(bins.overflow, 1);   // more tiles than it has slots
         }
         sw.ntile[b] = nt;
     }
@@ -1894,6 +1863,7 @@ k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__
                 const TileRuns r = tile_runs(g, B, b, sw.pad);
                 count_tiles(g, r, bins.cnt, zlo, zhi);
                 n = r.n;
+                if (n > sw.per) atomicOr(bins.overflow, 1);   // more tiles than it has slots
             }
             sw.ntile[b] = n;
         }
@@ -1985,7 +1955,7 @@ k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__
                 int rank = 0;
                 for (int j = 0; j < m; ++j) rank += ids[j] < v;
                 bins.items[beg + rank] = v;
-                sw.slots[(size_t)v * sw.per + min(ks[i], sw.per - 1)] = beg + rank;
+                if (ks[i] < sw.per) sw.slots[(size_t)v * sw.per + ks[i]] = beg + rank;
             }
             __syncwarp();
         } else if (lane == 0) {
@@ -2003,8 +1973,8 @@ k_swarm_bin(Geo g, BubbleDev B, Bins bins, SwarmBins sw, const int* __restrict__
                 sw.kidx[j + 1] = kv;
             }
             for (int i = beg; i < end; ++i) {
-                const int v = __ldcg(bins.items + i);
-                sw.slots[(size_t)v * sw.per + min(__ldcg(sw.kidx + i), sw.per - 1)] = i;
+                const int v = __ldcg(bins.items + i), kv = __ldcg(sw.kidx + i);
+                if (kv < sw.per) sw.slots[(size_t)v * sw.per + kv] = i;
             }
         }
         __syncwarp();

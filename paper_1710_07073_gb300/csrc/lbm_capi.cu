@@ -161,10 +161,12 @@ int check_walls(unsigned walls) {
     return 1;
 }
 
-// Tiles a window of half-width n can touch along an axis of tile size T.
-int axis_tile_bound(double n, int T) {
-    int cells = (int)std::ceil(2.0 * n) + 1;
-    return (cells + T - 1) / T + 1;
+// Tiles a window of half-width n can touch in this column.
+long long window_tile_bound(const lbm_ctx* c, double n) {
+    const int cells = (int)std::ceil(2.0 * n) + 1;
+    return (long long)axis_tile_bound(cells, c->nx, !(c->walls & 0x01), TX) *
+           axis_tile_bound(cells, c->ny, !(c->walls & 0x04), TY) *
+           axis_tile_bound(cells, c->nz, !(c->walls & 0x10), TZ);
 }
 
 void free_bubbles(lbm_ctx* c) {
@@ -787,8 +789,7 @@ int lbm_set_bubbles(lbm_ctx* c, int n, const double* pos3, const double* vel3,
     double dmax = 0.0;
     for (int b = 0; b < n; ++b) dmax = std::fmax(dmax, diam[b]);
     const double hwmax = c->p.width_factor * dmax;
-    const long long per = (long long)axis_tile_bound(hwmax + 1.0, TX) *
-                          axis_tile_bound(hwmax + 1.0, TY) * axis_tile_bound(hwmax + 1.0, TZ);
+    const long long per = window_tile_bound(c, hwmax + 1.0);
     const long long cap = per * n;
     if (cap >= (1LL << 31)) {
         free_bubbles(c);

@@ -15,6 +15,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lbm_tiles.hpp"
+
 namespace lbm {
 
 constexpr int Q = 19;
