@@ -1000,10 +1000,6 @@ __device__ void bin_small_block(const Geo& g, const BubbleDev& B, const SmallBin
     if (tid == 0) *sb.prev_n = n;
 }
 
-__device__ __forceinline__ int floor_div(int a, int b) {
-    return a >= 0 ? a / b : -((-a + b - 1) / b);
-}
-
 // Sweep order of the z blocks for the next step, written by one CTA (every
 // thread calls it): the blocks whose tile layer is not marked in `lay` (bit
 // l: layer l is guarded), ascending, then the guarded ones, ascending.  Each
@@ -1030,37 +1026,21 @@ __device__ void write_zperm(int nbz, int planes, const unsigned* lay, int* __res
 }
 
 // The z tile layers the support of a bubble, widened by GUARD_CELLS cells,
-// reaches: [l0, l1], to be wrapped on a periodic axis (l1 < l0: none).
-__device__ __forceinline__ void guarded_layers(const Geo& g, F2 z, float nh, float nl, int& l0,
-                                               int& l1) {
-    const bool periodic = !(g.walls & 0x10);
+// reaches.
+__device__ __forceinline__ LayerRun guarded_layers(const Geo& g, F2 z, float nh, float nl) {
     int lo, hi;
     support_cells(z, nh, nl, lo, hi);
-    lo = max(lo, -2 * g.nz) - GUARD_CELLS;
-    hi = min(hi, 3 * g.nz) + GUARD_CELLS;
-    if (!periodic) {
-        lo = max(lo, 0);
-        hi = min(hi, g.nz - 1);
-        l0 = lo / TZ;
-        l1 = hi < lo ? l0 - 1 : hi / TZ;
-    } else if (hi - lo + 1 >= g.nz) {
-        l0 = 0;
-        l1 = g.ntz - 1;
-    } else {
-        l0 = floor_div(lo, TZ);
-        l1 = floor_div(hi, TZ);
-    }
+    return layer_run<TZ>(max(lo, -2 * g.nz) - GUARD_CELLS, min(hi, 3 * g.nz) + GUARD_CELLS, g.nz,
+                         !(g.walls & 0x10));
 }
 
 // The same as bits of `lay` (atomicOr; shared or global memory).
 __device__ __forceinline__ void mark_guarded_layers(const Geo& g, F2 z, float nh, float nl,
                                                     unsigned* lay) {
     const int ntz = g.ntz;
-    int l0, l1;
-    guarded_layers(g, z, nh, nl, l0, l1);
-    for (int l = l0; l <= l1; ++l) {
-        int lw = l % ntz;
-        if (lw < 0) lw += ntz;
+    const LayerRun r = guarded_layers(g, z, nh, nl);
+    for (int l = r.l0; l <= r.l1; ++l) {
+        const int lw = l % ntz;
         atomicOr(&lay[lw >> 5], 1u << (lw & 31));
     }
 }
@@ -1137,11 +1117,8 @@ __device__ void bin_single(const Geo& g, const SmallBins& sb, const F2 c[3], flo
     }
     if (sb.safe == nullptr) return;
     const int ntz = g.ntz, at = tid - 32, nt = (int)blockDim.x - 32;
-    int l0 = 0, l1 = -1;
-    if (active) guarded_layers(g, c[2], nh, nl, l0, l1);
-    const int n = min(l1 - l0 + 1, ntz);
-    l0 = n == ntz ? 0 : l0 % ntz;
-    if (l0 < 0) l0 += ntz;
+    const LayerRun w = active ? guarded_layers(g, c[2], nh, nl) : LayerRun{0, -1};
+    const int l0 = w.l0, n = w.l1 - l0 + 1;
     // Guarded: [l0, e0) and, wrapped, [0, e1).
     const int e0 = min(l0 + n, ntz), e1 = l0 + n - e0;
     for (int l = at; l < ntz; l += nt)

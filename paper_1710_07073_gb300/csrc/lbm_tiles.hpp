@@ -53,4 +53,31 @@ LBM_HD int axis_tile_bound(int cells, int L, bool periodic, int T) {
     return periodic && L % T != 0 && whole < nt ? whole + 1 : whole;
 }
 
+// The tile layers [l0, l1] that hold a cell of [lo, hi], a window that may be
+// wider than the axis; on a periodic axis to be taken modulo their number.
+// l1 < l0: none.  (The cells are wrapped before they are divided: layers of a
+// window counted past a narrow last tile would be off by one.)
+struct LayerRun {
+    int l0, l1;
+};
+
+template <int T>
+LBM_HD LayerRun layer_run(int lo, int hi, int L, bool periodic) {
+    const int nt = (L + T - 1) / T;
+    if (!periodic) {
+        lo = lo < 0 ? 0 : lo;
+        hi = hi > L - 1 ? L - 1 : hi;
+        return hi < lo ? LayerRun{0, -1} : LayerRun{lo / T, hi / T};
+    }
+    if (hi - lo + 1 >= L) return LayerRun{0, nt - 1};
+    lo %= L;
+    hi %= L;
+    if (lo < 0) lo += L;
+    if (hi < 0) hi += L;
+    const int ls = lo / T, le = hi / T;
+    if (lo <= hi) return LayerRun{ls, le};
+    if (le >= ls) return LayerRun{0, nt - 1};
+    return LayerRun{ls, le + nt};
+}
+
 }  // namespace lbm

@@ -38,6 +38,22 @@ template <int T> void check(int lmax, int cmax, long long out[3]) {
                 }
             }
 }
+// Boxes and windows (wider ones too) whose layers are not the tiles of the cells.
+extern "C" void check_layers(int lmax, int cmax, long long out[2]) {
+    for (int L = 1; L <= lmax; ++L)
+        for (int p = 0; p < 2; ++p)
+            for (int cells = 1; cells <= cmax; ++cells)
+                for (int lo = 1 - cells; lo < L; ++lo) {
+                    std::set<int> want, got;
+                    for (int c = lo; c < lo + cells; ++c)
+                        if (p) want.insert((c % L + L) % L / 4);
+                        else if (c >= 0 && c < L) want.insert(c / 4);
+                    const LayerRun r = layer_run<4>(lo, lo + cells - 1, L, p);
+                    for (int l = r.l0; l <= r.l1; ++l) got.insert(p ? l % ((L + 3) / 4) : l);
+                    ++out[0];
+                    out[1] += got != want || r.l0 < 0 || r.l1 - r.l0 >= (L + 3) / 4;
+                }
+}
 extern "C" void check_tiles(int tile, int lmax, int cmax, long long out[3]) {
     if (tile == 4) check<4>(lmax, cmax, out);
     else check<32>(lmax, cmax, out);
@@ -62,3 +78,11 @@ def test_runs_and_bound(harness, tile, lmax):
     harness.check_tiles(tile, lmax, 22, out)
     assert out[0] > 100_000
     assert (out[1], out[2]) == (0, 0)
+
+
+# The guard of the overlapped step: a support widened by 4 cells on each side.
+def test_layers(harness):
+    out = (ctypes.c_longlong * 2)()
+    harness.check_layers(75, 30, out)
+    assert out[0] > 100_000
+    assert out[1] == 0
