@@ -539,6 +539,8 @@ struct AdjBox {
 };
 
 struct AdjView {
+    static_assert(alignof(BubbleRec) == 16 && sizeof(BubbleRec) % alignof(AdjBox) == 0 &&
+                  sizeof(AdjBox) % sizeof(int) == 0, "the shared buffer's declared alignment");
     BubbleRec* rec;
     AdjBox* box;
     int* spread;
@@ -613,7 +615,7 @@ k_adj_liquid_pair(const float* __restrict__ fn, const float* __restrict__ lam_ne
                   float* __restrict__ lam, Geo g, CollideParams cp,
                   const BubbleSnap* __restrict__ pre, const BubbleSnap* __restrict__ post, int nb,
                   int two_way) {
-    extern __shared__ unsigned char s_dyn[];
+    extern __shared__ __align__(16) unsigned char s_dyn[];
     AdjView sh(s_dyn, nb);
     sh.load(pre, post, two_way);
     const unsigned half = (unsigned)g.nx / 2u;
@@ -656,7 +658,7 @@ __global__ void __launch_bounds__(128)
 k_adj_liquid(const float* __restrict__ fn, const float* __restrict__ lam_next,
              float* __restrict__ lam, Geo g, CollideParams cp, const BubbleSnap* __restrict__ pre,
              const BubbleSnap* __restrict__ post, int nb, int two_way) {
-    extern __shared__ unsigned char s_dyn[];
+    extern __shared__ __align__(16) unsigned char s_dyn[];
     AdjView sh(s_dyn, nb);
     sh.load(pre, post, two_way);
     const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;   // 19 S < 2^32
