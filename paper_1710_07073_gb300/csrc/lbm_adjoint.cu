@@ -792,7 +792,8 @@ k_adj_bubbles(const float* __restrict__ fn, const float* __restrict__ lam_next, 
         if (lane == 0)
 #pragma unroll
             for (int i = 0; i < ADJ_SUMS; ++i) s_sum[tid >> 5][i] = sum[i];
-        __syncthreads();
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"n"(ADJ_BUBBLE_THREADS) : "memory");
         return;
     }
 
@@ -879,7 +880,11 @@ k_adj_bubbles(const float* __restrict__ fn, const float* __restrict__ lam_next, 
             }
         }
     }
-    __syncthreads();   // the workers' sums (and, within the warp, the replay)
+    // The workers' sums (and, within the warp, the replay).  The workers arrive
+    // and only this warp waits: a named barrier, since the two are different
+    // places in the code.
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(ADJ_BUBBLE_THREADS) : "memory");
     // The sums over the workers' warps, a value per lane.
     double tot = 0.0;
     if (lane < ADJ_SUMS)
