@@ -723,7 +723,7 @@ k_adj_bubbles(const float* __restrict__ fn, const float* __restrict__ lam_next, 
               const BubbleSnap* __restrict__ post, const double* __restrict__ diam, int nb,
               AdjConst ac, BubbleAdj* __restrict__ adj, double* __restrict__ grad_sD,
               double* __restrict__ grad_d, double* __restrict__ lul_out, double loss_seed) {
-    extern __shared__ unsigned char s_dyn[];
+    extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ double s_sum[ADJ_WORKERS / 32][ADJ_SUMS];
     __shared__ SubRec sub[ADJ_MAX_SUB];
     __shared__ Window s_win[2];   // at x^{n+1} and at x^n
@@ -978,7 +978,7 @@ k_adj_window(const float* __restrict__ fn, const float* __restrict__ lam_next,
              float* __restrict__ lam, Geo g, CollideParams cp, const BubbleSnap* __restrict__ pre,
              const BubbleSnap* __restrict__ post, const double* __restrict__ diam, int nb,
              AdjConst ac, const double* __restrict__ lul_in) {
-    extern __shared__ unsigned char s_dyn[];
+    extern __shared__ __align__(16) unsigned char s_dyn[];
     const int self = blockIdx.x / ADJ_WINDOW_CTAS, part = blockIdx.x % ADJ_WINDOW_CTAS;
     if (!pre[self].active) return;
     AdjView sh(s_dyn, nb);
