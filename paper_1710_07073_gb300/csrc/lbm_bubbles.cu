@@ -21,6 +21,8 @@
 #include <cstring>
 #include <vector>
 
+#include <cuda.h>
+
 #include "lbm_device.cuh"
 
 namespace lbm {
@@ -2561,23 +2563,59 @@ cudaError_t launch_status(const int* flag, const int* overflow, HostPage* page, 
     return cudaGetLastError();
 }
 
+// The pinned range that holds `host`: [*start, *start + *size).  The runtime's
+// attributes describe single addresses (mapped addresses equal host addresses,
+// so both ends of an array can be pinned with a pageable gap between them); the
+// range around one is the driver's to tell.
+static bool pinned_range(const void* host, uintptr_t* start, size_t* size) {
+    using Query = CUresult(CUDAAPI*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Query query = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult res;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault,
+                                             &res) != cudaSuccess ||
+            res != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return (Query)fn;
+    }();
+    CUdeviceptr at = 0;
+    CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[2] = {&at, size};
+    *size = 0;
+    if (!query || query(2, what, out, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return false;
+    *start = (uintptr_t)at;
+    return at != 0 && *size != 0;
+}
+
 double* mapped_output(double* host, size_t n) {
-    if (!host || n == 0) return nullptr;
-    cudaPointerAttributes a, b;
-    unsigned flags = 0;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
-        cudaPointerGetAttributes(&b, host + (n - 1)) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    const uintptr_t first = (uintptr_t)host, end = first + n * sizeof(double);
+    if (!host || n == 0 || first % sizeof(double) != 0) return nullptr;
+    uintptr_t device = 0;
+    for (uintptr_t at = first; at < end;) {   // usually one range
+        cudaPointerAttributes a;
+        uintptr_t start = 0;
+        size_t size = 0;
+        unsigned flags = 0;
+        if (cudaPointerGetAttributes(&a, (void*)at) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (at == first) device = (uintptr_t)a.devicePointer;
+        if (a.type != cudaMemoryTypeHost || !a.devicePointer ||
+            (uintptr_t)a.devicePointer - device != at - first ||
+            !pinned_range((void*)at, &start, &size) || at < start || at - start >= size)
+            return nullptr;
+        if (cudaHostGetFlags(&flags, (void*)at) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (flags & cudaHostRegisterReadOnly) return nullptr;
+        at = start + size;
     }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer ||
-        (double*)b.devicePointer - (double*)a.devicePointer != (ptrdiff_t)(n - 1))
-        return nullptr;
-    if (cudaHostGetFlags(&flags, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return (flags & cudaHostRegisterReadOnly) ? nullptr : (double*)a.devicePointer;
+    return device % sizeof(double) == 0 ? (double*)device : nullptr;
 }
 
 }  // namespace lbm
