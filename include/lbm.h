@@ -285,7 +285,10 @@ int lbm_get_bubbles(lbm_ctx* ctx, int cap, int* n, double* pos3, double* vel3,
                     double* ul3, double* psi3, int* active);
 
 /* FP64 totals over the box: out4 = {sum rho, sum rho u_x, sum rho u_y,
- * sum rho u_z} of the current pre-collision populations (Eq. 10). */
+ * sum rho u_z} of the current pre-collision populations (Eq. 10).  Each
+ * direction's f - w rho_l is summed in three floats (about 72 bits) over a
+ * thread's sites and those sums in FP64, in a fixed order: the error is that of
+ * summing a few thousand partial sums in FP64. */
 int lbm_get_totals(lbm_ctx* ctx, double* out4);
 
 /* Binning of the last step (Algorithm 1 step 2), for inspection.

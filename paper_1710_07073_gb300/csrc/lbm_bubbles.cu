@@ -2237,25 +2237,30 @@ __global__ void k_set_feq(const double* __restrict__ rho, const double* __restri
 #undef LBM_FEQ
 }
 
-// FP64 totals: per-thread compensated sums, per-block FP64 partials in fixed
-// order, then one block.
+// FP64 totals: per-thread sums in three floats, per-block FP64 partials in
+// fixed order, then one block.
 //
 // Bound by HBM (76 or 38 B per site, read once), as long as the FP64 pipe
 // stays out of the loop: it issues 2 FMAs per clock and SM here, and the 95
 // FP64 operations per site of a plain FP64 accumulation took 0.81 ms on
 // 128 x 128 x 256 where the reads take 0.05.  So each thread sums every
-// direction over its sites as hi + lo, two floats (Neumaier's compensated
-// summation: TwoSum, the rounding errors collected in lo), 7 FP32 operations
-// per value, and only the per-thread sums go through FP64.  The error is that
-// of about 48 bits against the sum of magnitudes.  On even rows a thread takes
-// an x-pair by aligned row loads and sums its two nodes in packed FP32, half
-// the instructions (odd rows: two sites at a time).  lbm_get_totals in FP64, by
-// scalar sums and by packed ones: 7.01, 0.76, 0.44 ms on 256 x 256 x 512 in
-// FP32 (the reads take 0.38) and 0.43 in FP16; 2.42 and 1.37 ms by scalar and
-// packed sums on 384 x 384 x 768.
-constexpr int TOT_BLOCK = 256;
+// direction over its sites as h + m + l, three floats: TwoSum into h, its
+// rounding error by TwoSum into m, that one's error into l (13 FP32
+// operations per value), and only the per-thread sums go through FP64.  h + m
+// is exact to 2^-48 of h and l holds what that leaves to 24 more bits, so the
+// error is that of the FP64 partials; two floats (7 operations) fell up to
+// 2^-48 of the sum of magnitudes short.  On even rows a thread takes an x-pair
+// by aligned row loads and sums its two nodes in packed FP32, half the
+// instructions (odd rows: two sites at a time).  lbm_get_totals in FP64, by two
+// floats and by three: 7.01, 0.48, 0.55 ms on 256 x 256 x 512 in FP32 (the reads
+// take 0.38), 1.57 and 1.80 ms by two and three on 384 x 384 x 768, 0.12 and
+// 0.15 on 127 x 127 x 255.  Error against exact sums, of the sum of magnitudes,
+// z momentum of 64 x 64 x 128 after 10 steps: 7e-16 in FP64, 5e-17 by either.
+constexpr int TOT_BLOCK = 192;
 // Resident CTAs per SM the kernel is compiled for, and the grid: whole waves
-// of 152 SMs.
+// of 152 SMs.  Three sums per direction and pair fill the registers: 12 warps
+// per SM with 168 each took 0.545 ms on 256 x 256 x 512, 16 with 128 (spills)
+// 0.724, 8 with 255 0.623.
 constexpr int TOT_PER_SM = 2;
 constexpr int TOT_GRID = 152 * TOT_PER_SM;
 static_assert(TOT_GRID <= TOTALS_PARTIALS_MAX, "a context's buffer of partials");
@@ -2303,30 +2308,65 @@ __device__ __noinline__ void totals_fp64(const typename Store<ST>::T* __restrict
     }
 }
 
-// TwoSum of a value that may itself be a product (a widened 16-bit value):
-// __fadd_rn keeps the compiler from contracting that product into the sum,
-// which would leave its rounding error out.
-__device__ __forceinline__ F2 two_sum_rn(float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fadd_rn(s, -a);
-    return F2{s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
-}
+// FP32 sums and differences of one node's value, or of an x-pair's two values
+// at once (packed).  __fadd_rn keeps the compiler from contracting a product
+// (a widened 16-bit value) into a sum, which would leave its error out.
+__device__ __forceinline__ float sum_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float diff_rn(float a, float b) { return __fadd_rn(a, -b); }
+__device__ __forceinline__ float2 sum_rn(float2 a, float2 b) { return add2(a, b); }
+__device__ __forceinline__ float2 diff_rn(float2 a, float2 b) { return sub2(a, b); }
 
-// The same on an x-pair's two nodes at once (packed FP32).
-__device__ __forceinline__ void two_sum_pair(float2& h, float2& l, float2 v) {
-    const float2 s = add2(h, v);
-    const float2 bb = sub2(s, h);
-    l = add2(l, add2(sub2(h, sub2(s, bb)), sub2(v, bb)));
-    h = s;
+// h + m + l.
+template <class V> struct F3 {
+    V h, m, l;
+    // Knuth's TwoSum: a becomes a + v, the result is its rounding error.
+    static __device__ __forceinline__ V add_to(V& a, V v) {
+        const V s = sum_rn(a, v), b = diff_rn(s, a);
+        const V e = sum_rn(diff_rn(a, diff_rn(s, b)), diff_rn(v, b));
+        a = s;
+        return e;
+    }
+    __device__ __forceinline__ void add(V v) { l = sum_rn(l, add_to(m, add_to(h, v))); }
+    __device__ __forceinline__ void add(const F3& o) {
+        add(o.h);
+        add(o.m);
+        l = sum_rn(l, o.l);
+    }
+    __device__ __forceinline__ void sub(const F3& o) {
+        const V z = diff_rn(o.h, o.h);   // zero (not finite: NaN, which the caller looks for)
+        add(F3{diff_rn(z, o.h), diff_rn(z, o.m), diff_rn(z, o.l)});
+    }
+};
+
+// Eq. 10 over the directions: opposite ones come in pairs (2k - 1, 2k).
+template <class V>
+__device__ __forceinline__ void totals_moments(const F3<V> dir[Q], V zero, F3<V> m[4]) {
+    m[0] = dir[0];
+#pragma unroll
+    for (int k = 1; k < 4; ++k) m[k] = F3<V>{zero, zero, zero};
+#pragma unroll
+    for (int j = 1; j < Q; j += 2) {
+        m[0].add(dir[j]);
+        m[0].add(dir[j + 1]);
+        F3<V> d = dir[j];
+        d.sub(dir[j + 1]);
+        if (cx(j) > 0) m[1].add(d);
+        if (cx(j) < 0) m[1].sub(d);
+        if (cy(j) > 0) m[2].add(d);
+        if (cy(j) < 0) m[2].sub(d);
+        if (cz(j) > 0) m[3].add(d);
+        if (cz(j) < 0) m[3].sub(d);
+    }
 }
 
 // Even rows: an x-pair per thread and pass, aligned row loads and packed sums.
 template <int ST>
 __device__ __forceinline__ void totals_pairs(const typename Store<ST>::T* __restrict__ f,
-                                             const Geo& g, const CollideParams& cp, F2 dir[Q]) {
-    float2 h[Q], l[Q];
+                                             const Geo& g, const CollideParams& cp,
+                                             F3<float> m[4]) {
+    F3<float2> dir[Q], mp[4];
 #pragma unroll
-    for (int j = 0; j < Q; ++j) h[j] = l[j] = f2(0.0f);
+    for (int j = 0; j < Q; ++j) dir[j] = F3<float2>{f2(0.0f), f2(0.0f), f2(0.0f)};
     const unsigned half = (unsigned)g.nx / 2u, n = (unsigned)g.S / 2u;
     for (unsigned p = blockIdx.x * TOT_BLOCK + threadIdx.x; p < n; p += gridDim.x * TOT_BLOCK) {
         const unsigned xy = p / half;
@@ -2337,26 +2377,27 @@ __device__ __forceinline__ void totals_pairs(const typename Store<ST>::T* __rest
         for (int j = 0; j < Q; ++j) {
             float2 v = Raw2<ST>::widen(rv[j]);
             if (Store<ST>::kScaled) v = mul2(v, f2(wf(j) * cp.inv_scale));
-            two_sum_pair(h[j], l[j], v);
+            dir[j].add(v);
         }
     }
+    totals_moments(dir, f2(0.0f), mp);
 #pragma unroll
-    for (int j = 0; j < Q; ++j) dir[j] = f2_add(F2{h[j].x, l[j].x}, h[j].y, l[j].y);
+    for (int k = 0; k < 4; ++k) {
+        m[k] = F3<float>{mp[k].h.x, mp[k].m.x, mp[k].l.x};
+        m[k].add(F3<float>{mp[k].h.y, mp[k].m.y, mp[k].l.y});
+    }
 }
 
-template <int ST, bool PAIR>
-__global__ void __launch_bounds__(TOT_BLOCK, TOT_PER_SM)
-k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, double* partials) {
-    __shared__ double sh[32];
-    F2 dir[Q];
+// Odd rows: two sites at a time, the loads of both issued first.
+template <int ST>
+__device__ __forceinline__ void totals_sites(const typename Store<ST>::T* __restrict__ f,
+                                             const Geo& g, const CollideParams& cp,
+                                             F3<float> m[4]) {
+    F3<float> dir[Q];
 #pragma unroll
-    for (int j = 0; j < Q; ++j) dir[j] = F2{0.0f, 0.0f};
+    for (int j = 0; j < Q; ++j) dir[j] = F3<float>{0.0f, 0.0f, 0.0f};
     const unsigned S = (unsigned)g.S, stride = gridDim.x * TOT_BLOCK;   // 19 S < 2^32
-    const unsigned s0 = blockIdx.x * TOT_BLOCK + threadIdx.x;
-    if constexpr (PAIR) totals_pairs<ST>(f, g, cp, dir);
-    // Odd rows: two sites at a time, the loads of both issued first (two_sum
-    // with zero changes nothing).
-    for (unsigned s = PAIR ? S : s0; s < S; s += 2 * stride) {
+    for (unsigned s = blockIdx.x * TOT_BLOCK + threadIdx.x; s < S; s += 2 * stride) {
         const bool two = s + stride < S;
         int x, y, z, x2, y2, z2;
         site_coords(g, s, x, y, z);
@@ -2369,28 +2410,29 @@ k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, d
         gather_finish<ST>(rb, cp, gb);
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
-            const F2 t = two_sum_rn(dir[j].h, ga[j]);
-            const F2 v = two_sum_rn(t.h, two ? gb[j] : 0.0f);
-            dir[j] = F2{v.h, dir[j].l + t.l + v.l};
+            dir[j].add(ga[j]);
+            dir[j].add(two ? gb[j] : 0.0f);   // zero changes nothing
         }
     }
-    // Eq. 10 over the directions: opposite ones come in pairs (2k - 1, 2k).
-    F2 m[4] = {dir[0], F2{0.0f, 0.0f}, F2{0.0f, 0.0f}, F2{0.0f, 0.0f}};
-#pragma unroll
-    for (int j = 1; j < Q; j += 2) {
-        m[0] = f2_add(f2_add(m[0], dir[j].h, dir[j].l), dir[j + 1].h, dir[j + 1].l);
-        const F2 d = f2_add(dir[j], -dir[j + 1].h, -dir[j + 1].l);
-        if (cx(j) != 0) m[1] = f2_add(m[1], (float)cx(j) * d.h, (float)cx(j) * d.l);
-        if (cy(j) != 0) m[2] = f2_add(m[2], (float)cy(j) * d.h, (float)cy(j) * d.l);
-        if (cz(j) != 0) m[3] = f2_add(m[3], (float)cz(j) * d.h, (float)cz(j) * d.l);
-    }
+    totals_moments(dir, 0.0f, m);
+}
+
+template <int ST, bool PAIR>
+__global__ void __launch_bounds__(TOT_BLOCK, TOT_PER_SM)
+k_totals(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams cp, double* partials) {
+    __shared__ double sh[32];
+    F3<float> m[4];
+    if constexpr (PAIR) totals_pairs<ST>(f, g, cp, m);
+    else totals_sites<ST>(f, g, cp, m);
     double acc[4];
     bool finite = true;
     for (int k = 0; k < 4; ++k) {
-        acc[k] = f2_to(m[k]);
-        finite = finite && isfinite(m[k].h) && isfinite(m[k].l);
+        acc[k] = ((double)m[k].h + (double)m[k].m) + (double)m[k].l;
+        finite = finite && isfinite(m[k].h) && isfinite(m[k].m) && isfinite(m[k].l);
     }
-    if (!finite) totals_fp64<ST, PAIR>(f, g, cp, s0, stride, acc);
+    if (!finite)
+        totals_fp64<ST, PAIR>(f, g, cp, blockIdx.x * TOT_BLOCK + threadIdx.x,
+                              gridDim.x * TOT_BLOCK, acc);
     for (int k = 0; k < 4; ++k) {
         const double t = block_sum(acc[k], sh);
         if (threadIdx.x == 0) partials[4 * blockIdx.x + k] = t;
