@@ -1395,7 +1395,7 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
                                             const TileHead& h, TileHead& next,
                                             const int* __restrict__ items,
                                             const BubbleRec* __restrict__ recs, int nb,
-                                            float* __restrict__ partial,
+                                            float* __restrict__ partial, int cap,
                                             typename Raw2<ST>::T (&rp)[PAIR ? Q : 1]) {
     constexpr bool PIPE = InterpOccupancy<ST, PAIR>::kPipe;
     const int t = h.t;
@@ -1565,12 +1565,12 @@ __device__ __forceinline__ void tile_interp(const typename Store<ST>::T* __restr
                 for (int o = INTERP_ROWS / 2; o > 0; o >>= 1)
                     v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
             if (row == 0 && k < cntc) {
-                float4* q = reinterpret_cast<float4*>(partial) +
-                            partial_stride(LIFT) / 4 * (size_t)(c0 + k);
+                const size_t p = (size_t)(c0 + k);
+                float4* q = reinterpret_cast<float4*>(partial) + partial_words(LIFT) * p;
                 q[0] = make_float4(v[0], v[1], v[2], LIFT ? v[3] : 0.0f);
                 if (LIFT) {
                     q[1] = make_float4(v[4], v[5], v[6], v[7]);
-                    q[2] = make_float4(v[8], 0.0f, 0.0f, 0.0f);
+                    partial[8 * (size_t)cap + p] = v[8];
                 }
             }
         }
@@ -1622,7 +1622,8 @@ k_tile_interp(const typename Store<ST>::T* __restrict__ f, Geo g, CollideParams 
         const int tnn = i + 2 * step < ntiles ? __ldcg(cover + i + 2 * step) : -1;
         if (i + step >= ntiles) pdl_trigger();   // this CTA's last tile
         __syncthreads();   // the shared tables of the previous tile are done with
-        tile_interp<ST, PAIR, LIFT>(f, g, cp, h, next, items, recs, nb, partial, rp);
+        tile_interp<ST, PAIR, LIFT>(f, g, cp, h, next, items, recs, nb, partial, cap,
+                                    rp);
         h = next;
         tn = tnn;
     }
@@ -1680,7 +1681,7 @@ template <bool LIFT>
 __global__ void __launch_bounds__(TAIL_THREADS)
 k_swarm_tail(Geo g, BubbleDev B, BubbleConst bc, int* __restrict__ flag, Bins bins,
              SwarmBins sw) {
-    constexpr int NV = win_vals(LIFT), NS = TAIL_SLOTS, NP = partial_stride(LIFT) / 4;
+    constexpr int NV = win_vals(LIFT), NS = TAIL_SLOTS, NP = partial_words(LIFT);
     pdl_wait();
     const int b = blockIdx.x * TAIL_THREADS + threadIdx.x;
     if (b == 0) *sw.ncover = 0;
@@ -1695,7 +1696,7 @@ k_swarm_tail(Geo g, BubbleDev B, BubbleConst bc, int* __restrict__ flag, Bins bi
         for (int q = 0; q < WIN_VALS_LIFT; ++q) acc[q] = 0.0f;
         for (int k0 = 0; k0 == 0 || k0 < n; k0 += NS) {
             int p[NS];
-            float v[NS][4 * NP];
+            float v[NS][LIFT ? NV : 4];
 #pragma unroll
             for (int i = 0; i < NS; ++i) p[i] = k0 + i < sw.per ? __ldcg(sl + k0 + i) : -1;
 #pragma unroll
@@ -1711,6 +1712,8 @@ k_swarm_tail(Geo g, BubbleDev B, BubbleConst bc, int* __restrict__ flag, Bins bi
                     v[i][4 * c + 2] = u.z;
                     v[i][4 * c + 3] = u.w;
                 }
+                if (LIFT)
+                    v[i][NV - 1] = p[i] >= 0 ? __ldcg(sw.partial + 8 * (size_t)bins.cap + p[i]) : 0.0f;
             }
 #pragma unroll
             for (int i = 0; i < NS; ++i)

@@ -842,7 +842,7 @@ int lbm_set_bubbles(lbm_ctx* c, int n, const double* pos3, const double* vel3,
         sw.kidx = (int*)dalloc(c, sizeof(int) * (size_t)cap);
         sw.slots = (int*)dalloc(c, sizeof(int) * (size_t)cap);   // n * per
         sw.ntile = (int*)dalloc(c, sizeof(int) * (size_t)n);
-        sw.partial = (float*)dalloc(c, PARTIAL_STRIDE_MAX * sizeof(float) * (size_t)cap);
+        sw.partial = (float*)dalloc(c, WIN_VALS_LIFT * sizeof(float) * (size_t)cap);
         sw.cover = (int*)dalloc(c, sizeof(int) * (size_t)c->bins.T);
         sw.ncover = (int*)dalloc(c, sizeof(int));
         sw.chunk_sums = (int*)dalloc(c, sizeof(int) * (size_t)sw.grid);

@@ -171,9 +171,10 @@ struct BubbleConst {
 // weights, are sums of the velocities times per-axis difference weights).
 constexpr int WIN_VALS_LIFT = 9;
 __host__ __device__ constexpr int win_vals(bool lift) { return lift ? WIN_VALS_LIFT : 3; }
-// Floats per (tile, bubble) entry of SwarmBins::partial: whole 16-byte accesses.
-constexpr int PARTIAL_STRIDE_MAX = 12;
-__host__ __device__ constexpr int partial_stride(bool lift) { return lift ? PARTIAL_STRIDE_MAX : 4; }
+// SwarmBins::partial by (tile, bubble) entry p of cap: the first 4 win values (8
+// with lift) as the 16-byte words p (2 p, 2 p + 1), the lift's ninth behind
+// all of them, at float 8 cap + p.
+__host__ __device__ constexpr int partial_words(bool lift) { return lift ? 2 : 1; }
 
 // A double as two floats (h = v rounded, l = the rest rounded) and back.
 __host__ __device__ inline void split_f2(double v, float& h, float& l) {
@@ -258,7 +259,7 @@ struct SwarmBins {
     int* slots;           // [nb * per] list position of bubble b's k-th tile
     int* ntile;           // [nb] tiles of bubble b in the last binning (0: not binned)
     int per;              // tiles a bubble's window can touch at most
-    float* partial;       // [PARTIAL_STRIDE_MAX * cap] Eq. 20 sums of each (tile, bubble) entry
+    float* partial;       // [WIN_VALS_LIFT * cap] Eq. 20 sums of each (tile, bubble) entry
     int pad;              // cells the lists reach beyond the supports (1 with lift)
     int* cover;           // [T] the tiles with a non-empty list (any order)
     int* ncover;          // [1] their number
