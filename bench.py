@@ -412,6 +412,8 @@ def run_batch(args, wl):
     avg_kernel_s = (k_ms / max(1, k_n)) * 1e-3
     achieved = bytes_per_site * S / avg_kernel_s / 1e9
     peak, peak_kind = measured_peak()
+    # Nodes per thread of the batch sweep (16-bit rows all of a multiple of 4: four).
+    nodes = 4 if storage != "f32" and all(c[0][0] % 4 == 0 for c in cols) else 2
     line = {
         "metric": METRIC, "value": round(value, 2), "unit": "MLUPS", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms / args.steps, 5),
@@ -424,7 +426,7 @@ def run_batch(args, wl):
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4),
                      "traffic": profile_traffic(storage, None, key="%s_batch64" % storage),
-                     "kernel": "k_collide_batch<%d,%d>" % (STORAGES[storage], planes),
+                     "kernel": "k_collide_batch<%d,%d,%d>" % (STORAGES[storage], planes, nodes),
                      "algorithmic_bytes_per_launch": bytes_per_site * S,
                      "avg_launch_ms": round(avg_kernel_s * 1e3, 5), "launches": k_n,
                      "peak_kind": peak_kind, "timed": "separate per-launch pass after the graph run"},
@@ -528,7 +530,8 @@ def run_adjoint(args):
                       "u0_direction": [g_e, fd_e, abs(g_e / fd_e - 1)],
                       "format": "[adjoint, central FD of the FP32 forward, relative difference]"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-                     "frac": round(achieved / peak, 4), "traffic": None, "kernel": "k_adj_liquid",
+                     "frac": round(achieved / peak, 4), "traffic": None,
+                     "kernel": "k_adj_liquid_pair",   # even rows
                      "algorithmic_bytes_per_launch": 3 * 19 * 4 * S,
                      "avg_launch_ms": round(k_ms / max(1, k_n), 5), "launches": k_n,
                      "peak_kind": peak_kind},

@@ -984,15 +984,32 @@ __device__ __forceinline__ void quad_block_free(const typename Store<ST>::T* __r
                             F, cp, flag, active);
 }
 
-// TAB: the force gather of long tile lists (per-axis weight tables).  NODES:
+// The form of a sweep kernel from its parameters behind ST, of which there are
+// as many as lbm_sweep_kernel's names show: [4,] TAB for the listed sweep, [4]
+// for the force-free one.
+template <int... P> struct ListedForm;
+template <int TAB> struct ListedForm<TAB> {
+    static constexpr int kNodes = 2;
+    static constexpr bool kTab = TAB != 0;
+};
+template <int NODES, int TAB> struct ListedForm<NODES, TAB> {
+    static constexpr int kNodes = NODES;
+    static constexpr bool kTab = TAB != 0;
+};
+template <int... N> struct FreeForm { static constexpr int kNodes = 2; };
+template <int NODES> struct FreeForm<NODES> { static constexpr int kNodes = NODES; };
+
+// kTab: the force gather of long tile lists (per-axis weight tables).  kNodes:
 // nodes per thread along x (four: quad_block below).
-template <int ST, int NODES, bool TAB>
-__global__ void __launch_bounds__(SweepShape<ST, NODES>::kThreads, SweepShape<ST, NODES>::kMinBlocks)
+template <int ST, int... P>
+__global__ void __launch_bounds__(SweepShape<ST, ListedForm<P...>::kNodes>::kThreads,
+                                  SweepShape<ST, ListedForm<P...>::kNodes>::kMinBlocks)
 k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
                       typename Store<ST>::T* __restrict__ fout, Geo g, CollideParams cp,
                       const int* tile_start, const int* tile_count, const int* items, int cap,
                       const BubbleRec* recs, int nb, int* __restrict__ flag,
                       const unsigned* safe, unsigned epoch, const int* zperm, ZSpan zs) {
+    constexpr bool TAB = ListedForm<P...>::kTab;
     __shared__ __align__(16) BubbleRec srec[FORCE_CHUNK];
     // The next bubble update may be scheduled once every CTA of the sweep has
     // started; it waits for the sweep to complete before it reads anything.
@@ -1003,7 +1020,7 @@ k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
     if (bz >= zs.hole) bz += zs.skip;
     if (zperm != nullptr) bz = __ldcg(zperm + blockIdx.z);
     const bool lead = (blockIdx.x | blockIdx.y | blockIdx.z) == 0;
-    if constexpr (NODES == 4)
+    if constexpr (ListedForm<P...>::kNodes == 4)
         quad_block<ST, TAB>(fin, fout, g, cp, tile_start, tile_count, items, cap, recs, nb, flag,
                             blockIdx.x, blockIdx.y, bz, srec, safe, epoch, lead);
     else
@@ -1016,14 +1033,15 @@ k_collide_stream_pair(const typename Store<ST>::T* __restrict__ fin,
 // (collide_pair<ST, false>, as k_collide_stream_pair runs it for a block with
 // an empty list), in a kernel without the force-gather code: the 16-bit
 // sweep runs about 3 % faster in it than in k_collide_stream_pair.
-template <int ST, int NODES>
-__global__ void __launch_bounds__(SweepShape<ST, NODES>::kThreads, SweepShape<ST, NODES>::kMinBlocks)
+template <int ST, int... N>
+__global__ void __launch_bounds__(SweepShape<ST, FreeForm<N...>::kNodes>::kThreads,
+                                  SweepShape<ST, FreeForm<N...>::kNodes>::kMinBlocks)
 k_collide_stream_free(const typename Store<ST>::T* __restrict__ fin,
                       typename Store<ST>::T* __restrict__ fout, Geo g, CollideParams cp,
                       int* __restrict__ flag, ZSpan zs) {
     int bz = zs.first + (int)blockIdx.z;
     if (bz >= zs.hole) bz += zs.skip;
-    if constexpr (NODES == 4) {
+    if constexpr (FreeForm<N...>::kNodes == 4) {
         quad_block_free<ST>(fin, fout, g, cp, flag, blockIdx.x, blockIdx.y, bz);
         return;
     }
@@ -1211,13 +1229,13 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
                                           flag, zs);
             switch (storage) {
                 case 0:
-                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<0, 2>, (const float*)fin,
+                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<0>, (const float*)fin,
                                               (float*)fout, g, cp, flag, zs);
                 case 1:
-                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<1, 2>, (const __half*)fin,
+                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<1>, (const __half*)fin,
                                               (__half*)fout, g, cp, flag, zs);
                 default:
-                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<2, 2>,
+                    return cudaLaunchKernelEx(&cfg, k_collide_stream_free<2>,
                                               (const __nv_bfloat16*)fin, (__nv_bfloat16*)fout, g,
                                               cp, flag, zs);
             }
@@ -1242,7 +1260,7 @@ cudaError_t launch_collide_stream(int storage, const void* fin, void* fout, cons
         switch (storage * 2 + (tab ? 1 : 0)) {
 #define LBM_LAUNCH_PAIR(SI, TB, T)                                                                \
     case SI * 2 + TB:                                                                             \
-        return cudaLaunchKernelEx(&cfg, k_collide_stream_pair<SI, 2, TB>, (const T*)fin, (T*)fout,   \
+        return cudaLaunchKernelEx(&cfg, k_collide_stream_pair<SI, TB>, (const T*)fin, (T*)fout,   \
                                   g, cp, start, count, items, cap, recs, nb, flag, safe, epoch,  \
                                   zperm, zs);
             LBM_LAUNCH_PAIR(0, 0, float)
