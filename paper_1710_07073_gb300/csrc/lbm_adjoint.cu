@@ -1207,8 +1207,8 @@ extern "C" int lbm_adj_backward(lbm_ctx* c, double dloss, double* grad_drag_scal
     float* lam[2] = {(float*)dalloc(c, fb), (float*)dalloc(c, fb)};
     BubbleAdj* adj = (BubbleAdj*)dalloc(c, sizeof(BubbleAdj) * nb);
     // grads[0, nb): dL/dd_b; grads[nb, 2 nb): each bubble's part of dL/ds_D
-    // (summed over the bubbles in order at the end); lul: the interpolation
-    // seed phase B hands to phase C.
+    // (summed over the bubbles in order at the end); lul: the interpolation's
+    // seed, from k_adj_bubbles to k_adj_window.
     double* grads = (double*)dalloc(c, sizeof(double) * 2 * (size_t)nb);
     double* lul = (double*)dalloc(c, sizeof(double) * 3 * (size_t)nb);
     double* du0 = grad_u0 ? (double*)dalloc(c, sizeof(double) * 3 * (size_t)g.S) : nullptr;

@@ -371,6 +371,9 @@ void free_bubbles(lbm_batch* b) {
     b->small.parts = 0;
 }
 
+// Tiles a window of half-width n covers on an axis, for the batch's limit on
+// (tile, bubble) pairs.  A window across a periodic boundary with a narrower
+// last tile takes one more: pairs beyond the lists are flagged when they occur.
 int axis_tile_bound(double n, int T) {
     const int cells = (int)std::ceil(2.0 * n) + 1;
     return (cells + T - 1) / T + 1;

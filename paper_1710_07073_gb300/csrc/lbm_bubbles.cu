@@ -34,8 +34,8 @@ namespace lbm {
 // ---- positions in two floats ------------------------------------------------
 // A position is carried through the sub-steps as hi + lo, two floats with
 // |lo| <= ulp(hi)/2 (about 48 significant bits), so the 10 sub-steps use the
-// FP32 pipe: FP64 issue is slow on this GPU and the bubble update is one
-// serial thread.  Sums use Knuth's TwoSum; the product error of u dt_b comes
+// FP32 pipe: FP64 issue is slow on this GPU and the sub-steps are one serial
+// chain per axis.  Sums use Knuth's TwoSum; the product error of u dt_b comes
 // from one FMA (the exact-product property of fused multiply-add).
 __device__ __forceinline__ F2 f2_from(double v) {
     const float h = (float)v;
@@ -144,10 +144,9 @@ __device__ __forceinline__ void node_velocity(const float gv[Q], const CollidePa
     u[2] = jz * inv_rho;
 }
 
-// Precision: positions are integrated in FP64 (they reach hundreds of lattice
-// units and move by 1e-5 per sub-step); velocities, forces and the mapping
-// weights are FP32.  FP64 latency on this GPU is long, so only the position
-// update, the window bounds and the wall tests use it.
+// Precision: positions are integrated in two floats (they reach hundreds of
+// lattice units and move by 1e-5 per sub-step), and so are the window bounds
+// and the wall tests; velocities, forces and the mapping weights are FP32.
 constexpr int BUBBLE_THREADS = 256;
 
 // The interpolation window of one bubble (Algorithm 1 step 2): the cells
@@ -297,7 +296,7 @@ __device__ __forceinline__ void add_window_node(const float wt[4], const float u
     }
 }
 
-// Whether that holds for every node of the window.
+// Whether no node of the window has a neighbour beyond a face.
 __device__ __forceinline__ bool window_inner(const Geo& g, const Window& w) {
     return w.lo[0] >= 1 && w.lo[0] + w.cnt[0] < g.nx && w.lo[1] >= 1 &&
            w.lo[1] + w.cnt[1] < g.ny && w.lo[2] >= 1 && w.lo[2] + w.cnt[2] < g.nz;
@@ -337,15 +336,6 @@ __device__ __forceinline__ void chunk_sum2(const typename Store<ST>::T* __restri
     node_velocity(gb, cp, ub);
     if (ha) add_window_node<LIFT>(wa, ua, acc);
     if (hb) add_window_node<LIFT>(wb, ub, acc);
-}
-
-__device__ __forceinline__ void warp_sum3(float& ax, float& ay, float& az) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ax += __shfl_xor_sync(0xffffffffu, ax, o);
-        ay += __shfl_xor_sync(0xffffffffu, ay, o);
-        az += __shfl_xor_sync(0xffffffffu, az, o);
-    }
 }
 
 // Sum of v[0..N) over the CTA's BUBBLE_THREADS threads, in thread 0 (fixed
@@ -1355,9 +1345,10 @@ static_assert(INTERP_THREADS % INTERP_ROWS == 0 && TX == 32 && TY == 4 && TZ == 
               "tile shape of the interpolation: a lane per column");
 // Resident CTAs per SM the interpolation is compiled for, and whether it loads
 // a tile's rows a tile ahead (kPipe): with 16-bit storage on even rows the 19
-// packed rows fit beside the tables and sums at 64 registers, and the
-// 384x384x768 swarm's FP16 step took 1.910 ms against 1.923 at 5 CTAs (48
-// registers) without; FP32's 38 do not (3 CTAs: 3.068 ms against 3.036).
+// packed rows fit beside the tables and sums at 64 registers but for 8 bytes (32
+// with lift), and the 384x384x768 swarm's FP16 step took 1.910 ms against 1.923
+// at 5 CTAs (48 registers) without; FP32's 38 do not (3 CTAs: 3.068 ms against
+// 3.036).
 template <int ST, bool PAIR> struct InterpOccupancy {
     static constexpr bool kPipe = PAIR && ST != 0;
     static constexpr int kMinBlocks = 4;

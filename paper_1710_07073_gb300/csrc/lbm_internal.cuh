@@ -234,7 +234,7 @@ struct SmallBins {
     // set its own sweep reads.  Null: not kept.
     unsigned* safe;    // [ntz] (the set this launch writes)
     unsigned safe_epoch;
-    // Order of the next sweep's z blocks (PZ planes each): the blocks of
+    // Order of the next sweep's z blocks (`planes` planes each): the blocks of
     // cleared layers first, then the guarded ones, each in ascending order,
     // so that the sweep reaches the layers that wait for the update last.
     // Null: not kept.
@@ -296,9 +296,9 @@ struct BatchColumn {
 // the bubble update before it (`overlap`): CTAs whose z tile layer holds
 // safe[layer] == epoch run without waiting for the update; the others (and
 // CTA 0) wait for it before reading the tile lists.
-// zperm (may be null): the order of the z blocks (PZ planes each) in which
-// the CTAs are handed out, a permutation of 0 .. ceil(nz / PZ) - 1.
-// A subset of the sweep's z blocks (PZ planes each): CTA z-index i sweeps
+// zperm (may be null): the order of the z blocks (sweep_planes planes each) in
+// which the CTAs are handed out, a permutation of 0 .. blocks - 1.
+// A subset of the sweep's z blocks: CTA z-index i sweeps
 // block first + i, moved past the hole [hole, hole + skip) when it reaches it;
 // `count` blocks in all.
 struct ZSpan {
